@@ -258,8 +258,8 @@ hkv_status hkv_evict_all(const hkv_config *cfg, const hkv_cache *cache, hkv_stre
 /* One decode step of one layer: the append of the new token (Sec. 3, KV
  * Cache) fused with the attention of Eq. 1 over the cache including that
  * token. One kernel launch when every CTA's share of the layer spans at
- * most 128 heads (bounded from the config: the heads of a layer times the
- * tiles of the longest segment it allows, over the grid), else two chained
+ * most 256 heads (bounded from the config: the heads of a layer times the
+ * rows of the longest segment it allows, over the grid), else two chained
  * kernels (attention, then a finishing kernel that combines heads split
  * across CTAs and advances the counters); hkv_decode_step_launches tells
  * which. out[s][h][:] = softmax(q k^T / sqrt(d)) V over the
@@ -300,8 +300,8 @@ hkv_status hkv_decode_step_identify(const hkv_config *cfg, const hkv_cache *cach
 /* Eq. 1 for one new query per head over that head's live tokens (any mix
  * of lengths): out[s][h][:] = softmax(q k^T / sqrt(d)) V, fp32 accumulation,
  * written in fp32 ([S][H][head_dim]). Split-K over the layer's total token
- * count, then a second kernel combines the heads split across CTAs;
- * workspace of hkv_workspace_size bytes.
+ * count, in one launch or two as hkv_decode_step's; workspace of
+ * hkv_workspace_size bytes.
  * A head with len = 0 yields zeros. */
 hkv_status hkv_decode_attention(const hkv_config *cfg, const hkv_cache *cache, int layer,
                                 const void *q, float *out, void *workspace, size_t ws_bytes,
@@ -313,10 +313,10 @@ hkv_status hkv_decode_attention(const hkv_config *cfg, const hkv_cache *cache, i
  * and budgets all device memory, may have no way to provide the workspace
  * that hkv_decode_attention takes. Here the split-K partials, the records
  * of heads split between CTAs and the kernels' control block live in a
- * fixed device array inside the library (1.06 MiB: 1 MiB of partials,
- * 64 KiB of records, 256 bytes), which every GPU that loads the library
- * holds until the process exits. Nothing in it has to start at zero: each
- * call writes what it reads. Same inputs, outputs and results as
+ * fixed device array inside the library (2.06 MiB: 1 MiB of partials for
+ * each of the two designs, 64 KiB of records, 256 bytes), which every GPU
+ * that loads the library holds until the process exits. The caller
+ * initialises nothing. Same inputs, outputs and results as
  * hkv_decode_attention; it allocates nothing.
  *  - The first call on a device, with that device current, looks up the
  *    array's device address and prepares the kernel; make that first call

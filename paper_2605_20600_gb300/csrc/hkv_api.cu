@@ -142,23 +142,6 @@ MethodArgs method_args(const hkv_config *cfg) {
 
 int heads_per_layer(const hkv_config *c) { return c->n_seqs * c->n_heads; }
 
-// longest segment any call may see: a dense head (C + E) or a compressed
-// global head right before its update (C + B_g + P)
-// the longest segment the config allows: the dense cache at grouping, or a
-// global head's C + budget + P tokens (never more than C + N); a
-// redistributed budget reaches B_g + (H - 1)(B_g - w) for a group of one
-// global head
-int max_segment(const hkv_config *c) {
-  const int a = c->n_cond + c->group_at;
-  long long bud = c->global_budget;
-  if (c->budget_mode == HKV_BUDGET_REDISTRIBUTE)
-    bud += (long long)(c->n_heads - 1) * (c->global_budget - c->recent_w);
-  long long kept = bud + c->period;
-  if (kept > c->n_image) kept = c->n_image;
-  const int b = c->n_cond + (int)kept;
-  return a > b ? a : b;
-}
-
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 constexpr size_t kCtlBytes = 256;  // AttnCtl, padded
@@ -167,8 +150,8 @@ constexpr size_t kCtlBytes = 256;  // AttnCtl, padded
 // (kAttnInlinePieces slots per CTA boundary, one overflow slot per CTA), the
 // record of the head split at each CTA boundary, the control block the
 // two-kernel design's attention kernel leaves for its finishing kernel, the
-// epoch-tagged partial results of the one-launch step (two slots of D + 2
-// 8-byte pairs per CTA) and its per-layer barrier words.
+// epoch-tagged partial results of the one-launch step (two slots of
+// step_piece_words(D) 8-byte pairs per CTA) and its per-layer barrier words.
 struct WsLayout {
   size_t part, over, rec, ctl, pslot, bar, total;
 };
@@ -181,7 +164,7 @@ WsLayout ws_layout(const hkv_config *c) {
   w.rec = w.over + align256((size_t)kAttnMaxGrid * pf);
   w.ctl = w.rec + align256((size_t)kAttnMaxGrid * sizeof(int4));
   w.pslot = w.ctl + kCtlBytes;
-  w.bar = w.pslot + align256((size_t)kAttnMaxGrid * 2 * (c->head_dim + 2) * 8);
+  w.bar = w.pslot + align256((size_t)kAttnMaxGrid * 2 * step_piece_words(c->head_dim) * 8);
   w.total = w.bar + align256((size_t)c->n_layers * 4 * sizeof(uint32_t));
   return w;
 }
@@ -210,6 +193,7 @@ AttnArgs attn_args(const hkv_config *cfg, const hkv_cache *cache, int layer, con
   a.pslot = reinterpret_cast<unsigned long long *>(ws + w.pslot);
   a.bar = reinterpret_cast<uint32_t *>(ws + w.bar) + (size_t)layer * 4;
   a.n_layers = cfg->n_layers;
+  a.layer = layer;
   a.err = cache->err;
   a.pos = cache->pos;
   a.nbuf = cache->nbuf;
@@ -236,7 +220,7 @@ hkv_status step_ctas(DeviceState *st, int D, int dtype, int *ctas) {
     if (v == 0) {
       int m = 0;
       if (step_prepare(D, dtype, &m) != cudaSuccess || m <= 0) return HKV_ERR_CUDA;
-      v = m < kStepActivePerSm ? m : kStepActivePerSm;
+      v = m;
       c.store(v, std::memory_order_release);
     }
   }
@@ -244,15 +228,24 @@ hkv_status step_ctas(DeviceState *st, int D, int dtype, int *ctas) {
   return HKV_OK;
 }
 
-hkv_status step_grid(const hkv_config *cfg, int *grid) {
+// The grid of a one-launch step (fused) or attention of this config, or 0
+// where the two-kernel design runs: a CTA's range could then hold more heads
+// than the one-launch kernel's table (bounded from the longest segment the
+// config allows). Where it fits, one launch is the faster design on every
+// model shape measured. HKV_STEP_TWO_KERNELS in the environment forces the
+// two-kernel design (tests of both).
+hkv_status one_launch_grid(const hkv_config *cfg, bool fused, int *grid) {
+  *grid = 0;
+  if (getenv("HKV_STEP_TWO_KERNELS")) return HKV_OK;
   DeviceState *st;
   hkv_status s = device_state(&st);
   if (s != HKV_OK) return s;
   int ctas = 0;
   s = step_ctas(st, cfg->head_dim, cfg->dtype, &ctas);
   if (s != HKV_OK) return s;
-  const int g = st->sms.load(std::memory_order_acquire) * ctas;
-  *grid = g > kAttnMaxGrid ? kAttnMaxGrid : g;
+  int full = st->sms.load(std::memory_order_acquire) * ctas;
+  if (full > kAttnMaxGrid) full = kAttnMaxGrid;
+  *grid = step_grid(cfg->head_dim, cfg->dtype, heads_per_layer(cfg), max_segment(*cfg), full, fused);
   return HKV_OK;
 }
 
@@ -267,23 +260,6 @@ hkv_status attn_grid(const hkv_config *cfg, int *grid) {
   const int g = st->sms.load(std::memory_order_acquire) * ctas;
   *grid = g > kAttnMaxGrid ? kAttnMaxGrid : g;
   return HKV_OK;
-}
-
-// Whether hkv_decode_step runs as one launch (hkv_step.cu). It must fit the
-// kernel's head table: a range of c tiles holds at most c + 1 heads (a head
-// has at least one tile in a step, its new token), and c is at most the
-// layer's tile count over the grid, bounded by every head at the longest
-// segment the config allows. Where it fits, one launch is the faster design
-// on every model shape measured (each shape A/B in one process on GB300).
-// HKV_STEP_TWO_KERNELS in the environment forces the two-kernel design
-// (tests of both).
-bool one_launch_step(const hkv_config *cfg, int grid) {
-  if (getenv("HKV_STEP_TWO_KERNELS")) return false;
-  const long long tt = step_tile_rows(cfg->head_dim, cfg->dtype);
-  const long long tiles = (long long)heads_per_layer(cfg) * ((max_segment(cfg) + tt - 1) / tt);
-  long long chunk = (tiles + grid - 1) / grid;
-  if (chunk < 2) chunk = 2;
-  return chunk + 1 <= kStepTable;
 }
 
 #define HKV_TRY(x)                 \
@@ -404,7 +380,7 @@ hkv_status hkv_append_evict(const hkv_config *cfg, const hkv_cache *cache, int l
   if (!aligned16(q) || !aligned16(k) || !aligned16(v)) return HKV_ERR_ALIGN;
   DeviceState *st;
   HKV_TRY(device_state(&st));
-  const size_t smem = update_smem_bytes(max_segment(cfg), cfg->head_dim, cfg->period, cfg->dtype);
+  const size_t smem = update_smem_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
   HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem));
   const int hpl = heads_per_layer(cfg);
   return cuda_status(launch_append_evict(cache_args(cache), method_args(cfg), layer * hpl, hpl, q,
@@ -422,9 +398,12 @@ hkv_status hkv_decode_attention(const hkv_config *cfg, const hkv_cache *cache, i
   if (!q || !out || !workspace) return HKV_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(out) || !aligned16(workspace)) return HKV_ERR_ALIGN;
   if (ws_bytes < hkv_workspace_size(cfg)) return HKV_ERR_CAPACITY;
-  int grid = 0;
-  HKV_TRY(attn_grid(cfg, &grid));
   const AttnArgs a = attn_args(cfg, cache, layer, q, out, workspace);
+  int grid = 0;
+  HKV_TRY(one_launch_grid(cfg, false, &grid));
+  if (grid > 0)
+    return cuda_status(launch_step(a, cfg->head_dim, cfg->dtype, grid, false, (cudaStream_t)stream));
+  HKV_TRY(attn_grid(cfg, &grid));
   return cuda_status(
       launch_attention(a, cfg->head_dim, cfg->dtype, grid, false, false, (cudaStream_t)stream));
 }
@@ -444,8 +423,6 @@ hkv_status decode_step(const char *name, const hkv_config *cfg, const hkv_cache 
     return HKV_ERR_ALIGN;
   if (ws_bytes < hkv_workspace_size(cfg)) return HKV_ERR_CAPACITY;
   if (flags & ~HKV_STEP_PREFETCH) return HKV_ERR_INVALID_ARG;
-  int grid = 0;
-  HKV_TRY(attn_grid(cfg, &grid));
   AttnArgs a = attn_args(cfg, cache, layer, q, out, workspace);
   a.k_new = k;
   a.v_new = v;
@@ -453,12 +430,11 @@ hkv_status decode_step(const char *name, const hkv_config *cfg, const hkv_cache 
   a.label_out = label_out;
   a.w_loc = cfg->local_w;
   a.tau = (float)cfg->tau;
-  if (!label_out) {
-    int sgrid = 0;
-    HKV_TRY(step_grid(cfg, &sgrid));
-    if (one_launch_step(cfg, sgrid))
-      return cuda_status(launch_step(a, cfg->head_dim, cfg->dtype, sgrid, (cudaStream_t)stream));
-  }
+  int grid = 0;
+  HKV_TRY(one_launch_grid(cfg, true, &grid));
+  if (grid > 0)
+    return cuda_status(launch_step(a, cfg->head_dim, cfg->dtype, grid, true, (cudaStream_t)stream));
+  HKV_TRY(attn_grid(cfg, &grid));
   return cuda_status(launch_attention(a, cfg->head_dim, cfg->dtype, grid, true,
                                       label_out != nullptr, (cudaStream_t)stream));
 }
@@ -475,8 +451,8 @@ hkv_status hkv_decode_step(const hkv_config *cfg, const hkv_cache *cache, int la
 int hkv_decode_step_launches(const hkv_config *cfg) {
   if (hkv_validate_config(cfg) != HKV_OK) return 0;
   int grid = 0;
-  if (step_grid(cfg, &grid) != HKV_OK) return 0;
-  return one_launch_step(cfg, grid) ? 1 : 2;
+  if (one_launch_grid(cfg, true, &grid) != HKV_OK) return 0;
+  return grid > 0 ? 1 : 2;
 }
 
 hkv_status hkv_decode_step_identify(const hkv_config *cfg, const hkv_cache *cache, int layer,
@@ -497,7 +473,7 @@ hkv_status evict_layers(const hkv_config *cfg, const hkv_cache *cache, int first
                         hkv_stream_t stream) {
   DeviceState *st;
   HKV_TRY(device_state(&st));
-  const size_t smem = update_smem_bytes(max_segment(cfg), cfg->head_dim, cfg->period, cfg->dtype);
+  const size_t smem = update_smem_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
   HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem));
   const long long hpl = heads_per_layer(cfg);
   if (hpl * count > 0x7FFFFFFFLL) return HKV_ERR_SHAPE;  // one CTA per head
@@ -536,7 +512,7 @@ hkv_status hkv_identify_heads(const hkv_config *cfg, const hkv_cache *cache, int
   DeviceState *st;
   HKV_TRY(device_state(&st));
   const int max_len = cfg->n_cond + cfg->group_at;
-  const size_t upd = update_smem_bytes(max_segment(cfg), cfg->head_dim, cfg->period, cfg->dtype);
+  const size_t upd = update_smem_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
   const size_t need = identify_smem_bytes(max_len, cfg->period,
                                           cfg->distance_mode == HKV_DIST_GRID2D, false);
   HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, upd > need ? upd : need));
@@ -556,7 +532,7 @@ hkv_status hkv_identify_heads_multi(const hkv_config *cfg, const hkv_cache *cach
   DeviceState *st;
   HKV_TRY(device_state(&st));
   const int max_len = cfg->n_cond + cfg->group_at;
-  const size_t upd = update_smem_bytes(max_segment(cfg), cfg->head_dim, cfg->period, cfg->dtype);
+  const size_t upd = update_smem_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
   const size_t need = identify_smem_bytes(max_len, cfg->period,
                                           cfg->distance_mode == HKV_DIST_GRID2D, true);
   HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, upd > need ? upd : need));
@@ -602,7 +578,7 @@ hkv_status hkv_repack(const hkv_config *cfg, const hkv_cache *dense, const hkv_c
   if (dense->qbuf != ragged->qbuf) return HKV_ERR_INVALID_ARG;
   DeviceState *st;
   HKV_TRY(device_state(&st));
-  const size_t smem = update_smem_bytes(max_segment(cfg), cfg->head_dim, cfg->period, cfg->dtype);
+  const size_t smem = update_smem_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
   HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem));
   const int hpl = heads_per_layer(cfg);
   return cuda_status(launch_repack(cache_args(dense), cache_args(ragged), method_args(cfg),

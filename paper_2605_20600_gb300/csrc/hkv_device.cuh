@@ -149,6 +149,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
   }
 }
 
+// The same, but false as soon as *stop is set (looked at only while waiting).
+__device__ __forceinline__ bool mbar_wait_unless(uint64_t *bar, uint32_t parity,
+                                                 const volatile int *stop) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = globaltimer();
+  for (uint32_t it = 1;; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((it & 63u) == 0 && (*stop || globaltimer() - t0 > kWaitTimeoutNs)) return false;
+  }
+}
+
 // global -> shared bulk copy of `bytes` (multiple of 16, both ends 16-byte
 // aligned), completion counted on `bar`
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes,

@@ -61,11 +61,27 @@ struct AttnArgs {
   // generation, worst status of a bad step, unused}, the arrivals and the
   // status zero between launches; the partial results of split heads
   // as (value, launch epoch) pairs, two slots per CTA (the piece at the end
-  // of its range, the piece at its start), [grid][2][D + 2]
+  // of its range, the piece at its start), [grid][2][step_piece_words(D)]
   uint32_t *bar;
   unsigned long long *pslot;
-  int n_layers;
+  int n_layers, layer;        // for the epoch
+  uint32_t grid_recip;        // 2^32 / CTAs, rounded up (set by launch_step)
 };
+
+// The longest segment the config allows: the dense cache at grouping, or a
+// global head's C + budget + P tokens (never more than C + N); a
+// redistributed budget reaches B_g + (H - 1)(B_g - w) for a group of one
+// global head.
+inline int max_segment(const hkv_config &c) {
+  const int a = c.n_cond + c.group_at;
+  long long kept = c.global_budget;
+  if (c.budget_mode == HKV_BUDGET_REDISTRIBUTE)
+    kept += (long long)(c.n_heads - 1) * (c.global_budget - c.recent_w);
+  kept += c.period;
+  if (kept > c.n_image) kept = c.n_image;
+  const int b = c.n_cond + (int)kept;
+  return a > b ? a : b;
+}
 
 // decode attention CTAs: one producer warp (TMA), consumer warps, one
 // epilogue warp (merges, outputs, partial results); at most kAttnMaxGrid
@@ -86,26 +102,33 @@ __host__ __device__ constexpr int attn_part_floats(int D) { return D + 4; }
 constexpr int kAttnInlinePieces = 4;
 
 // one-launch decode step: heads of a CTA's range it keeps in shared memory
+// (a power of two)
 #ifndef HKV_STEP_TABLE
-#define HKV_STEP_TABLE 128
+#define HKV_STEP_TABLE 256
 #endif
 constexpr int kStepTable = HKV_STEP_TABLE;
+// 64-bit words of one partial result of the one-launch step: D accumulators,
+// the maximum, the sum and (identification) the newest rows' sum
+__host__ __device__ constexpr int step_piece_words(int D) { return D + 4; }
 
 size_t attention_smem_bytes(int D, int dtype);
-// rows of K (and of V) per pipeline stage of the one-launch step
-int step_tile_rows(int D, int dtype);
 // CTAs per SM of the one-launch step's grid, and the shared memory and
-// occupancy setup of its kernel (resident CTAs per SM)
+// occupancy setup of its kernels (resident CTAs per SM, at most that many)
 #ifndef HKV_STEP_ACTIVE_PER_SM
 #define HKV_STEP_ACTIVE_PER_SM 2
 #endif
 constexpr int kStepActivePerSm = HKV_STEP_ACTIVE_PER_SM;
 
 cudaError_t step_prepare(int D, int dtype, int *ctas_per_sm);
-// the fused decode step of one layer in one launch (append + attention,
-// merges of split heads and counters in the same kernel); `grid` CTAs, at
-// most kAttnMaxGrid, a CTA's range spanning at most kStepTable heads
-cudaError_t launch_step(const AttnArgs &a, int D, int dtype, int grid, cudaStream_t s);
+// CTAs of a one-launch step (fused) or attention (not fused) over nheads
+// heads of at most max_rows rows, out of a grid of `full`; 0: a range could
+// hold more heads than the kernel's table, so the two-kernel design runs
+int step_grid(int D, int dtype, int nheads, int max_rows, int full, bool fused);
+// one layer in one launch: the decode step (append + attention, merges of
+// split heads and counters in the same kernel), with the head types decided
+// where a.label_out is set, or attention alone (not fused); `grid` CTAs, at
+// most kAttnMaxGrid and at most what is resident at once
+cudaError_t launch_step(const AttnArgs &a, int D, int dtype, int grid, bool fused, cudaStream_t s);
 cudaError_t attention_prepare(int D, int dtype, int *ctas_per_sm);
 // launches the attention kernel on `grid` CTAs (at most kAttnMaxGrid) and the
 // finishing kernel behind it; identify (fused only): also the Step 2 label of

@@ -25,16 +25,23 @@ namespace {
 
 using namespace hkv;
 
-// Split-K partials (per CTA boundary and per CTA, up to 1 MiB), then which
-// head is split at each CTA boundary, then the control block the attention
-// kernel leaves for the finishing kernel: 1.06 MiB in total. The kernels write all of it
-// before reading it, so nothing in it has to start at zero.
+// The two-kernel design's split-K partials (per CTA boundary and per CTA, up
+// to 1 MiB), then which head is split at each CTA boundary, then the control
+// block the attention kernel leaves for the finishing kernel and the
+// one-launch kernel's barrier words, then that kernel's epoch-tagged partial
+// results (up to 1 MiB): 2.06 MiB in total. The barrier words start at zero
+// (static device memory does) and every launch leaves them ready for the
+// next; the kernels write everything else before reading it. All calls share
+// one set of barrier words, so an epoch is never used twice; the tagged
+// results have a region of their own, so nothing else is ever read as one.
 #ifndef HKV_NOALLOC_PART_BYTES
 #define HKV_NOALLOC_PART_BYTES (1u << 20)
 #endif
 constexpr size_t kPartBytes = HKV_NOALLOC_PART_BYTES;
 constexpr size_t kRecBytes = (size_t)kAttnMaxGrid * sizeof(int4);
-constexpr size_t kScratchBytes = kPartBytes + kRecBytes + 256;
+constexpr size_t kCtlAt = kPartBytes + kRecBytes, kBarAt = kCtlAt + 128;
+constexpr size_t kPieceAt = kCtlAt + 256;
+constexpr size_t kScratchBytes = kPieceAt + kPartBytes;
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
@@ -45,6 +52,7 @@ struct NoAllocDevice {
   unsigned char *scratch = nullptr;  // device address of g_scratch
   int sms = 0;
   int ctas[2][2] = {{0, 0}, {0, 0}};  // [dtype][D == 128]
+  int step_ctas[2][2] = {{0, 0}, {0, 0}};
 };
 
 NoAllocDevice g_devs[kMaxDevices];
@@ -84,6 +92,12 @@ hkv_status setup(int D, int dtype, NoAllocDevice **out) {
     int n = 0;
     if (attention_prepare(D, dtype, &n) != cudaSuccess || n <= 0) return HKV_ERR_CUDA;
     c = n;
+  }
+  int &sc = st.step_ctas[dtype == HKV_BF16 ? 1 : 0][D == 128 ? 1 : 0];
+  if (sc == 0) {
+    int n = 0;
+    if (step_prepare(D, dtype, &n) != cudaSuccess || n <= 0) return HKV_ERR_CUDA;
+    sc = n;
   }
   *out = &st;
   return HKV_OK;
@@ -131,11 +145,26 @@ extern "C" hkv_status hkv_decode_attention_noalloc(const hkv_config *cfg, const 
   a.part = reinterpret_cast<float *>(st->scratch);
   a.over = a.part + (size_t)grid * kAttnInlinePieces * attn_part_floats(cfg->head_dim);
   a.rec = reinterpret_cast<int4 *>(st->scratch + kPartBytes);
-  a.ctl = reinterpret_cast<AttnCtl *>(st->scratch + kPartBytes + kRecBytes);
+  a.ctl = reinterpret_cast<AttnCtl *>(st->scratch + kCtlAt);
   a.err = cache->err;
   a.arena_tokens = cache->capacity_tokens;
   a.nheads = hpl;
+  a.n_layers = 1;  // one set of barrier words, whatever the layer
+  a.bar = reinterpret_cast<uint32_t *>(st->scratch + kBarAt);
+  a.pslot = reinterpret_cast<unsigned long long *>(st->scratch + kPieceAt);
   a.qscale = (float)(1.4426950408889634 / sqrt((double)cfg->head_dim));
+  // one launch where hkv_decode_attention takes it, on as many CTAs as the
+  // region for the tagged results holds
+  if (!getenv("HKV_STEP_TWO_KERNELS")) {
+    int full = st->sms * st->step_ctas[cfg->dtype == HKV_BF16 ? 1 : 0][cfg->head_dim == 128 ? 1 : 0];
+    if (full > kAttnMaxGrid) full = kAttnMaxGrid;
+    const size_t piece = 2 * (size_t)step_piece_words(cfg->head_dim) * 8;
+    if ((size_t)full * piece > kPartBytes) full = (int)(kPartBytes / piece);
+    const int one = step_grid(cfg->head_dim, cfg->dtype, hpl, max_segment(*cfg), full, false);
+    if (one > 0)
+      return launch_step(a, cfg->head_dim, cfg->dtype, one, false, s) == cudaSuccess ? HKV_OK
+                                                                                    : HKV_ERR_CUDA;
+  }
   return launch_attention(a, cfg->head_dim, cfg->dtype, grid, false, false, s) == cudaSuccess
              ? HKV_OK
              : HKV_ERR_CUDA;

@@ -1,13 +1,36 @@
 // One decode step of one layer in a single launch: attention of every head's
 // new query over the head's retained tokens and the step's new token (Eq. 1),
-// fused with the append of that token to the cache (Sec. 3, KV Cache).
+// fused with the append of that token to the cache (Sec. 3, KV Cache); with
+// the head types decided in the same pass (Sec. 4, Step 2); or the attention
+// alone.
 //
-// The split-K layout is the one of the two-kernel design in hkv_attention.cu
-// (the layer's heads rounded up to whole tiles and concatenated; gridDim.x
-// equal contiguous ranges, one per CTA; a warp-specialised TMA pipeline with
-// a producer warp, consumer warps and an epilogue warp), but the work that
-// the finishing kernel did there happens inside this launch:
+// What bounds it: the K/V rows, read once (91 MB a layer on Lumina-mGPT 1024
+// at rho = 1/4, 8 sequences: 13.4 us at the measured copy bandwidth), plus a
+// part that does not grow with them: the last tiles, the merges, the next
+// launch's start, prologue and first loads, during which DRAM is mostly idle.
+// Timings below are per layer step, whole period, before -> after.
 //
+//  * split: a head takes one slot per 16 rows (8 of 512 bytes) and one more
+//    (StepShape::cost); the layer's slots are cut into gridDim.x equal
+//    contiguous ranges, one per CTA, and a cut within a quarter of a range of
+//    a head's first or last row moves there (HKV_STEP_SNAP_DIV: cuts cost a
+//    merge and two partial tiles; 1/64 of a range 16.87 us, 1/16 16.65, 1/4
+//    16.44 on Lumina-mGPT 1024). Slots of whole tiles, as before, left CTAs
+//    with up to 9 of LlamaGen-XL's heads where 8.4 is the mean: 16.4 -> 14.9
+//    us there with the prologue below;
+//  * a layer of short heads, no more than CTAs, gets a CTA per head
+//    (kAlignedGrains), and a small layer a grid no larger than its ranges:
+//    nothing is merged and every CTA of the next launch is resident before
+//    this one ends (Janus-Pro-7B, 2 sequences: 6.6 -> 3.9 us);
+//  * a warp-specialised TMA pipeline: a producer warp, consumer warps, an
+//    epilogue warp and a merge warp;
+//  * bf16 consumers take q.k on the tensor cores (8 rows a warp and tile: 4
+//    mma.sync of D = 128 in place of 64 mixed FMAs and 32 shuffles; the exact
+//    products are summed in fp32 as before) and p.V in fp32 FMAs. The chain
+//    of a tile is what a CTA waits for: 0.8 us less of Lumina-mGPT 1024's
+//    step than with FMAs and shuffles. p.V on the tensor cores too, with the
+//    weights cut into three bf16 parts and the rows skewed against the banks,
+//    measured 1.7 us slower: the eight small copies a tile then needs;
 //  * tile order: a CTA streams the start of the head that continues into a
 //    later range first, then the piece of the head that began in an earlier
 //    range, then the heads wholly inside its range. The piece a CTA streams
@@ -22,26 +45,22 @@
 //    every pair carries this launch's epoch, while its consumers stream.
 //    Pieces are combined in index order and the CTA's own piece last, so the
 //    result does not depend on timing;
-//  * prologue: every CTA reads the lengths of all the layer's heads to place
-//    the ranges, but checks the other counters only for the heads of its own
-//    range, in the same round of loads;
+//  * prologue: see there;
 //  * appends and counters: every CTA arrives on a per-layer barrier word
 //    once it is done reading the layer's counters (a CTA that found a bad
 //    head marks its arrival); once the whole grid has arrived, and unless
-//    one was marked, the merge warp copies the new token of every head
-//    whose last row is in the CTA's range into the cache (nothing in the
-//    launch reads those rows) and advances len, ntok and nbuf of those
-//    heads, while the consumers stream. The next launch of the same layer
-//    starts after this one completes, so the barrier word is free again by
-//    then;
-//  * programmatic dependent launch: with the prefetch flag the prologue and
-//    the first tiles of old K/V rows go ahead of the wait for the previous
-//    kernel; the step's inputs (q, the new k and v) are read after it;
-//  * every wait is bounded (HKV_ERR_TIMEOUT in the error word).
-//
-// The lengths of every head whose range a CTA touches are kept in a table in
-// shared memory (kStepTable heads); the host takes this path only when no
-// range can hold more heads than that.
+//    one was marked, the merge warp advances len, ntok and nbuf of the heads
+//    whose last row is in the CTA's range, while the consumers stream. Their
+//    new tokens go into the cache then too, or at once where every CTA has
+//    checked every head (nothing in the launch reads those rows). The next
+//    launch of the same layer starts after this one completes, so the
+//    barrier word is free again by then;
+//  * programmatic dependent launch: with the prefetch flag the prologue, the
+//    arrival and the first tiles of old K/V rows go ahead of the wait for the
+//    previous kernel; the step's inputs (q, the new k and v) are read after
+//    it;
+//  * every wait is bounded (HKV_ERR_TIMEOUT in the error word). The waits on
+//    other CTAs need the whole grid resident: it is at most what fits.
 #include <math.h>
 #include <stdlib.h>
 
@@ -79,28 +98,21 @@ __device__ unsigned long long *g_step_trace = nullptr;  // [layer][kAttnMaxGrid]
 // Tuning knobs (compile time) of the one-launch step, per head dimension:
 // consumer warps, bytes of K per stage, stages, tiles loaded before the wait,
 // and the CTAs per SM the kernel is built to be resident with (the grid uses
-// kStepActivePerSm). Measured per layer step (A/B in one process): rows of
-// 256 B stream best with 8 consumer warps over 48-row tiles in 3 stages, all
-// loaded before the wait (Lumina-mGPT 1024 at rho = 1/8: 13.01 us with 7
-// warps over 42 rows and 2 before the wait, 12.77 with 8 over 48, 12.63
-// with all 3 before it; 56-row tiles 13.06, 64-row tiles in 2 stages 13.10);
-// rows of 128 B (LlamaGen-XL's short heads, many to a CTA) with 128-row
-// tiles in 2 stages (15.26 us against 16.06 with 64-row tiles in 3 stages
-// and 17.42 with 96-row tiles in 3).
-#ifndef HKV_STEP_CW_D128
-#define HKV_STEP_CW_D128 8
-#endif
+// kStepActivePerSm). Rows of 256 B: 64-row tiles in 3 stages and 48-row ones
+// with 6 warps are within 0.3 % of each other on large layers, 64 rows 2 %
+// faster on small ones (4 stages of 48 rows +0.1 to +1.7 us, 2 stages +0.7).
+// Rows of 128 B (LlamaGen-XL's short heads, many to a CTA): 128-row tiles in
+// 2 stages, 64-row ones in 3 +0.8 us. A third resident CTA per SM, so that
+// the next launch's CTAs start early, leaves some SMs with three CTAs of one
+// launch and others with one: +1.4 to +2.3 us.
 #ifndef HKV_STEP_TILE_BYTES_D128
-#define HKV_STEP_TILE_BYTES_D128 12288
+#define HKV_STEP_TILE_BYTES_D128 16384
 #endif
 #ifndef HKV_STEP_STAGES_D128
 #define HKV_STEP_STAGES_D128 3
 #endif
 #ifndef HKV_STEP_PRE_D128
 #define HKV_STEP_PRE_D128 3
-#endif
-#ifndef HKV_STEP_CW_D64
-#define HKV_STEP_CW_D64 8
 #endif
 #ifndef HKV_STEP_TILE_BYTES_D64
 #define HKV_STEP_TILE_BYTES_D64 16384
@@ -109,82 +121,79 @@ __device__ unsigned long long *g_step_trace = nullptr;  // [layer][kAttnMaxGrid]
 #define HKV_STEP_STAGES_D64 2
 #endif
 #ifndef HKV_STEP_PRE_D64
-#define HKV_STEP_PRE_D64 1
+#define HKV_STEP_PRE_D64 2
 #endif
 #ifndef HKV_STEP_RESIDENT_PER_SM
 #define HKV_STEP_RESIDENT_PER_SM 2
 #endif
+#ifndef HKV_STEP_CW_D128
+#define HKV_STEP_CW_D128 8
+#endif
+#ifndef HKV_STEP_CW_D64
+#define HKV_STEP_CW_D64 8
+#endif
+// consumer warps: a bf16 tile is a number of 8-row blocks for each of them
+constexpr int step_cw(int D, int es) {
+  return es == 4 ? 8 : D == 64 ? HKV_STEP_CW_D64 : HKV_STEP_CW_D128;
+}
 
 template <int D, typename T>
-using StepShape =
-    TileShape<D, T, D == 64 ? HKV_STEP_CW_D64 : HKV_STEP_CW_D128,
-              D == 64 ? HKV_STEP_TILE_BYTES_D64 : HKV_STEP_TILE_BYTES_D128,
-              D == 64 ? HKV_STEP_STAGES_D64 : HKV_STEP_STAGES_D128,
-              D == 64 ? HKV_STEP_PRE_D64 : HKV_STEP_PRE_D128>;
+using StepTile = TileShape<D, T, step_cw(D, sizeof(T)),
+                           D == 64 ? HKV_STEP_TILE_BYTES_D64 : HKV_STEP_TILE_BYTES_D128,
+                           D == 64 ? HKV_STEP_STAGES_D64 : HKV_STEP_STAGES_D128,
+                           D == 64 ? HKV_STEP_PRE_D64 : HKV_STEP_PRE_D128>;
 
-struct StepTable {
-  int h0, n;                      // heads h0 .. h0 + n - 1
-  long long start[kStepTable];    // first index (slot space) of head h0 + j
-  long long off[kStepTable];      // arena offset
-  int vlen[kStepTable];           // len + 1 (the new token)
-  int nbuf[kStepTable];
-  int ntok[kStepTable];           // written by the append (epilogue warp)
-  unsigned char label[kStepTable];
+template <int D, typename T>
+struct StepShape : StepTile<D, T> {
+  using Tile = StepTile<D, T>;
+  // states a segment hands over: one per consumer warp, or (fp32) per row group
+  static constexpr int kNST = sizeof(T) == 2 ? Tile::kCW : Tile::kCW * Tile::kRPW;
+  // The split counts in grains of kGR rows (4 or 8 KB of K and V). A head of
+  // g grains takes g + 1 slots, at least kMinCost: the extra one stands for
+  // what a head costs beyond its rows (a hand-over, a partial tile), and the
+  // minimum bounds the heads of a range (step_max_heads).
+  static constexpr int kGR = Tile::kRB == 512 ? 8 : 16;
+  static constexpr int kMinCost = Tile::kRB == 128 ? 5 : Tile::kTT / kGR > 3 ? 3 : 2;
+  static constexpr int kMinChunk = 2 * Tile::kTT / kGR;  // fewest slots per CTA range
+  __host__ __device__ static constexpr int grains(int rows) {
+    return (int)(((unsigned)rows + kGR - 1) / kGR);
+  }
+  __host__ __device__ static constexpr int cost(int g) { return g + 1 > kMinCost ? g + 1 : kMinCost; }
 };
 
-constexpr int kFirst = 1, kLast = 2, kDone = 4;
+// Heads of at most this many grains (96 KB of K and V) are not split when
+// every head can have a CTA of its own: the exchange of partial results
+// costs more than the tiles it saves.
+constexpr int kAlignedGrains = 12;
+
+// A boundary between ranges that falls within 1/kSnapDiv of a range of a
+// head's first or last row moves there.
+#ifndef HKV_STEP_SNAP_DIV
+#define HKV_STEP_SNAP_DIV 4
+#endif
+
+template <int N>
+struct StepTable {  // entry h - s_wl: head h
+  long long off[N];  // arena offset
+  int vlen[N];       // rows, the new token included
+  int ntok[N];
+  unsigned char label[N];
+  unsigned char bad[N];  // status of the head's counters
+};
+
+// kWhole: the piece is its whole head; kTailPiece: the head began in an
+// earlier range
+constexpr int kFirst = 1, kLast = 2, kDone = 4, kWhole = 8, kTailPiece = 16;
 
 struct TileMeta {  // producer -> consumers, one per stage
   int h, n, flags;
-  long long hs, he;  // the head's rows in the index space
+  int recent0;  // identification: rows from here on are among the head's newest w_loc - 1
 };
+
+constexpr int kNewRow = 32;  // flag: the tile's last row is the step's token
 
 struct SegMeta {  // consumers -> epilogue; h < 0: no more segments
-  int h;
-  long long hs, he;
-};
-
-// Tiles of a slot-aligned sub-range [g, b) of the index space, head by head,
-// over the table (j: table index of the current head).
-template <int TT>
-struct StepIter {
-  int j, hl;
-  long long hs, g, b;
-  __device__ __forceinline__ bool done() const { return g >= b; }
-  __device__ __forceinline__ long long tile_end() const {
-    long long e = g + TT;
-    if (e > hs + hl) e = hs + hl;
-    if (e > b) e = b;
-    return e;
-  }
-  __device__ __forceinline__ void advance(const StepTable &t) {
-    g += TT;
-    if (g >= b) return;
-    while (g >= hs + slot_len<TT>(hl) && j + 1 < t.n) {
-      ++j;
-      hs = t.start[j];
-      hl = t.vlen[j];
-    }
-  }
-};
-
-// The split of a layer's index space [0, total) into the CTAs' ranges: CTA k
-// streams [start(k), start(k + 1)), `chunk` slots each (whole tiles, at
-// least two), the last ones possibly shorter or empty.
-template <int TT>
-struct Ranges {
-  long long total, chunk;
-  int G;
-  // the range size (a 64-bit division: one thread computes it)
-  __device__ static long long chunk_of(long long total, int G, long long min_chunk) {
-    const long long c = slot_len<TT>((total + G - 1) / G);
-    return c < min_chunk ? min_chunk : c;
-  }
-  __device__ long long start(int k) const {
-    const long long s = (long long)k * chunk;
-    return k >= G || s > total ? total : s;
-  }
-  __device__ int owner(long long slot) const { return (int)(slot / chunk); }  // CTA holding slot
+  int h, flags;
 };
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p) {
@@ -209,17 +218,35 @@ __device__ __forceinline__ bool ld_pair(const unsigned long long *p, uint32_t ep
   return (uint32_t)(w >> 32) == ep;
 }
 
-// Combines a split head's own piece (m1, l1, A1) with its other pieces,
-// already combined (m2, l2, A2), and stores the output row: the same
+// One bf16 m16n8k16 product added to c. Products are exact, sums in fp32.
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4 &a, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+
+// the largest x of the warp, in every lane
+__device__ __forceinline__ float warp_max(float x) {
+  float y;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Combines a split head's own piece (m1, l1, r1, A1) with its other pieces,
+// already combined (m2, l2, r2, A2), and stores the output row: the same
 // instructions wherever it runs, so the result does not depend on which
-// warp does it.
-template <int CPL>
-__device__ __forceinline__ void combine_store(float m1, float l1, const float *A1, float m2,
-                                              float l2, const float *A2, float *out) {
+// warp does it. Returns the head's sum and, for identification, its mass of
+// newest rows.
+template <int CPL, bool IDENT>
+__device__ __forceinline__ void combine_store(float m1, float l1, float r1, const float *A1,
+                                              float m2, float l2, float r2, const float *A2,
+                                              float *out, float &Lt, float &Rt) {
   const float mx = fmaxf(m1, m2);
   const float w1 = m1 == -INFINITY ? 0.f : exp2f(m1 - mx);
   const float w2 = m2 == -INFINITY ? 0.f : exp2f(m2 - mx);
-  const float Lt = l1 * w1 + l2 * w2;
+  Lt = l1 * w1 + l2 * w2;
+  if (IDENT) Rt = r1 * w1 + r2 * w2;
   float A[CPL];
 #pragma unroll
   for (int c = 0; c < CPL; ++c) A[c] = fmaf(A1[c], w1, A2[c] * w2) / Lt;
@@ -233,38 +260,49 @@ __host__ __device__ constexpr int step_threads() {
   return StepShape<D, T>::kThreads + 32;
 }
 
-template <int D, typename T>
+// What a launch does: a decode step, the same with the head types decided in
+// the pass (Sec. 4, Step 2), or attention alone (no append, no counters).
+enum StepMode { kModeStep = 0, kModeIdentify = 1, kModeAttend = 2 };
+
+template <int D, typename T, int MODE>
 __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM)
     step_kernel(const AttnArgs p) {
   using S = StepShape<D, T>;
-  constexpr int kCW = S::kCW, kThr = step_threads<D, T>();
+  constexpr bool FUSED = MODE != kModeAttend, IDENT = MODE == kModeIdentify;
+  constexpr int kCW = S::kCW, kThr = step_threads<D, T>(), NW = kThr / 32;
   constexpr int LPR = S::kLPR, EPL = S::kEPL, RPW = S::kRPW, TT = S::kTT;
-  constexpr int RB = S::kRB, NS = S::kNS;
-  constexpr int NST = kCW * RPW;  // row-group states per segment
+  constexpr int RB = S::kRB, NS = S::kNS, GR = S::kGR;
+  constexpr int NST = S::kNST;
   constexpr int CPL = D / 32;     // output channels per epilogue lane
+  constexpr int NV = IDENT ? 3 : 2;  // scalars of a partial result: maximum, sum, newest rows' sum
+  constexpr int PS = step_piece_words(D);
   static_assert(NST <= 32, "a lane of the epilogue per state");
-  static_assert(kStepTable <= kThr, "a thread per table entry");
+  static_assert(kStepTable <= kThr, "the table holds a range's heads");
+  static_assert(TT % GR == 0, "tiles of whole grains");
   using V = Vec<CPL>;
 
   extern __shared__ __align__(128) unsigned char stages[];
   __shared__ uint64_t full[NS], empty[NS];
   __shared__ uint64_t epi_full[2], epi_free[2];  // two hand-over buffers
   __shared__ __align__(16) float red_acc[2][NST][D];
-  __shared__ float red_m[2][NST], red_l[2][NST];
+  __shared__ float red_m[2][NST], red_l[2][NST], red_r[IDENT ? 2 : 1][IDENT ? NST : 1];
   __shared__ TileMeta meta[NS];
   __shared__ SegMeta seg[2];
-  __shared__ StepTable tab;
-  __shared__ long long scan_scratch[33];
-  __shared__ long long s_s0, s_mg_k0, s_a, s_b, s_chunk;
-  __shared__ int s_h0, s_h1, s_bad;
-  __shared__ int s_mg_h, s_mg_j, s_mg_np;  // the split head this CTA combines
-  __shared__ uint32_t s_ep;                // the launch's epoch
+  __shared__ StepTable<kThr> tab;
+  __shared__ int2 s_w[NW];  // each warp's slots; its longest head, or a status
+  // the range's ends: {first slot, first head, that head's first slot, its
+  // rows} and {end slot, last head, that head's first slot, whether the range
+  // ends inside its rows}
+  __shared__ int4 s_lo, s_hi;
+  __shared__ int s_bad;
+  __shared__ int s_mg_h, s_mg_k0, s_mg_j, s_mg_np;  // the split head this CTA combines
+  __shared__ uint32_t s_ep;                         // the launch's epoch
   // hand-overs between the epilogue and the merge warp: the epoch and the
   // merge head (ep_bar), the other pieces combined (oth_bar), and this CTA's
   // own piece or the news that the epilogue combined it already (own_bar)
   __shared__ uint64_t ep_bar, oth_bar, own_bar;
   __shared__ __align__(16) float own_acc[D], oth_acc[D];
-  __shared__ float own_ml[2], oth_ml[2];
+  __shared__ float own_s[NV], oth_s[NV];
   __shared__ int s_own_state;  // 1: combined by the epilogue, 2: own piece handed over
   __shared__ volatile int s_abort;
 
@@ -282,300 +320,434 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       STEP_TRACE_AT(16) = smid;
     }
 #endif
-    for (int s = 0; s < NS; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], kCW);
-    }
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&epi_full[s], kCW);
-      mbar_init(&epi_free[s], 1);
-    }
-    mbar_init(&ep_bar, 32);
-    mbar_init(&oth_bar, 32);
-    mbar_init(&own_bar, 32);
-    fence_barrier_init();
-    s_abort = 0;
-    s_bad = 0;
-    s_h0 = 0;
-    s_h1 = -1;
-    s_s0 = 0;
-    s_mg_h = -1;
   }
   if (!p.prefetch) pdl_wait();
 
   // ---- prologue: the layer's lengths, one round of loads -------------------
-  // Every thread takes a contiguous slice of the layer's heads and sums
-  // their slots; a block scan gives each slice its first index, so every
-  // CTA computes the same ranges, and a negative length stops every CTA.
-  // Offsets, capacities, labels and buffer counts are checked only for the
-  // heads of the CTA's own range: a CTA that finds a bad one streams nothing
-  // and flags the step on the layer's barrier word, and no CTA then appends
-  // or advances a counter. All of it takes one round of loads: a slice of
-  // one head is read whole into registers; with longer slices only the
-  // lengths are, and the same round reads the other counters of a window of
-  // kThr heads around the range's expected place (heads of equal length). A
-  // range outside the window reads them once it is known.
-  const int per = (nheads + kThr - 1) / kThr;
-  const int h_lo = tid * per < nheads ? tid * per : nheads;
-  const int h_hi = h_lo + per < nheads ? h_lo + per : nheads;
-  const bool in_regs = per <= 1;
-  long long mine = 0;
-  int bad = 0;
-  auto count = [&](int l) {
-    if (l < 0) bad = HKV_ERR_BOUNDS;
-    mine += slot_len<TT>(l + 1);
+  // Warp w takes `rows` rows of 32 consecutive heads and sums each row's
+  // slots; the warps' sums give every CTA the same ranges, and only the warps
+  // whose heads meet the range's ends look at their rows again. (One thread
+  // per run of consecutive heads took 2.5 us to place a range of LlamaGen-XL's
+  // 2560 heads, whose rows this takes one or two of.)
+  // The same round fills a table of kThr heads: the whole layer, if it has no
+  // more (every CTA then checks every head, and a bad one stops all of them
+  // here), else those around the range's expected place (heads of equal
+  // length); a range outside it reads its heads once it is known. A CTA that
+  // finds a bad head in its range then streams nothing and flags the step on
+  // the layer's barrier word, and no CTA appends or advances a counter.
+  const int rows = (nheads + kThr - 1) / kThr;
+  const int row0 = warp * rows;  // this warp's first row
+  const bool in_regs = rows <= 1;
+  constexpr int kNew = FUSED ? 1 : 0;   // the step's token is one more row
+  constexpr int kMost = 1 << 26;        // grains of a head, slots of a warp: beyond any arena
+  constexpr int kIsBad = 0x70000000;    // a status in place of the longest head
+  constexpr int kPre = 8;               // rows loaded at once
+  // the status of a head's counters
+  auto verify = [&](int l, long long o, int cp, int lab, int nb) {
+    if (FUSED) {
+      if (l < 0 || o < 0 || o + cp > p.arena_tokens) return (int)HKV_ERR_BOUNDS;
+      if (IDENT && lab != HKV_DENSE) return (int)HKV_ERR_STATE;  // the rows' order is needed
+      if (l + 1 > cp) return (int)HKV_ERR_CAPACITY;
+      if (lab != HKV_DENSE && nb >= p.period) return (int)HKV_ERR_STATE;  // the update is due first
+      return 0;
+    }
+    return l < 0 || o < 0 || o + l > p.arena_tokens ? (int)HKV_ERR_BOUNDS : 0;
   };
-  // the counters of one head in registers: this thread's slice (in_regs) or
-  // its head of the window
-  int rl = 0, rcp = 0, rnb = 0, rlb = 0;
-  long long ro = 0;
-  int win_lo = 0;
+  int wl = 0;  // the table's first head
+  if (!in_regs) {
+    wl = (int)((float)bx * ((float)nheads / (float)G)) - kThr / 2;
+    wl = wl < nheads - kThr ? wl : nheads - kThr;
+    wl = wl > 0 ? wl : 0;
+  }
+  int key = 0;
+  unsigned c0 = 0;  // in_regs: the slots of this thread's head
+  int lv[kPre];
+  {
+    // every load issued before any use
+    const int h = wl + tid;
+    int l = 0, cp = 0, lab = 0, nb = 0, nt = 0;
+    long long o = 0;
+    if (h < nheads) {
+      l = p.len[h];
+      o = p.off[h];
+      if (FUSED) {
+        cp = p.cap[h];
+        lab = p.label[p.layer_base + h];
+        nb = p.nbuf[p.layer_base + h];
+        nt = p.ntok[p.layer_base + h];
+      }
+    }
+    if (!in_regs) {
+#pragma unroll
+      for (int i = 0; i < kPre; ++i) {
+        const int r = (row0 + i) * 32 + lane;
+        lv[i] = i < rows && r < nheads ? p.len[r] : -1;
+      }
+    }
+    // the barriers, while the loads are on their way (the merge warp's lane)
+    if (tid == kThr - 32) {
+      for (int s = 0; s < NS; ++s) {
+        mbar_init(&full[s], 1);
+        mbar_init(&empty[s], kCW);
+      }
+      for (int s = 0; s < 2; ++s) {
+        mbar_init(&epi_full[s], kCW);
+        mbar_init(&epi_free[s], 1);
+      }
+      mbar_init(&ep_bar, 32);
+      mbar_init(&oth_bar, 32);
+      mbar_init(&own_bar, 32);
+      fence_barrier_init();
+      s_abort = 0;
+      s_bad = 0;
+      s_mg_h = -1;
+    }
+    if (h < nheads) {
+      const int e = verify(l, o, cp, lab, nb);
+      tab.vlen[tid] = l + kNew;
+      tab.off[tid] = o;
+      tab.bad[tid] = (unsigned char)e;
+      if (FUSED) {
+        tab.ntok[tid] = nt;
+        tab.label[tid] = (unsigned char)lab;
+      }
+      if (in_regs) {
+        const int g = S::grains(l + kNew);
+        const int st = e ? e : g > kMost ? (int)HKV_ERR_BOUNDS : 0;
+        key = st ? kIsBad + st : g;
+        c0 = st ? 0u : (unsigned)S::cost(g);
+      }
+    }
+  }
+  // the slots of a head of length l of row i (a bad one: 0, and the status)
+  auto slots = [&](int h, int l) {
+    if (h >= nheads) return 0u;
+    const int g = S::grains(l + kNew);
+    const bool ok = FUSED ? l >= 0 && g <= kMost : g <= kMost && !verify(l, p.off[h], 0, 0, 0);
+    if (!ok) key = kIsBad + HKV_ERR_BOUNDS;
+    return ok ? (unsigned)S::cost(g) : 0u;
+  };
+  unsigned rowsum = 0;  // lane i: the slots of row i (up to 32 rows)
+  long long wsum = 0;
   if (in_regs) {
-    if (h_lo < h_hi) {  // every load issued before any use
-      rl = p.len[h_lo];
-      ro = p.off[h_lo];
-      rcp = p.cap[h_lo];
-      rlb = p.label[p.layer_base + h_lo];
-      rnb = p.nbuf[p.layer_base + h_lo];
-      count(rl);
-    }
+    rowsum = __reduce_add_sync(0xFFFFFFFFu, c0);
+    wsum = rowsum;
   } else {
-    const int guess = (int)((float)bx * ((float)nheads / (float)G));
-    win_lo = guess - kThr / 2;
-    win_lo = win_lo < nheads - kThr ? win_lo : nheads - kThr;
-    win_lo = win_lo > 0 ? win_lo : 0;
-    const int wh = win_lo + tid;
-    if (wh < nheads) {
-      ro = p.off[wh];
-      rcp = p.cap[wh];
-      rlb = p.label[p.layer_base + wh];
-      rnb = p.nbuf[p.layer_base + wh];
+#pragma unroll
+    for (int i = 0; i < kPre; ++i) {
+      if (i < rows) {
+        const unsigned r = __reduce_add_sync(0xFFFFFFFFu, slots((row0 + i) * 32 + lane, lv[i]));
+        if (lane == i) rowsum = r;
+        wsum += r;
+      }
     }
-#pragma unroll 4
-    for (int h = h_lo; h < h_hi; ++h) count(p.len[h]);
+#pragma unroll 1
+    for (int i = kPre; i < rows; ++i) {
+      const int h = (row0 + i) * 32 + lane;
+      const unsigned r = __reduce_add_sync(0xFFFFFFFFu, slots(h, h < nheads ? p.len[h] : 0));
+      if (lane == i) rowsum = r;
+      wsum += r;
+    }
   }
-  long long total;
-  const long long slice_start = block_excl_scan<long long>(mine, scan_scratch, &total);
-  if (tid == 0) STEP_TRACE(10);
-  if (bad) s_bad = bad;
-  if (tid == 0) {  // this CTA's range (a 64-bit division: one thread)
-    Ranges<TT> r0;
-    r0.total = total;
-    r0.G = G;
-    r0.chunk = Ranges<TT>::chunk_of(total, G, S::kMinChunk);
-    s_chunk = r0.chunk;
-    s_a = r0.start(bx);
-    s_b = r0.start(bx + 1);
-  }
+  if (wsum > kMost) key = kIsBad + HKV_ERR_BOUNDS;
+  key = __reduce_max_sync(0xFFFFFFFFu, key);
+  if (lane == 0) s_w[warp] = make_int2((int)wsum, key);
   __syncthreads();
-  Ranges<TT> rg;
-  rg.total = total;
-  rg.G = G;
-  rg.chunk = s_chunk;
-  if (s_bad) {  // every CTA sees it: none reads further or arrives
+  if (tid == 0) STEP_TRACE(10);
+  const int2 sw = lane < NW ? s_w[lane] : make_int2(0, 0);
+  const int total = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)sw.x);
+  const int longest = __reduce_max_sync(0xFFFFFFFFu, sw.y);
+  if (longest >= kIsBad) {  // every CTA sees it: none reads further or arrives
     pdl_wait();
-    if (bx == 0 && tid == 0) set_err(p.err, (uint32_t)s_bad);
+    if (bx == 0 && tid == 0) {
+      set_err(p.err, (uint32_t)(longest - kIsBad));
+      p.ctl->valid = 0;
+    }
     return;
   }
-  const long long a = s_a, b = s_b;
-  bool active = a < total;
-  if (active && mine > 0) {  // the heads holding the range's first and last index
-    const bool has_a = slice_start <= a && a < slice_start + mine;
-    const bool has_b = slice_start <= b - 1 && b - 1 < slice_start + mine;
-    if (has_a || has_b) {
-      long long st = slice_start;
-      auto visit = [&](int h, int l) {
-        const long long L = slot_len<TT>(l + 1);
-        if (has_a && a >= st && a < st + L) {
-          s_h0 = h;
-          s_s0 = st;
-        }
-        if (has_b && b - 1 >= st && b - 1 < st + L) s_h1 = h;
-        st += L;
+  // a CTA per head where every head is short (see kAlignedGrains), else G
+  // ranges of `chunk` slots
+  const bool aligned = in_regs && nheads <= G && longest <= kAlignedGrains;
+  // total / G rounded up, from the grid's reciprocal (rounded up, so the
+  // quotient is exact or one too large)
+  int chunk = G == 1 ? total : (int)__umulhi((unsigned)(total + G - 1), p.grid_recip);
+  if ((long long)chunk * G > total + G - 1) --chunk;
+  if (chunk < S::kMinChunk) chunk = S::kMinChunk;
+  const int tol = chunk / HKV_STEP_SNAP_DIV;
+  const long long a64 = (long long)bx * chunk, b64 = a64 + chunk;
+  const int a_raw = a64 < total ? (int)a64 : total, b_raw = b64 < total ? (int)b64 : total;
+  bool active = aligned ? bx < nheads : a_raw < total;
+  // boundary x inside the slots [s, s + cost) of a head of g grains
+  auto snap = [&](int x, int s, int g) {
+    if (x - s <= tol) return s;
+    return x >= s + g - tol ? s + S::cost(g) : x;
+  };
+  // places head h (slots from s, v rows): whether it is in the range, and
+  // the range's ends when they fall into it
+  auto place = [&](int h, int s, int v) {
+    const int g = S::grains(v), e = s + S::cost(g);
+    if (a_raw >= e || b_raw <= s) return false;
+    bool in = true;
+    if (a_raw >= s) {
+      const int x = snap(a_raw, s, g);
+      const bool next = x == e;
+      s_lo = make_int4(x, next ? h + 1 : h, next ? e : s, v);
+      in = !next;
+    }
+    if (b_raw <= e) {
+      const int x = b_raw == e ? e : snap(b_raw, s, g);
+      s_hi = make_int4(x, x == s ? h - 1 : h, s, x > s && x < e);
+      in = in && x != s;
+    }
+    return in;
+  };
+  if (!aligned && active) {
+    const int before = (int)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? (unsigned)sw.x : 0u);
+    if (before < b_raw && before + (int)wsum > a_raw) {  // warp-uniform
+      // one row: its heads in order
+      auto place_row = [&](int i, int at) {
+        const int h = (row0 + i) * 32 + lane;
+        const bool in = h < nheads;
+        const int j = h - wl;
+        const bool here = j >= 0 && j < kThr;
+        const int v = !in ? 0 : here ? tab.vlen[j] : p.len[h] + kNew;
+        const int c = in ? S::cost(S::grains(v)) : 0;
+        const int incl = warp_incl_scan(c);
+        if (in && place(h, at + incl - c, v) && FUSED && !in_regs && here && tab.bad[j])
+          atomicMax(&s_bad, (int)tab.bad[j]);
+        return __shfl_sync(0xFFFFFFFFu, incl, 31);
       };
       if (in_regs) {
-        visit(h_lo, rl);
-      } else {
-        for (int h = h_lo; h < h_hi; ++h) visit(h, p.len[h]);
-      }
-    }
-  }
-  __syncthreads();
-  if (tid == 0) STEP_TRACE(11);
-  int n = active ? s_h1 - s_h0 + 1 : 0;
-  int own_bad = 0;
-  if (n > kStepTable) {  // excluded by the host; the step is not taken
-    own_bad = HKV_ERR_CAPACITY;
-    n = 0;
-    active = false;
-  }
-  const int h0 = s_h0;
-  // the table entry of head h with its checks
-  auto enter = [&](int h, long long st, int l, long long o, int cp, int lab, int nb) {
-    const int j = h - h0;
-    int e = 0;
-    if (o < 0 || o + cp > p.arena_tokens) e = HKV_ERR_BOUNDS;
-    else if (l + 1 > cp) e = HKV_ERR_CAPACITY;
-    else if (lab != HKV_DENSE && nb >= p.period) e = HKV_ERR_STATE;  // the update is due first
-    if (e) atomicMax(&s_bad, e);
-    if (st >= 0) {
-      tab.start[j] = st;
-      tab.vlen[j] = l + 1;
-    }
-    tab.off[j] = o;
-    tab.nbuf[j] = nb;
-    tab.label[j] = (unsigned char)lab;
-  };
-  if (in_regs) {  // the slice owner enters its head
-    if (active && h_lo < h_hi && h_lo >= h0 && h_lo < h0 + n)
-      enter(h_lo, slice_start, rl, ro, rcp, rlb, rnb);
-  } else {
-    // the slice owners place the range's heads in the index space ...
-    if (active && h_lo <= h0 + n - 1 && h_hi > h0) {
-      long long st = slice_start;
-      for (int h = h_lo; h < h_hi && h < h0 + n; ++h) {
-        const int l = p.len[h];
-        if (h >= h0) {
-          tab.start[h - h0] = st;
-          tab.vlen[h - h0] = l + 1;
+        place_row(0, before);
+      } else if (rows <= 32) {
+        const int incl = warp_incl_scan((int)rowsum);
+        const int rs = before + incl - (int)rowsum;
+        unsigned hit = __ballot_sync(0xFFFFFFFFu, lane < rows && rs < b_raw && before + incl > a_raw);
+        while (hit) {
+          const int i = __ffs(hit) - 1;
+          hit &= hit - 1;
+          place_row(i, __shfl_sync(0xFFFFFFFFu, rs, i));
         }
-        st += slot_len<TT>(l + 1);
+      } else {
+        int at = before;
+#pragma unroll 1
+        for (int i = 0; i < rows && at < b_raw; ++i) at += place_row(i, at);
       }
     }
-    // ... and a thread per head checks the rest: from registers when the
-    // window holds the whole range, else from one more round of loads
-    const bool in_win = h0 >= win_lo && h0 + n <= win_lo + kThr;
-    const int jt = in_win ? win_lo + tid - h0 : tid;
-    if (active && jt >= 0 && jt < n) {
-      const int h = h0 + jt, i = p.layer_base + h;
-      if (in_win)
-        enter(h, -1, p.len[h], ro, rcp, rlb, rnb);
-      else
-        enter(h, -1, p.len[h], p.off[h], p.cap[h], p.label[i], p.nbuf[i]);
-    }
-  }
-  if (tid == 0) {
-    tab.h0 = h0;
-    tab.n = n;
   }
   __syncthreads();
-  if (s_bad) {  // a bad head in this range: stream nothing
-    own_bad = own_bad > s_bad ? own_bad : s_bad;
-    active = false;
+  int a = 0, b = 0, h0 = bx, n = 1, s0 = 0, s1 = 0, v0 = 0;
+  bool has_s = false, has_e = false;
+  if (!aligned && active) {
+    const int4 lo = s_lo, hi = s_hi;
+    a = lo.x;
+    b = hi.x;
+    h0 = lo.y;
+    n = hi.y - lo.y + 1;
+    s0 = lo.z;
+    v0 = lo.w;
+    s1 = hi.z;
+    active = a < b && n > 0;
+    has_s = active && s0 < a;
+    has_e = active && hi.w;
   }
+  const int h1 = h0 + n - 1;
+  int own_bad = 0;
+  if (!in_regs) {
+    if (FUSED && active && n > kStepTable) {  // excluded by the host; the step is not taken
+      own_bad = HKV_ERR_CAPACITY;
+      active = false;
+    }
+    if (active && (h0 < wl || h0 + n > wl + kThr)) {  // CTA-uniform
+      wl = h0;
+      const int h = h0 + tid, i = p.layer_base + h;
+      if (tid < n) {
+        const int l = p.len[h];
+        const long long o = p.off[h];
+        tab.vlen[tid] = l + kNew;
+        tab.off[tid] = o;
+        if (FUSED) {
+          const int cp = p.cap[h], lab = p.label[i], nb = p.nbuf[i], nt = p.ntok[i];
+          const int e = verify(l, o, cp, lab, nb);
+          if (e) atomicMax(&s_bad, e);
+          tab.ntok[tid] = nt;
+          tab.label[tid] = (unsigned char)lab;
+        }
+      }
+      __syncthreads();
+    }
+    if (FUSED && s_bad) {  // a bad head in this range: stream nothing
+      own_bad = own_bad > s_bad ? own_bad : s_bad;
+      active = false;
+    }
+  }
+  if (!active) has_s = has_e = false;
   // From here on nothing reads the layer's counters in global memory: the
-  // merge warp arrives on the layer's barrier word below.
+  // merge warp arrives on the layer's barrier word below. (Attention alone
+  // over more heads than the table holds looks them up; nothing writes them.)
   if (tid == 0) STEP_TRACE(1);
 
-  // ---- the range's sub-ranges, in streaming order --------------------------
-  // S: the piece of the head that began before a; E: the start of the head
-  // that continues past b; M: the heads in between.
-  long long sub_g[3], sub_b[3];
-  int sub_j[3], nsub = 0;
-  if (active) {
-    const long long hs0 = tab.start[0];
-    const long long se0 = hs0 + slot_len<TT>(tab.vlen[0]);
-    const long long hs1 = tab.start[n - 1];
-    const long long he1 = hs1 + tab.vlen[n - 1];
-    const bool has_s = hs0 < a;
-    const bool has_e = he1 > b && (n > 1 || !has_s);
-    const long long s_end = se0 < b ? se0 : b;
-    const long long e_beg = hs1 > a ? hs1 : a;
-    if (has_e) {
-      sub_g[nsub] = e_beg, sub_b[nsub] = b, sub_j[nsub] = n - 1;
-      ++nsub;
-    }
-    if (has_s) {
-      sub_g[nsub] = a, sub_b[nsub] = s_end, sub_j[nsub] = 0;
-      ++nsub;
-    }
-    const long long m_lo = has_s ? s_end : a, m_hi = has_e ? e_beg : b;
-    if (m_lo < m_hi) {
-      sub_g[nsub] = m_lo, sub_b[nsub] = m_hi, sub_j[nsub] = has_s ? 1 : 0;
-      ++nsub;
-    }
-  }
-
-  if (tid == 0) STEP_TRACE(12);
-
   // ---- producer state (warp 0, lane 0) ------------------------------------
+  // Pieces in streaming order: the start of the head that continues past the
+  // range, the piece of the head that began before it, the heads in between.
   const bool producer = tid == 0;
-  StepIter<TT> pit;
-  int sr = 0;  // current sub-range
-  auto start_sub = [&](int r) {
-    pit.j = sub_j[r];
-    pit.hs = tab.start[pit.j];
-    pit.hl = tab.vlen[pit.j];
-    pit.g = sub_g[r];
-    pit.b = sub_b[r];
+  const bool in_tab = FUSED || n <= kThr;
+  auto vlen_of = [&](int h) { return in_tab ? tab.vlen[h - wl] : p.len[h] + kNew; };
+  auto off_of = [&](int h) { return in_tab ? tab.off[h - wl] : (long long)p.off[h]; };
+  int ph = 0, ch = h0 + (has_s ? 1 : 0);    // next piece; next whole head
+  const int ch_end = has_e ? h1 - 1 : h1;   // last whole head
+  int ph_h = 0, ph_r = 0, ph_end = 0, ph_v = 0, ph_flags = 0;  // the piece: head, rows, length
+  long long ph_off = 0;
+  bool have = false, at_start = false;
+  auto open_piece = [&](int h, int from, long long to, int flags) {
+    ph_h = h;
+    ph_v = vlen_of(h);
+    ph_off = off_of(h);
+    ph_r = from;
+    ph_end = to < ph_v ? (int)to : ph_v;
+    ph_flags = flags;
+    at_start = true;
+    have = true;
   };
-  pit.g = pit.b = 0;
-  pit.j = 0;
-  pit.hs = 0;
-  pit.hl = 0;
-  if (nsub > 0) start_sub(0);
-  auto more = [&]() {  // moves to the next sub-range when one is exhausted
-    while (pit.done() && sr + 1 < nsub) start_sub(++sr);
-    return !pit.done();
+  auto next_piece = [&]() {
+    have = false;
+    if (ph == 0) {
+      ph = 1;
+      if (has_e && !(has_s && n == 1)) {
+        open_piece(h1, 0, (long long)(b - s1) * GR, 0);
+        return;
+      }
+    }
+    if (ph == 1) {
+      ph = 2;
+      if (has_s) {
+        open_piece(h0, (a - s0) * GR, (long long)(b - s0) * GR, kTailPiece);
+        return;
+      }
+    }
+    if (active && ch <= ch_end) {
+      open_piece(ch, 0, 0x7FFFFFFF, kWhole);
+      ++ch;
+    }
   };
-  int issued = 0;
+  int st_i = 0;                // stage of the next tile
+  uint32_t st_ph = 1;          // its empty barrier's parity (1: not used yet)
   // the arena rows are read once per step: evict them from L2 first (measured:
   // 0.4-0.55 us per step slower without the hint)
   const uint64_t stream_pol = producer ? l2_evict_first_policy() : 0;
-  struct Pending {
-    int h, slot_new;
-    bool first, has_new;
-  };
-  auto issue_old = [&](Pending &pd) {  // describe, expect and copy the arena rows
-    const int stage = issued % NS;
-    const long long ge = pit.tile_end();
-    const long long he = pit.hs + pit.hl;
-    const int r0 = (int)(pit.g - pit.hs), r1 = (int)(ge - pit.hs);
-    const int real = pit.hl - 1;  // rows in the arena
-    const int n_old = (r1 < real ? r1 : real) - r0;
+  auto issue_old = [&](int stage) {  // describe, expect and copy the arena rows
+    const int left = ph_end - ph_r;
+    const int rows = left < TT ? left : TT;
+    const int real = ph_v - kNew;  // rows in the arena
+    const int n_old = (ph_r + rows < real ? ph_r + rows : real) - ph_r;
     unsigned char *dk = stages + stage * S::kStageBytes;
-    const int h = h0 + pit.j;
-    pd.h = h;
-    pd.slot_new = real - r0;
-    pd.first = pit.g == pit.hs || pit.g == sub_g[sr];
-    pd.has_new = r1 == pit.hl;
-    TileMeta &mt = meta[stage];
-    mt.h = h;
-    mt.n = (int)(ge - pit.g);
-    mt.flags = (pd.first ? kFirst : 0) | (ge == (pit.b < he ? pit.b : he) ? kLast : 0);
-    mt.hs = pit.hs;
-    mt.he = he;
     if (n_old > 0) {
       const uint32_t bytes = (uint32_t)n_old * RB;
-      const long long row = tab.off[pit.j] + r0;
+      const long long row = ph_off + ph_r;
       mbar_expect_tx(&full[stage], 2 * bytes);
       bulk_g2s_hint(dk, static_cast<const unsigned char *>(p.K) + row * RB, bytes, &full[stage],
                     stream_pol);
       bulk_g2s_hint(dk + TT * RB, static_cast<const unsigned char *>(p.V) + row * RB, bytes,
                     &full[stage], stream_pol);
     }
-    pit.advance(tab);
-    ++issued;
+    const bool last = left <= TT;
+    TileMeta mt;
+    mt.h = ph_h;
+    mt.n = rows;
+    mt.flags = ph_flags | (at_start ? kFirst : 0) | (last ? kLast : 0) |
+               (FUSED && ph_r + rows == ph_v ? kNewRow : 0);
+    const int rc = ph_v - (p.w_loc - 1) - ph_r;
+    mt.recent0 = IDENT ? (rc < 0 ? 0 : rc < TT ? rc : TT) : 0;
+    meta[stage] = mt;
+    at_start = false;
+    ph_r += TT;
+    if (last) next_piece();
   };
-  auto issue_extra = [&](const Pending &pd, int stage) {  // the step's inputs, then arrive
+  auto issue_extra = [&](int stage) {  // the step's inputs, then arrive
     unsigned char *dk = stages + stage * S::kStageBytes;
     unsigned char *dv = dk + TT * RB;
-    mbar_arrive_expect_tx(&full[stage], (pd.has_new ? 2 * RB : 0) + (pd.first ? RB : 0));
-    if (pd.has_new) {
-      bulk_g2s(dk + pd.slot_new * RB,
-               static_cast<const unsigned char *>(p.k_new) + (size_t)pd.h * RB, RB, &full[stage]);
-      bulk_g2s(dv + pd.slot_new * RB,
-               static_cast<const unsigned char *>(p.v_new) + (size_t)pd.h * RB, RB, &full[stage]);
+    const int h = meta[stage].h, flags = meta[stage].flags;
+    const size_t src = (size_t)h * RB;
+    mbar_arrive_expect_tx(&full[stage], (flags & kNewRow ? 2 * RB : 0) + (flags & kFirst ? RB : 0));
+    if (flags & kFirst)
+      bulk_g2s(dv + TT * RB, static_cast<const unsigned char *>(p.q) + src, RB, &full[stage]);
+    if (flags & kNewRow) {
+      const int at = (meta[stage].n - 1) * RB;
+      bulk_g2s(dk + at, static_cast<const unsigned char *>(p.k_new) + src, RB, &full[stage]);
+      bulk_g2s(dv + at, static_cast<const unsigned char *>(p.v_new) + src, RB, &full[stage]);
     }
-    if (pd.first)
-      bulk_g2s(dv + TT * RB, static_cast<const unsigned char *>(p.q) + (size_t)pd.h * RB, RB,
-               &full[stage]);
   };
-  Pending pre[NS];
   int n_pre = 0;
-  if (producer)
-    for (; n_pre < (p.prefetch ? S::kPre : NS) && more(); ++n_pre) issue_old(pre[n_pre]);
+  if (producer) {
+    next_piece();
+    const int lim = p.prefetch ? S::kPre : NS;
+#pragma unroll 1
+    while (n_pre < lim && have) issue_old(n_pre++);
+  }
   if (tid == 0) STEP_TRACE(7);
+
+  // ---- merge warp: the launch's epoch and the split head this CTA combines --
+  // The split head: the first of the range when this CTA is that head's
+  // first middle CTA (its whole range inside the head) or, for a head in two
+  // pieces, holds its last row. The epoch is unique per (layer, launch of
+  // that layer), from the generation of the layer's barrier word; the
+  // epilogue waits for both only when it meets a split head.
+  //
+  // Then this CTA arrives on the layer's barrier words {arrivals,
+  // generation, worst status}: it is done reading counters. The last of the
+  // grid to arrive resets the count and publishes the next generation, which
+  // the others watch. A CTA with a bad head arrives after the wait for the
+  // previous kernel, raises the worst status and adds 1 << 16 more; the last
+  // arriver then marks the generation (the step is not taken) and reports
+  // the worst status, the same whichever CTAs found bad heads first. The
+  // words belong to this layer, whose previous launch is complete, so the
+  // others arrive ahead of that wait.
+  constexpr uint32_t kBadStep = 0x80000000u;  // in the generation: step not taken
+  uint32_t gen0 = 0, gen1 = 0;
+  int bar_done = 0;
+  auto arrive = [&]() {  // lane 0 of the merge warp
+    const uint32_t inc = own_bad ? 0x10001u : 1u;
+    if (own_bad) {
+      atomicMax(p.bar + 2, (uint32_t)own_bad);
+      __threadfence();  // the status before the arrival
+    }
+    const uint32_t old = atomicAdd(p.bar, inc);
+    if ((old & 0xFFFFu) == (uint32_t)G - 1) {
+      const bool bad_step = ((old + inc) >> 16) != 0;
+      if (bad_step) {
+        __threadfence();  // the bad CTAs' statuses after their arrivals
+        set_err(p.err, atomicExch(p.bar + 2, 0u));
+      }
+      p.bar[0] = 0;
+      gen1 = (((gen0 & ~kBadStep) + 1u) & ~kBadStep) | (bad_step ? kBadStep : 0u);
+      st_release(p.bar + 1, gen1);
+      bar_done = 1;
+    }
+  };
+  if (warp == kCW + 2) {
+    if (lane == 0) {
+      if (has_s) {
+        const int er = s0 + S::grains(v0);
+        int k0 = (int)((unsigned)s0 / (unsigned)chunk);
+        if ((long long)(k0 + 1) * chunk - s0 <= tol) ++k0;  // that boundary moved to the head's start
+        int k1 = (int)((unsigned)(er - 1) / (unsigned)chunk);
+        const long long x1 = (long long)k1 * chunk;
+        if (x1 > s0 && x1 >= er - tol) --k1;  // that one to its end
+        const int np = k1 - k0 + 1;
+        if ((np >= 3 ? k0 + 1 : k1) == bx) {
+          s_mg_k0 = k0;
+          s_mg_np = np;
+          s_mg_j = bx - k0;
+          s_mg_h = h0;
+        }
+      }
+      gen0 = ld_acquire(p.bar + 1);
+      s_ep = ((gen0 & ~kBadStep) + 1u) * (uint32_t)p.n_layers + (uint32_t)p.layer;
+      if (!own_bad) arrive();
+    }
+    __syncwarp();
+    mbar_arrive(&ep_bar);  // all 32 lanes: the epilogue may read s_ep, s_mg_*
+  }
 
   if (p.prefetch) pdl_wait();  // the step's inputs are visible from here on
   if (tid == 0) STEP_TRACE(2);
@@ -585,37 +757,35 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     // ---- producer ----------------------------------------------------------
     if (producer) {
       long long w_empty = 0;  // cycles waiting for free stages (tracer)
-      int armed = 0;  // stages whose producer arrival is done (issued order)
-#pragma unroll
-      for (int j = 0; j < NS; ++j)
-        if (j < n_pre) issue_extra(pre[j], j);
-      armed = n_pre;
-      while (more()) {
-        const int stage = issued % NS;
+#pragma unroll 1
+      for (int j = 0; j < n_pre; ++j) issue_extra(j);
+      st_i = n_pre < NS ? n_pre : 0;
+      st_ph = n_pre < NS ? 1u : 0u;
+      int armed = n_pre;  // tiles armed in all
+      auto stage_free = [&]() {  // (the parity of a stage not used yet reads as complete)
+        if (!s_abort && mbar_wait(&empty[st_i], st_ph)) return true;
+        s_abort = 1;
+        set_err(p.err, HKV_ERR_TIMEOUT);
+        return false;
+      };
+      while (have) {
         const long long c0 = STEP_CLK();
-        if (s_abort ||
-            (issued >= NS && !mbar_wait(&empty[stage], (uint32_t)(issued / NS - 1) & 1u))) {
-          s_abort = 1;
-          set_err(p.err, HKV_ERR_TIMEOUT);
-          break;
-        }
+        if (!stage_free()) break;
         w_empty += STEP_CLK() - c0;
-        Pending pd;
-        issue_old(pd);
-        issue_extra(pd, stage);
-        armed = issued;
-      }
-      if (!s_abort) {  // no more tiles: a closing record for the consumers
-        const int stage = issued % NS;
-        if (issued >= NS && !mbar_wait(&empty[stage], (uint32_t)(issued / NS - 1) & 1u)) {
-          s_abort = 1;
-          set_err(p.err, HKV_ERR_TIMEOUT);
-        } else {
-          meta[stage].flags = kDone;
-          mbar_arrive(&full[stage]);
+        issue_old(st_i);
+        issue_extra(st_i);
+        ++armed;
+        if (++st_i == NS) {
+          st_i = 0;
+          st_ph ^= 1u;
         }
+      }
+      if (stage_free()) {  // no more tiles: a closing record for the consumers
+        meta[st_i].flags = kDone;
+        mbar_arrive(&full[st_i]);
       }
       STEP_TRACE_SET(20, w_empty);
+      if (!FUSED && bx == 0) p.ctl->valid = 1;  // the launch passed its checks
       if (s_abort) {
         // No bulk copy may land in shared memory after the CTA exits: wait
         // (bounded) for every armed stage that may still be in flight. A
@@ -626,20 +796,20 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     }
   } else if (warp <= kCW) {
     // ---- consumers ---------------------------------------------------------
-    const int ctid = tid - 32, cw = warp - 1;
+    const int cw = warp - 1;
     const int grp = lane / LPR, col = lane % LPR;
     using M = LaneMath<T>;
     static_assert(M::kEPL == EPL, "lane mapping");
-    typename M::Q q;
+    constexpr bool MMA = sizeof(T) == 2;
     float2 acc[EPL / 2];
-    float m = -INFINITY, l = 0.f;
+    float m = -INFINITY, l = 0.f, lr = 0.f;  // lr: identification's newest-row mass
     int nseg = 0;
 #pragma unroll
     for (int e = 0; e < EPL / 2; ++e) acc[e] = make_float2(0.f, 0.f);
     int n_tiles = 0;
     long long w_full = 0, w_hand = 0;  // cycles waiting for tiles, for the epilogue (tracer)
     // hands one segment's state (or the closing record) to the epilogue
-    auto hand_over = [&](const SegMeta *sm) {
+    auto hand_over = [&](int h, int flags) {
       const int bb = nseg & 1;
       const long long c0 = STEP_CLK();
       if (nseg >= 2 && !s_abort &&
@@ -648,94 +818,211 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         set_err(p.err, HKV_ERR_TIMEOUT);
       }
       w_hand += STEP_CLK() - c0;
-      if (sm) {
+      if (h >= 0 && MMA) {
+        // The row groups share the maximum; their sums are halved between
+        // the lanes of two groups at a time, so that each lane ends with its
+        // own channels. l and lr are split over the quads.
+        float *dst = &red_acc[bb][cw][col * EPL];
+        float2 x0 = acc[0], x1 = acc[1];
+        {
+          const bool hi = lane & 16;
+          const float2 s0v = hi ? acc[0] : acc[2], s1v = hi ? acc[1] : acc[3];
+          x0 = hi ? acc[2] : acc[0];
+          x1 = hi ? acc[3] : acc[1];
+          x0.x += __shfl_xor_sync(0xFFFFFFFFu, s0v.x, 16);
+          x0.y += __shfl_xor_sync(0xFFFFFFFFu, s0v.y, 16);
+          x1.x += __shfl_xor_sync(0xFFFFFFFFu, s1v.x, 16);
+          x1.y += __shfl_xor_sync(0xFFFFFFFFu, s1v.y, 16);
+        }
+        if (RPW == 2) {
+          *reinterpret_cast<float4 *>(dst + (lane & 16 ? 4 : 0)) = make_float4(x0.x, x0.y, x1.x, x1.y);
+        } else {
+          const bool hi = lane & 8;
+          const float2 sv = hi ? x0 : x1;
+          float2 x = hi ? x1 : x0;
+          x.x += __shfl_xor_sync(0xFFFFFFFFu, sv.x, 8);
+          x.y += __shfl_xor_sync(0xFFFFFFFFu, sv.y, 8);
+          *reinterpret_cast<float2 *>(dst + (lane & 16 ? 4 : 0) + (hi ? 2 : 0)) = x;
+        }
+        float ls = l, rs = lr;
+#pragma unroll
+        for (int o = 4; o <= 16; o <<= 1) {
+          ls += __shfl_xor_sync(0xFFFFFFFFu, ls, o);
+          if (IDENT) rs += __shfl_xor_sync(0xFFFFFFFFu, rs, o);
+        }
+        if (lane == 0) {
+          red_m[bb][cw] = m;
+          red_l[bb][cw] = ls;
+          if (IDENT) red_r[bb][cw] = rs;
+        }
+      } else if (h >= 0) {
         const int si = cw * RPW + grp;
-        float2 *dst = reinterpret_cast<float2 *>(&red_acc[bb][si][col * EPL]);
+        float2 *dst = reinterpret_cast<float2 *>(&red_acc[bb][si % NST][col * EPL]);
 #pragma unroll
         for (int e = 0; e < EPL / 2; ++e) dst[e] = acc[e];
         if (col == 0) {
-          red_m[bb][si] = m;
-          red_l[bb][si] = l;
+          red_m[bb][si % NST] = m;
+          red_l[bb][si % NST] = l;
+          if (IDENT) red_r[bb][si % NST] = lr;
         }
-        if (cw == 0 && lane == 0) seg[bb] = *sm;
-      } else if (cw == 0 && lane == 0) {
-        seg[bb].h = -1;
+      }
+      if (cw == 0 && lane == 0) {
+        seg[bb].h = h;
+        seg[bb].flags = flags;
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&epi_full[bb]);
       ++nseg;
     };
-    for (int tile = 0;; ++tile) {
-      const int stage = tile % NS;
+    constexpr int NJ = MMA ? D / 32 : 1;          // 16-byte pieces of a row per lane
+    constexpr int NB = MMA ? TT / (kCW * 8) : 1;  // 8-row blocks per warp and tile
+    constexpr int VS = MMA ? 8 / RPW : 1;         // row steps of a block's V
+    static_assert(!MMA || TT % (kCW * 8) == 0, "blocks of 8 rows");
+    uint32_t qb[NJ][2];
+    typename M::Q q;
+    int stage = 0;
+    uint32_t fph = 0;  // parity of the stage's full barrier
+    for (;;) {
       const long long c0 = STEP_CLK();
-      if (!s_abort && !mbar_wait(&full[stage], (uint32_t)(tile / NS) & 1u)) {
+      if (!mbar_wait_unless(&full[stage], fph, &s_abort)) {
         s_abort = 1;
         set_err(p.err, HKV_ERR_TIMEOUT);
+        break;
       }
-      if (tile > 0) w_full += STEP_CLK() - c0;
-      if (s_abort) break;
-      const int flags = meta[stage].flags;
+      if (n_tiles > 0) w_full += STEP_CLK() - c0;
+      const TileMeta mt4 = meta[stage];
+      const int flags = mt4.flags;
       if (flags & kDone) break;
-      if (tile == 0 && ctid == 0) STEP_TRACE(3);
+      if (n_tiles == 0 && tid == 32) STEP_TRACE(3);
       ++n_tiles;
-      const int nr = meta[stage].n;
+      const int nr = mt4.n;
       const unsigned char *Ks = stages + stage * S::kStageBytes;
       const unsigned char *Vs = Ks + TT * RB;
       if (flags & kFirst) {  // first tile of this head in this piece
-        M::load_q(q, *reinterpret_cast<const uint4 *>(Vs + TT * RB + col * 16), p.qscale);
+        if constexpr (MMA) {
+#pragma unroll
+          for (int j = 0; j < NJ; ++j) {
+            const uint4 u = *reinterpret_cast<const uint4 *>(Vs + TT * RB + ((lane & 3) + 4 * j) * 16);
+            qb[j][0] = lane & 4 ? u.y : u.x;
+            qb[j][1] = lane & 4 ? u.w : u.z;
+          }
+        } else {
+          M::load_q(q, *reinterpret_cast<const uint4 *>(Vs + TT * RB + col * 16), p.qscale);
+        }
 #pragma unroll
         for (int e = 0; e < EPL / 2; ++e) acc[e] = make_float2(0.f, 0.f);
         m = -INFINITY;
         l = 0.f;
+        lr = 0.f;
       }
-      float sc[S::kSteps];
+      if constexpr (MMA) {
+        if (cw * 8 < nr) {  // the warp has rows in this tile
+          // q.k of 8 rows on the tensor cores. Lane (g, t) = (lane / 4,
+          // lane % 4) reads pieces t + 4j of row g, four registers x y z w of
+          // two channels each, and passes them as the A fragment as they
+          // are: x and z are then row g of A (k 0..7 and 8..15), y and w row
+          // g + 8. The even columns of B hold the query's channels of x and
+          // z, the odd ones those of y and w, so the row's dot product is
+          // C[g][even] + C[g + 8][odd]: c[0] + c[3] in all lanes of quad g.
+          uint4 vf[NB][VS];
+          float dots[NB];
+          float mt = -INFINITY;
 #pragma unroll
-      for (int st = 0; st < S::kSteps; ++st) {
-        const int r = st * (kCW * RPW) + cw * RPW + grp;
-        float dot = 0.f;
-        if (r < nr) dot = M::dot(q, *reinterpret_cast<const uint4 *>(Ks + r * RB + col * 16));
+          for (int b8 = 0; b8 < NB; ++b8) {
+            const int rb = (b8 * kCW + cw) * 8;
+            dots[b8] = -INFINITY;
+            if (rb < nr) {  // warp-uniform
+              const unsigned char *kr = Ks + (rb + (lane >> 2)) * RB + (lane & 3) * 16;
+              uint4 kf[NJ];
 #pragma unroll
-        for (int o = LPR / 2; o >= 1; o >>= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, o);
-        sc[st] = r < nr ? M::score(dot, p.qscale) : -INFINITY;
-      }
-      float mt = sc[0];
+              for (int j = 0; j < NJ; ++j) kf[j] = *reinterpret_cast<const uint4 *>(kr + j * 64);
+              // V: whole rows by groups of lanes, RPW rows a step; rows past
+              // the tile's are not read (they may hold anything)
+              const unsigned char *vr = Vs + (rb + grp) * RB + col * 16;
 #pragma unroll
-      for (int st = 1; st < S::kSteps; ++st) mt = fmaxf(mt, sc[st]);
-      const float mn = fmaxf(m, mt);
-      if (mn != -INFINITY) {
-        const float corr = ex2_approx(m - mn);  // measured: 0.11 us per step less than exp2f
-        l *= corr;
+              for (int st = 0; st < VS; ++st)
+                vf[b8][st] = rb + st * RPW + grp < nr
+                                 ? *reinterpret_cast<const uint4 *>(vr + st * RPW * RB)
+                                 : make_uint4(0u, 0u, 0u, 0u);
+              float c[2][4] = {};
 #pragma unroll
-        for (int e = 0; e < EPL / 2; ++e) acc[e] = __fmul2_rn(acc[e], make_float2(corr, corr));
+              for (int j = 0; j < NJ; ++j) mma_bf16(c[j & 1], kf[j], qb[j][0], qb[j][1]);
+              if (rb + (lane >> 2) < nr) dots[b8] = (c[0][0] + c[1][0]) + (c[0][3] + c[1][3]);
+              mt = fmaxf(mt, dots[b8]);
+            }
+          }
+          const float mn = fmaxf(m, warp_max(mt) * p.qscale);
+          if (mn != -INFINITY) {  // warp-uniform
+            if (mn != m) {
+              const float corr = ex2_approx(m - mn);  // measured: 0.11 us per step less than exp2f
+              l *= corr;
+              if (IDENT) lr *= corr;
+#pragma unroll
+              for (int e = 0; e < EPL / 2; ++e) acc[e] = __fmul2_rn(acc[e], make_float2(corr, corr));
+              m = mn;
+            }
+#pragma unroll
+            for (int b8 = 0; b8 < NB; ++b8) {
+              const int rb = (b8 * kCW + cw) * 8;
+              if (rb < nr) {
+                // of row rb + lane / 4; one rounding of the exponent
+                const float pr = ex2_approx(fmaf(dots[b8], p.qscale, -mn));
+                l += pr;
+                if (IDENT && rb + (lane >> 2) >= mt4.recent0) lr += pr;
+#pragma unroll
+                for (int st = 0; st < VS; ++st)
+                  M::add_v(acc, vf[b8][st], __shfl_sync(0xFFFFFFFFu, pr, (st * RPW + grp) * 4));
+              }
+            }
+          }
+        }
+      } else {
+        float sc[S::kSteps];
 #pragma unroll
         for (int st = 0; st < S::kSteps; ++st) {
           const int r = st * (kCW * RPW) + cw * RPW + grp;
-          if (r < nr) {
-            const float pr = ex2_approx(sc[st] - mn);
-            l += pr;
-            M::add_v(acc, *reinterpret_cast<const uint4 *>(Vs + r * RB + col * 16), pr);
-          }
+          float dot = 0.f;
+          if (r < nr) dot = M::dot(q, *reinterpret_cast<const uint4 *>(Ks + r * RB + col * 16));
+#pragma unroll
+          for (int o = LPR / 2; o >= 1; o >>= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, o);
+          sc[st] = r < nr ? M::score(dot, p.qscale) : -INFINITY;
         }
-        m = mn;
+        float mt = sc[0];
+#pragma unroll
+        for (int st = 1; st < S::kSteps; ++st) mt = fmaxf(mt, sc[st]);
+        const float mn = fmaxf(m, mt);
+        if (mn != -INFINITY) {
+          const float corr = ex2_approx(m - mn);
+          l *= corr;
+          if (IDENT) lr *= corr;
+#pragma unroll
+          for (int e = 0; e < EPL / 2; ++e) acc[e] = __fmul2_rn(acc[e], make_float2(corr, corr));
+#pragma unroll
+          for (int st = 0; st < S::kSteps; ++st) {
+            const int r = st * (kCW * RPW) + cw * RPW + grp;
+            if (r < nr) {
+              const float pr = ex2_approx(sc[st] - mn);
+              l += pr;
+              if (IDENT && r >= mt4.recent0) lr += pr;
+              M::add_v(acc, *reinterpret_cast<const uint4 *>(Vs + r * RB + col * 16), pr);
+            }
+          }
+          m = mn;
+        }
       }
-      if (flags & kLast) {  // last tile of this head in this piece: hand it over
-        SegMeta sm;
-        sm.h = meta[stage].h;
-        sm.hs = meta[stage].hs;
-        sm.he = meta[stage].he;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[stage]);
-        hand_over(&sm);
-      } else {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[stage]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[stage]);
+      if (flags & kLast) hand_over(mt4.h, flags);  // last tile of this head in this piece
+      if (++stage == NS) {
+        stage = 0;
+        fph ^= 1u;
       }
     }
-    if (ctid == 0) STEP_TRACE(4);
-    if (ctid == 0) STEP_TRACE_SET(17, n_tiles);
-    hand_over(nullptr);  // nothing more
-    if (ctid == 0) STEP_TRACE_SET(21, w_full);
-    if (ctid == 0) STEP_TRACE_SET(22, w_hand);
+    if (tid == 32) STEP_TRACE(4);
+    if (tid == 32) STEP_TRACE_SET(17, n_tiles);
+    hand_over(-1, 0);  // nothing more
+    if (tid == 32) STEP_TRACE_SET(21, w_full);
+    if (tid == 32) STEP_TRACE_SET(22, w_hand);
   } else if (warp == kCW + 1) {
     // ---- epilogue: combine each segment's row-group states ----------------
     bool have_ep = false;  // the epoch and the merge head (merge warp)
@@ -753,7 +1040,6 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       const SegMeta sg = seg[bb];
       if (sg.h < 0) break;
       const int h = sg.h;
-      const long long hs = sg.hs, he = sg.he;
       // lane s < NST weighs state s
       const float ms = lane < NST ? red_m[bb][lane] : -INFINITY;
       float mx = ms;
@@ -761,8 +1047,12 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       for (int o = 16; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
       const float ws = ms == -INFINITY ? 0.f : exp2f(ms - mx);
       float L = lane < NST ? red_l[bb][lane] * ws : 0.f;
+      float LR = IDENT && lane < NST ? red_r[bb][lane] * ws : 0.f;
 #pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) L += __shfl_xor_sync(0xFFFFFFFFu, L, o);
+      for (int o = 16; o >= 1; o >>= 1) {
+        L += __shfl_xor_sync(0xFFFFFFFFu, L, o);
+        if (IDENT) LR += __shfl_xor_sync(0xFFFFFFFFu, LR, o);
+      }
       float A[CPL];
 #pragma unroll
       for (int c = 0; c < CPL; ++c) A[c] = 0.f;
@@ -776,7 +1066,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&epi_free[bb]);  // the consumers may reuse the buffer
-      const bool whole = hs >= a && he <= b;
+      const bool whole = sg.flags & kWhole;
       if (!whole && !have_ep) {
         if (!mbar_wait(&ep_bar, 0u)) {
           s_abort = 1;
@@ -786,9 +1076,15 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         have_ep = true;
       }
       if (whole) {  // the whole head is in this CTA's range
+        // (attention alone: a head without rows gives zeros)
+        const bool none = !FUSED && L == 0.f;
 #pragma unroll
-        for (int c = 0; c < CPL; ++c) A[c] /= L;
+        for (int c = 0; c < CPL; ++c) A[c] = none ? 0.f : A[c] / L;
         V::st(p.out + (size_t)h * D + CPL * lane, A);
+        // Sec. 4 Step 2: local iff the newest w_loc - 1 tokens hold a share
+        // tau of the attention
+        if (IDENT && lane == 0)
+          p.label_out[p.layer_base + h] = LR >= p.tau * L ? HKV_LOCAL : HKV_GLOBAL;
       } else if (h == s_mg_h) {  // this CTA combines the head
         // the other pieces already combined by the merge warp: finish here;
         // else hand this piece to the merge warp
@@ -796,28 +1092,32 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         ready = __shfl_sync(0xFFFFFFFFu, ready, 0);
         if (ready) {
           mbar_wait(&oth_bar, 0u);  // complete: every lane acquires oth_*
-          float A2[CPL];
+          float A2[CPL], Lt, Rt = 0.f;
           V::lds(&oth_acc[CPL * lane], A2);
-          combine_store<CPL>(mx, L, A, oth_ml[0], oth_ml[1], A2,
-                             p.out + (size_t)h * D + CPL * lane);
+          combine_store<CPL, IDENT>(mx, L, LR, A, oth_s[0], oth_s[1], IDENT ? oth_s[NV - 1] : 0.f,
+                                    A2, p.out + (size_t)h * D + CPL * lane, Lt, Rt);
+          if (IDENT && lane == 0)
+            p.label_out[p.layer_base + h] = Rt >= p.tau * Lt ? HKV_LOCAL : HKV_GLOBAL;
           STEP_TRACE_SET(18, globaltimer());
         } else {
           V::st(&own_acc[CPL * lane], A);
           if (lane == 0) {
-            own_ml[0] = mx;
-            own_ml[1] = L;
+            own_s[0] = mx;
+            own_s[1] = L;
+            if (IDENT) own_s[NV - 1] = LR;
           }
         }
         if (lane == 0) s_own_state = ready ? 1 : 2;
         __syncwarp();
         mbar_arrive(&own_bar);  // all 32 lanes
       } else {  // a piece for the combining CTA: epoch-tagged, no fence needed
-        unsigned long long *ps = p.pslot + ((size_t)bx * 2 + (hs < a ? 1 : 0)) * (D + 2);
+        unsigned long long *ps = p.pslot + ((size_t)bx * 2 + (sg.flags & kTailPiece ? 1 : 0)) * PS;
 #pragma unroll
         for (int c = 0; c < CPL; ++c) st_pair(ps + CPL * lane + c, A[c], s_ep);
         if (lane == 0) {
           st_pair(ps + D, mx, s_ep);
           st_pair(ps + D + 1, L, s_ep);
+          if (IDENT) st_pair(ps + D + 2, LR, s_ep);
         }
       }
     }
@@ -825,60 +1125,8 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     STEP_TRACE_SET(9, k);
     if (lane == 0) STEP_TRACE_SET(23, w_epi);
   } else {
-    // ---- merge warp: barrier, appends, counters, the combined split head ---
-    // The split head this CTA combines, if any: the head of its range's
-    // first index when this CTA is that head's first middle CTA (its whole
-    // range inside the head) or, for a head in two pieces, holds its last
-    // row. Then the launch's epoch, unique per (layer, launch of that
-    // layer), from the generation of the layer's barrier word; the epilogue
-    // waits for both only when it meets a split head.
-    constexpr uint32_t kBadStep = 0x80000000u;  // in the generation: step not taken
-    uint32_t gen0 = 0;
-    if (lane == 0) {
-      if (active && tab.start[0] < a) {
-        const long long hs0 = tab.start[0], he0 = hs0 + tab.vlen[0];
-        const long long k0 = rg.owner(hs0), k1 = rg.owner(he0 - 1);
-        const long long np = k1 - k0 + 1;
-        if ((np >= 3 ? k0 + 1 : k1) == bx) {
-          s_mg_k0 = k0;
-          s_mg_np = (int)np;
-          s_mg_j = (int)(bx - k0);
-          s_mg_h = h0;
-        }
-      }
-      gen0 = ld_acquire(p.bar + 1);
-      s_ep = ((gen0 & ~kBadStep) + 1u) * (uint32_t)p.n_layers + (uint32_t)(p.layer_base / nheads);
-    }
-    __syncwarp();
-    mbar_arrive(&ep_bar);  // all 32 lanes: the epilogue may read s_ep, s_mg_*
-    // Arrive on the layer's barrier words {arrivals, generation, worst
-    // status}: this CTA is done reading counters. The last of the grid to
-    // arrive resets the count and publishes the next generation, which the
-    // others watch. A CTA with a bad head raises the worst status and adds
-    // 1 << 16 more; the last arriver then marks the generation (the step is
-    // not taken) and reports the worst status, the same whichever CTAs found
-    // bad heads first.
-    const uint32_t inc = own_bad ? 0x10001u : 1u;
-    uint32_t gen1 = 0;
-    int bar_done = 0;
-    if (lane == 0) {
-      if (own_bad) {
-        atomicMax(p.bar + 2, (uint32_t)own_bad);
-        __threadfence();  // the status before the arrival
-      }
-      const uint32_t old = atomicAdd(p.bar, inc);
-      if ((old & 0xFFFFu) == (uint32_t)G - 1) {
-        const bool bad_step = ((old + inc) >> 16) != 0;
-        if (bad_step) {
-          __threadfence();  // the bad CTAs' statuses after their arrivals
-          set_err(p.err, atomicExch(p.bar + 2, 0u));
-        }
-        p.bar[0] = 0;
-        gen1 = (((gen0 & ~kBadStep) + 1u) & ~kBadStep) | (bad_step ? kBadStep : 0u);
-        st_release(p.bar + 1, gen1);
-        bar_done = 1;
-      }
-    }
+    // ---- merge warp: appends, counters, the combined split head -------------
+    if (lane == 0 && own_bad) arrive();
     gen0 = __shfl_sync(0xFFFFFFFFu, gen0, 0);
     bar_done = __shfl_sync(0xFFFFFFFFu, bar_done, 0);
     const uint64_t t0 = globaltimer();
@@ -894,49 +1142,34 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       // empty pieces in both of this CTA's slots, so that no combining CTA
       // waits for them (the step is not taken; the outputs are not defined)
       for (int sl = 0; sl < 2; ++sl) {
-        unsigned long long *ps = p.pslot + ((size_t)bx * 2 + sl) * (D + 2);
+        unsigned long long *ps = p.pslot + ((size_t)bx * 2 + sl) * PS;
         for (int c = lane; c < D; c += 32) st_pair(ps + c, 0.f, s_ep);
         if (lane == 0) {
           st_pair(ps + D, -INFINITY, s_ep);
           st_pair(ps + D + 1, 0.f, s_ep);
+          if (IDENT) st_pair(ps + D + 2, 0.f, s_ep);
         }
       }
     }
-
-    while (!s_abort && !bar_done) {
+    auto poll = [&]() {  // whether the whole grid has arrived
+      if (bar_done) return true;
       if (lane == 0) {
         gen1 = ld_acquire(p.bar + 1);
         bar_done = gen1 != gen0;
       }
       bar_done = __shfl_sync(0xFFFFFFFFu, bar_done, 0);
-      if (!bar_done && timed_out()) break;
-    }
-    gen1 = __shfl_sync(0xFFFFFFFFu, gen1, 0);
-    __syncwarp();
-    STEP_TRACE_SET(19, globaltimer());
-    const bool taken = !s_abort && bar_done && !(gen1 & kBadStep) && active;
-
-    // Appends: the CTA holding a head's last row writes the new token (K/V
-    // row at index len, its position, q into the ring of the periodic
-    // update), then advances that head's counters. Nothing in this launch
-    // reads them; they wait for the barrier only to learn whether the step
-    // is taken, which it is by then long before the consumers finish.
-    if (taken) {
-      for (int j0 = 0; j0 < n; j0 += 32) {  // ntok of 32 heads per round
-        const int j = j0 + lane;
-        if (j < n && tab.start[j] + tab.vlen[j] > a && tab.start[j] + tab.vlen[j] <= b)
-          tab.ntok[j] = p.ntok[p.layer_base + h0 + j];
-      }
-      __syncwarp();
+      return bar_done != 0;
+    };
+    // The heads whose last row is in the range (a range's first head always
+    // reaches past its start; only its last one can continue past its end).
+    const int napp = active ? (has_e ? n - 1 : n) : 0;
+    // Appends: the K/V row at index len, its position, q into the ring of the
+    // periodic update. Nothing in this launch reads them.
+    auto append = [&]() {
       // the K, V and q rows of every appended head as 16-byte chunks, a
       // lane per chunk, every load of a round issued before its stores
       constexpr int CH = RB / 16;  // chunks of a row
       constexpr int NU = 8;        // chunks per lane and round
-      // The appended heads (a < he <= b) are the table's first napp entries:
-      // the first head's rows always reach past a, and only the last head
-      // can continue past b.
-      const int napp = tab.start[n - 1] + tab.vlen[n - 1] <= b ? n : n - 1;
-      constexpr int first_app = 0;
       const int units = napp * 3 * CH;
       for (int u0 = 0; u0 < units; u0 += 32 * NU) {
         uint4 x[NU];
@@ -946,17 +1179,17 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
           const int u = u0 + v * 32 + lane;
           dst[v] = nullptr;
           if (u < units) {
-            const int jj = first_app + u / (3 * CH), w3 = (u / CH) % 3, cc = u % CH;
-            const int h = h0 + jj, i = p.layer_base + h;
+            const int w3 = (u / CH) % 3, cc = u % CH;
+            const int h = h0 + u / (3 * CH), i = p.layer_base + h, j = h - wl;
             const unsigned char *src = w3 == 0 ? static_cast<const unsigned char *>(p.k_new)
                                      : w3 == 1 ? static_cast<const unsigned char *>(p.v_new)
                                                : static_cast<const unsigned char *>(p.q);
             x[v] = reinterpret_cast<const uint4 *>(src + (size_t)h * RB)[cc];
-            const long long row = tab.off[jj] + tab.vlen[jj] - 1;
+            const long long row = tab.off[j] + tab.vlen[j] - 1;
             unsigned char *d = w3 == 0 ? static_cast<unsigned char *>(p.K) + row * RB
                              : w3 == 1 ? static_cast<unsigned char *>(p.V) + row * RB
                                        : static_cast<unsigned char *>(p.qbuf) +
-                                             ((size_t)i * p.period + tab.ntok[jj] % p.period) * RB;
+                                             ((size_t)i * p.period + tab.ntok[j] % p.period) * RB;
             dst[v] = d + (size_t)cc * 16;
           }
         }
@@ -964,29 +1197,49 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         for (int v = 0; v < NU; ++v)
           if (dst[v]) *reinterpret_cast<uint4 *>(dst[v]) = x[v];
       }
-      for (int jj = first_app + lane; jj < first_app + napp; jj += 32)
-        p.pos[tab.off[jj] + tab.vlen[jj] - 1] = p.n_cond + tab.ntok[jj];
+      for (int h = h0 + lane; h < h0 + napp; h += 32) {
+        const int j = h - wl;
+        p.pos[tab.off[j] + tab.vlen[j] - 1] = p.n_cond + tab.ntok[j];
+      }
+    };
+    auto advance = [&]() {  // the counters of the appended heads
+      for (int h = h0 + lane; h < h0 + napp; h += 32) {
+        const int i = p.layer_base + h, j = h - wl;
+        p.len[h] = tab.vlen[j];
+        p.ntok[i] = tab.ntok[j] + 1;
+        if (tab.label[j] != HKV_DENSE) ++p.nbuf[i];
+      }
+    };
+    // Counters advance once the whole grid has arrived (every CTA has read
+    // them). With in_regs every CTA has checked every head, so the step is
+    // known to be taken and the appends need not wait for that; otherwise the
+    // barrier also tells whether some CTA found a bad head.
+    bool advanced = !FUSED;
+    if (FUSED && in_regs) {
+      append();
+      if (poll()) {
+        advance();
+        advanced = true;
+      }
+    } else if (FUSED) {
+      while (!s_abort && !poll())
+        if (timed_out()) break;
+      gen1 = __shfl_sync(0xFFFFFFFFu, gen1, 0);
+      STEP_TRACE_SET(19, globaltimer());
+      if (!s_abort && bar_done && !(gen1 & kBadStep)) {
+        append();
+        advance();
+      }
+      advanced = true;
     }
     STEP_TRACE_SET(8, globaltimer());
-    if (taken) {
-      for (int j = lane; j < n; j += 32) {
-        const long long hs = tab.start[j], he = hs + tab.vlen[j];
-        if (he > a && he <= b) {
-          const int h = h0 + j, i = p.layer_base + h;
-          p.len[h] = tab.vlen[j];
-          p.ntok[i] = tab.ntok[j] + 1;
-          if (tab.label[j] != HKV_DENSE) p.nbuf[i] = tab.nbuf[j] + 1;
-        }
-      }
-    }
 
     // The split head this CTA combines: the other pieces, combined in index
     // order once all of them carry this launch's epoch, then this CTA's own
     // piece (from the epilogue), so the result does not depend on timing.
     const int mh = s_mg_h;
     if (mh >= 0 && !s_abort) {
-      const int np = s_mg_np, mj = s_mg_j;
-      const long long k0 = s_mg_k0;
+      const int np = s_mg_np, mj = s_mg_j, k0 = s_mg_k0;
 #ifdef HKV_STEP_TEST_STALL
       // test builds only: wait for an epoch no launch writes, so that the
       // bounded wait runs out (HKV_ERR_TIMEOUT) with no bulk copy involved
@@ -994,44 +1247,49 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
 #else
       const uint32_t want = s_ep;
 #endif
-      float om = -INFINITY, ol = 0.f, oA[CPL];
-#pragma unroll
-      for (int c = 0; c < CPL; ++c) oA[c] = 0.f;
+      float om = -INFINITY, ol = 0.f, orr = 0.f, oA[CPL];
       for (;;) {
         bool ready = true;
         om = -INFINITY;
-        ol = 0.f;
+        ol = orr = 0.f;
 #pragma unroll
         for (int c = 0; c < CPL; ++c) oA[c] = 0.f;
         for (int t = 0; t < np && ready; ++t) {
           if (t == mj) continue;
           // piece t: the end piece of CTA k0, the start piece of the others
-          const unsigned long long *ps = p.pslot + ((size_t)(k0 + t) * 2 + (t > 0 ? 1 : 0)) * (D + 2);
-          float At[CPL], mt, lt;
+          const unsigned long long *ps = p.pslot + ((size_t)(k0 + t) * 2 + (t > 0 ? 1 : 0)) * PS;
+          float At[CPL], mt, lt, rt = 0.f;
           bool ok = true;
 #pragma unroll
           for (int c = 0; c < CPL; ++c) ok &= ld_pair(ps + CPL * lane + c, want, At[c]);
           ok &= ld_pair(ps + D, want, mt);
           ok &= ld_pair(ps + D + 1, want, lt);
+          if (IDENT) ok &= ld_pair(ps + D + 2, want, rt);
           ready = __all_sync(0xFFFFFFFFu, ok);
           if (!ready) break;
           const float mn = fmaxf(om, mt);
           const float co = om == -INFINITY ? 0.f : exp2f(om - mn);
           const float ct = mt == -INFINITY ? 0.f : exp2f(mt - mn);
           ol = ol * co + lt * ct;
+          orr = orr * co + rt * ct;
 #pragma unroll
           for (int c = 0; c < CPL; ++c) oA[c] = fmaf(At[c], ct, oA[c] * co);
           om = mn;
         }
         if (ready || timed_out()) break;
+        if (!advanced && poll()) {
+          advance();
+          advanced = true;
+        }
       }
       // hand the combined other pieces to the epilogue (not after a wait
       // that ran out: the head's output is then not written)
       if (!s_abort) {
         V::st(&oth_acc[CPL * lane], oA);
         if (lane == 0) {
-          oth_ml[0] = om;
-          oth_ml[1] = ol;
+          oth_s[0] = om;
+          oth_s[1] = ol;
+          if (IDENT) oth_s[NV - 1] = orr;
         }
         __syncwarp();
         mbar_arrive(&oth_bar);  // all 32 lanes
@@ -1042,12 +1300,20 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       __syncwarp();
       if (!s_abort && s_own_state == 2) {
         mbar_wait(&own_bar, 0u);  // complete: every lane acquires own_*
-        float A1[CPL];
+        float A1[CPL], Lt, Rt = 0.f;
         V::lds(&own_acc[CPL * lane], A1);
-        combine_store<CPL>(own_ml[0], own_ml[1], A1, om, ol, oA,
-                           p.out + (size_t)mh * D + CPL * lane);
+        combine_store<CPL, IDENT>(own_s[0], own_s[1], IDENT ? own_s[NV - 1] : 0.f, A1, om, ol, orr,
+                                  oA, p.out + (size_t)mh * D + CPL * lane, Lt, Rt);
+        if (IDENT && lane == 0)
+          p.label_out[p.layer_base + mh] = Rt >= p.tau * Lt ? HKV_LOCAL : HKV_GLOBAL;
         STEP_TRACE_SET(18, globaltimer());
       }
+    }
+    if (!advanced) {
+      while (!s_abort && !poll())
+        if (timed_out()) break;
+      STEP_TRACE_SET(19, globaltimer());
+      if (!s_abort && bar_done) advance();
     }
     if (lane == 0) STEP_TRACE(6);
   }
@@ -1058,18 +1324,31 @@ size_t step_smem() {
   return (size_t)StepShape<D, T>::kNS * StepShape<D, T>::kStageBytes;
 }
 
-template <int D, typename T>
-cudaError_t step_prepare_t(int *ctas) {
+template <int D, typename T, int MODE>
+cudaError_t step_prepare_m(int *ctas) {
   const size_t smem = step_smem<D, T>();
-  cudaError_t e = cudaFuncSetAttribute(step_kernel<D, T>,
+  cudaError_t e = cudaFuncSetAttribute(step_kernel<D, T, MODE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, step_kernel<D, T>,
-                                                       step_threads<D, T>(), smem);
+  int n = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_kernel<D, T, MODE>,
+                                                    step_threads<D, T>(), smem);
+  if (n < *ctas) *ctas = n;
+  return e;
 }
 
 template <int D, typename T>
-cudaError_t step_launch_t(const AttnArgs &a, int grid, cudaStream_t s) {
+cudaError_t step_prepare_t(int *ctas) {
+  *ctas = kStepActivePerSm;
+  cudaError_t e = step_prepare_m<D, T, kModeStep>(ctas);
+  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeIdentify>(ctas);
+  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeAttend>(ctas);
+  return e;
+}
+
+template <int D, typename T>
+cudaError_t step_launch_t(AttnArgs a, int grid, bool fused, cudaStream_t s) {
+  a.grid_recip = (uint32_t)(((1ull << 32) + grid - 1) / grid);  // (not used for a grid of one)
   static const bool pdl = getenv("HKV_NO_PDL") == nullptr;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
@@ -1085,7 +1364,25 @@ cudaError_t step_launch_t(const AttnArgs &a, int grid, cudaStream_t s) {
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, step_kernel<D, T>, a);
+  if (!fused) return cudaLaunchKernelEx(&cfg, step_kernel<D, T, kModeAttend>, a);
+  if (a.label_out) return cudaLaunchKernelEx(&cfg, step_kernel<D, T, kModeIdentify>, a);
+  return cudaLaunchKernelEx(&cfg, step_kernel<D, T, kModeStep>, a);
+}
+
+// The CTAs a layer of n heads gets out of a full grid, and whether the
+// launch fits: see launch_step.
+template <int D, typename T>
+int step_grid_t(long long n, long long max_rows, int full, bool fused) {
+  using S = StepShape<D, T>;
+  const long long g = (max_rows + S::kGR - 1) / S::kGR;
+  const long long total = n * (g + 1 > S::kMinCost ? g + 1 : S::kMinCost);
+  long long chunk = (total + full - 1) / full;
+  if (chunk < S::kMinChunk) chunk = S::kMinChunk;
+  if (n > kStepTable && chunk / S::kMinCost + 2 > kStepTable) return 0;
+  if (!fused) return full;
+  if (n <= full && n <= kStepTable && g <= kAlignedGrains) return (int)n;
+  const long long need = (total + S::kMinChunk - 1) / S::kMinChunk;
+  return need < full ? (int)need : full;
 }
 
 }  // namespace
@@ -1096,9 +1393,12 @@ extern "C" int hkv_debug_set_step_trace(unsigned long long *buf) {
 }
 #endif
 
-int step_tile_rows(int D, int dtype) {
-  if (dtype == HKV_BF16) return D == 64 ? StepShape<64, __nv_bfloat16>::kTT : StepShape<128, __nv_bfloat16>::kTT;
-  return D == 64 ? StepShape<64, float>::kTT : StepShape<128, float>::kTT;
+int step_grid(int D, int dtype, int nheads, int max_rows, int full, bool fused) {
+  if (dtype == HKV_BF16)
+    return D == 64 ? step_grid_t<64, __nv_bfloat16>(nheads, max_rows, full, fused)
+                   : step_grid_t<128, __nv_bfloat16>(nheads, max_rows, full, fused);
+  return D == 64 ? step_grid_t<64, float>(nheads, max_rows, full, fused)
+                 : step_grid_t<128, float>(nheads, max_rows, full, fused);
 }
 
 cudaError_t step_prepare(int D, int dtype, int *ctas) {
@@ -1107,12 +1407,13 @@ cudaError_t step_prepare(int D, int dtype, int *ctas) {
   return D == 64 ? step_prepare_t<64, float>(ctas) : step_prepare_t<128, float>(ctas);
 }
 
-cudaError_t launch_step(const AttnArgs &a, int D, int dtype, int grid, cudaStream_t s) {
+cudaError_t launch_step(const AttnArgs &a, int D, int dtype, int grid, bool fused, cudaStream_t s) {
   if (grid < 1 || grid > kAttnMaxGrid) return cudaErrorInvalidValue;
   if (dtype == HKV_BF16)
-    return D == 64 ? step_launch_t<64, __nv_bfloat16>(a, grid, s)
-                   : step_launch_t<128, __nv_bfloat16>(a, grid, s);
-  return D == 64 ? step_launch_t<64, float>(a, grid, s) : step_launch_t<128, float>(a, grid, s);
+    return D == 64 ? step_launch_t<64, __nv_bfloat16>(a, grid, fused, s)
+                   : step_launch_t<128, __nv_bfloat16>(a, grid, fused, s);
+  return D == 64 ? step_launch_t<64, float>(a, grid, fused, s)
+                 : step_launch_t<128, float>(a, grid, fused, s);
 }
 
 }  // namespace hkv

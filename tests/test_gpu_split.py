@@ -1,0 +1,121 @@
+"""How the one-launch kernel (decode step, attention alone, and the step with
+identification) cuts a layer into CTA ranges, at the sizes where the cut
+changes: a CTA per head up to 12 grains (16 rows; 8 rows of 512 bytes) a
+head, layers around the prologue's table (288 or 352 heads) and around eight
+rows of 32 heads a warp, heads of every length around a grain and a tile,
+and heads split over many CTAs. Every output against Eq. 1 in fp64, the
+appends exact."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp32": 1e-5, "bf16": 2e-3}
+
+
+def _lens(kind, n, grain, rng):
+    if kind == "aligned":      # every head fits the 12 grains, some exactly
+        return np.where(rng.random(n) < 0.3, 12 * grain - 1, rng.integers(0, 12 * grain, n))
+    if kind == "just over":    # one grain too many in one head
+        x = rng.integers(0, 12 * grain, n)
+        x[n // 2] = 12 * grain
+        return x
+    if kind == "edges":
+        e = np.array([0, 1, grain - 2, grain - 1, grain, 2 * grain - 1, 4 * grain - 1, 4 * grain,
+                      8 * grain - 1, 8 * grain, 8 * grain + 1])
+        return e[rng.integers(0, len(e), n)]
+    x = rng.integers(0, 40, n)  # "long": a few heads over many CTAs
+    x[[0, n // 3, n - 1]] = [5000, 3001, 1777]
+    return x
+
+
+CASES = [("aligned", 1), ("aligned", 64), ("aligned", 256), ("just over", 64), ("edges", 287),
+         ("edges", 288), ("edges", 289), ("edges", 351), ("edges", 352), ("edges", 353),
+         ("edges", 2304), ("edges", 2817), ("edges", 3300), ("long", 7), ("long", 300),
+         ("long", 900)]
+
+
+@pytest.mark.parametrize("D,dtype", [(128, "bf16"), (64, "bf16"), (128, "fp32"), (64, "fp32")])
+@pytest.mark.parametrize("kind,n", CASES)
+def test_split(kind, n, D, dtype):
+    import torch
+    from paper_2605_20600_gb300 import hkv as H
+    from paper_2605_20600_gb300.engine import CacheBuffers, torch_dtype
+    rng = np.random.default_rng(n + D)
+    grain = 8 if dtype == "fp32" and D == 128 else 16
+    L, layer = 2, 1
+    lens = _lens(kind, L * n, grain, rng).astype(np.int64)
+    lens[layer * n:] = _lens(kind, n, grain, rng)
+    top = int(lens.max()) + 2
+    cfg = H.make_config(n_layers=L, n_seqs=1, n_heads=n, head_dim=D, dtype=dtype, n_cond=1,
+                        n_image=max(top, 64), row_len=8, recent_w=8, local_w=5, period=8,
+                        group_at=max(top - 2, 9), global_budget=16)
+    caps = lens + 2
+    off = np.concatenate([[0], np.cumsum(caps)[:-1]])
+    total = int(caps.sum())
+    cb = CacheBuffers(cfg, total, "cuda")
+    dt = torch_dtype(cfg)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    cb.k.normal_(generator=g)
+    cb.v.normal_(generator=g)
+    live = torch.zeros(total, dtype=torch.bool, device="cuda")
+    for o, m in zip(off, lens):
+        live[int(o):int(o) + int(m)] = True
+    cb.v[~live] = float("nan")          # rows past a head's length must not be read as values
+    cb.k[~live] = float("nan")
+    cb.off.copy_(torch.from_numpy(off))
+    cb.cap.copy_(torch.from_numpy(caps.astype(np.int32)))
+    cb.len.copy_(torch.from_numpy(lens.astype(np.int32)))
+    cb.ntok.fill_(20)
+    q, k, v = (torch.randn(1, n, D, generator=g, device="cuda").to(dt) for _ in range(3))
+    sl = slice(layer * n, (layer + 1) * n)
+    m, o = lens[sl], off[sl]
+    at = torch.from_numpy(o)[:, None] + torch.arange(int(m.max()) + 1)[None]
+    ok = torch.arange(int(m.max()) + 1)[None] < torch.from_numpy(m)[:, None]
+    at = torch.where(ok, at, 0).cuda()
+    ok = ok.cuda()
+    K = torch.where(ok[:, :, None], cb.k[at].double(), 0.0)
+    V = torch.where(ok[:, :, None], cb.v[at].double(), 0.0)
+
+    def ref(new):
+        Kx, Vx, okx = K, V, ok
+        if new:
+            Kx, Vx = torch.cat([K, k[0].double()[:, None]], 1), torch.cat([V, v[0].double()[:, None]], 1)
+            okx = torch.cat([ok, torch.ones(n, 1, dtype=torch.bool, device="cuda")], 1)
+        s = torch.einsum("nrd,nd->nr", Kx, q[0].double()) / D ** 0.5
+        p = torch.softmax(s.masked_fill(~okx, -torch.inf), 1)
+        p = torch.where(okx.any(1)[:, None], p, 0.0)
+        return torch.einsum("nr,nrd->nd", p, Vx), p
+
+    ws = torch.zeros(H.hkv_workspace_size(cfg), dtype=torch.uint8, device="cuda")
+    st = torch.cuda.current_stream().cuda_stream
+    out = torch.full((1, n, D), float("nan"), device="cuda")
+    H.hkv_decode_attention(cfg, cb.c, layer, q, out, ws, ws.numel(), st)
+    H.hkv_check(cb.c)
+    assert (out[0].double() - ref(False)[0]).abs().max().item() <= TOL[dtype]
+    exp, p = ref(True)
+    label = torch.full((L * n,), 7, dtype=torch.uint8, device="cuda")
+    counters = [t.clone() for t in (cb.len, cb.ntok, cb.nbuf)]
+    for identify in (True, False):
+        for t, b in zip((cb.len, cb.ntok, cb.nbuf), counters):
+            t.copy_(b)
+        out.fill_(float("nan"))
+        if identify:
+            H.hkv_decode_step_identify(cfg, cb.c, layer, q, k, v, out, label, ws, ws.numel(), 0, st)
+        else:
+            H.hkv_decode_step(cfg, cb.c, layer, q, k, v, out, ws, ws.numel(), 0, st)
+        H.hkv_check(cb.c)
+        assert (out[0].double() - exp).abs().max().item() <= TOL[dtype]
+        assert torch.equal(cb.len[sl], counters[0][sl] + 1)
+        assert torch.equal(cb.len[:layer * n], counters[0][:layer * n])
+        assert torch.equal(cb.ntok[sl], counters[1][sl] + 1)
+        rows = torch.from_numpy(o + m).cuda()
+        assert torch.equal(cb.k[rows], k[0]) and torch.equal(cb.v[rows], v[0])
+        assert (cb.pos[rows] == 1 + 20).all()
+        assert torch.equal(cb.qbuf[sl, 20 % 8], q[0])
+    # the newest w_loc - 1 = 4 tokens against tau = 0.9
+    width = torch.from_numpy(m).cuda() + 1
+    order = torch.arange(p.shape[1] - 1, device="cuda")[None]
+    newest = torch.where(order >= (width - 4)[:, None], p[:, :-1], 0.0).sum(1) + p[:, -1]
+    sure = (newest - 0.9).abs() > 1e-5
+    assert torch.equal(label[sl][sure], torch.where(newest >= 0.9, 0, 1).to(torch.uint8)[sure])
