@@ -63,7 +63,7 @@ def build(force: bool = False, extra_flags=(), lib_path: str | None = None,
     os.makedirs(bdir, exist_ok=True)
     cc = nvcc()
     headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
-    headers.append(os.path.join(ROOT, "include", "hkv.h"))
+    headers += [os.path.join(ROOT, "include", f) for f in ("hkv.h", "hkv_layers.h")]
     objs, cmds = [], []
     for src in SOURCES:
         s = os.path.join(CSRC, src)

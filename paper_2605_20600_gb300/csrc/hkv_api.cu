@@ -14,6 +14,7 @@
 
 #include "hkv.h"
 #include "hkv_kernels.h"
+#include "hkv_layers.h"
 
 namespace {
 
@@ -88,9 +89,11 @@ hkv_status attention_ctas(DeviceState *st, int D, int dtype, int *ctas) {
   return HKV_OK;
 }
 
-hkv_status update_ready(DeviceState *st, int D, int dtype, size_t smem) {
+// prepares the cache kernels for `smem` bytes; `limit`: what the interface
+// promises to refuse above 227 KB
+hkv_status update_ready(DeviceState *st, int D, int dtype, size_t smem, size_t limit) {
   std::atomic<size_t> &have = st->update_smem[dt_index(dtype)][d_index(D)];
-  if (smem > kMaxSmem) return HKV_ERR_CAPACITY;
+  if (limit > kMaxSmem || smem > kMaxSmem) return HKV_ERR_CAPACITY;
   if (have.load(std::memory_order_acquire) < smem) {
     std::lock_guard<std::mutex> lk(g_mu);
     if (have.load(std::memory_order_relaxed) < smem) {
@@ -380,11 +383,13 @@ hkv_status hkv_append_evict(const hkv_config *cfg, const hkv_cache *cache, int l
   if (!aligned16(q) || !aligned16(k) || !aligned16(v)) return HKV_ERR_ALIGN;
   DeviceState *st;
   HKV_TRY(device_state(&st));
-  const size_t smem = update_smem_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
-  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem));
+  const int seg = max_segment(*cfg);
+  const size_t smem = update_smem_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype);
+  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem,
+                       update_limit_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype)));
   const int hpl = heads_per_layer(cfg);
   return cuda_status(launch_append_evict(cache_args(cache), method_args(cfg), layer * hpl, hpl, q,
-                                         k, v, cfg->head_dim, cfg->dtype, smem,
+                                         k, v, cfg->head_dim, cfg->dtype, seg, smem,
                                          (cudaStream_t)stream));
 }
 
@@ -473,12 +478,14 @@ hkv_status evict_layers(const hkv_config *cfg, const hkv_cache *cache, int first
                         hkv_stream_t stream) {
   DeviceState *st;
   HKV_TRY(device_state(&st));
-  const size_t smem = update_smem_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
-  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem));
+  const int seg = max_segment(*cfg);
+  const size_t smem = update_smem_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype);
+  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem,
+                       update_limit_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype)));
   const long long hpl = heads_per_layer(cfg);
   if (hpl * count > 0x7FFFFFFFLL) return HKV_ERR_SHAPE;  // one CTA per head
   return cuda_status(launch_evict(cache_args(cache), method_args(cfg), (int)(first * hpl),
-                                  (int)(count * hpl), cfg->head_dim, cfg->dtype, smem,
+                                  (int)(count * hpl), cfg->head_dim, cfg->dtype, seg, smem,
                                   (cudaStream_t)stream));
 }
 
@@ -512,10 +519,10 @@ hkv_status hkv_identify_heads(const hkv_config *cfg, const hkv_cache *cache, int
   DeviceState *st;
   HKV_TRY(device_state(&st));
   const int max_len = cfg->n_cond + cfg->group_at;
-  const size_t upd = update_smem_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
+  const size_t upd = update_limit_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
   const size_t need = identify_smem_bytes(max_len, cfg->period,
                                           cfg->distance_mode == HKV_DIST_GRID2D, false);
-  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, upd > need ? upd : need));
+  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, need, upd > need ? upd : need));
   const int hpl = heads_per_layer(cfg);
   return cuda_status(launch_identify(cache_args(cache), method_args(cfg), layer * hpl, hpl, q,
                                      label_out, nh_out, cfg->head_dim, cfg->dtype, max_len,
@@ -532,10 +539,10 @@ hkv_status hkv_identify_heads_multi(const hkv_config *cfg, const hkv_cache *cach
   DeviceState *st;
   HKV_TRY(device_state(&st));
   const int max_len = cfg->n_cond + cfg->group_at;
-  const size_t upd = update_smem_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
+  const size_t upd = update_limit_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
   const size_t need = identify_smem_bytes(max_len, cfg->period,
                                           cfg->distance_mode == HKV_DIST_GRID2D, true);
-  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, upd > need ? upd : need));
+  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, need, upd > need ? upd : need));
   const int hpl = heads_per_layer(cfg);
   return cuda_status(launch_identify_multi(cache_args(cache), method_args(cfg), layer * hpl, hpl,
                                            label_out, nh_out, cfg->head_dim, cfg->dtype, max_len,
@@ -568,22 +575,42 @@ hkv_status hkv_allocate_budgets(const hkv_config *cfg, const uint8_t *label, int
   return HKV_OK;
 }
 
+namespace {
+
+// repack of the layers [first, first + count) in one launch
+hkv_status repack_layers(const hkv_config *cfg, const hkv_cache *dense, const hkv_cache *ragged,
+                         int first, int count, hkv_stream_t stream) {
+  HKV_TRY(check_cache(dense));
+  HKV_TRY(check_cache(ragged));
+  if (first < 0 || first >= cfg->n_layers) return HKV_ERR_INVALID_ARG;
+  if (dense->qbuf != ragged->qbuf) return HKV_ERR_INVALID_ARG;
+  DeviceState *st;
+  HKV_TRY(device_state(&st));
+  const int seg = max_segment(*cfg);
+  const size_t smem = update_smem_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype);
+  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem,
+                       update_limit_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype)));
+  const int hpl = heads_per_layer(cfg);
+  return cuda_status(launch_repack(cache_args(dense), cache_args(ragged), method_args(cfg),
+                                   first * hpl, count * hpl, cfg->head_dim, cfg->dtype, seg, smem,
+                                   (cudaStream_t)stream));
+}
+
+}  // namespace
+
 hkv_status hkv_repack(const hkv_config *cfg, const hkv_cache *dense, const hkv_cache *ragged,
                       int layer, hkv_stream_t stream) {
   HKV_TRY(injected("repack"));
   HKV_TRY(hkv_validate_config(cfg));
-  HKV_TRY(check_cache(dense));
-  HKV_TRY(check_cache(ragged));
-  if (layer < 0 || layer >= cfg->n_layers) return HKV_ERR_INVALID_ARG;
-  if (dense->qbuf != ragged->qbuf) return HKV_ERR_INVALID_ARG;
-  DeviceState *st;
-  HKV_TRY(device_state(&st));
-  const size_t smem = update_smem_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
-  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem));
-  const int hpl = heads_per_layer(cfg);
-  return cuda_status(launch_repack(cache_args(dense), cache_args(ragged), method_args(cfg),
-                                   layer * hpl, hpl, cfg->head_dim, cfg->dtype, smem,
-                                   (cudaStream_t)stream));
+  return repack_layers(cfg, dense, ragged, layer, 1, stream);
+}
+
+hkv_status hkv_repack_all(const hkv_config *cfg, const hkv_cache *dense, const hkv_cache *ragged,
+                          hkv_stream_t stream) {
+  HKV_TRY(injected("repack_all"));
+  HKV_TRY(injected("repack"));
+  HKV_TRY(hkv_validate_config(cfg));
+  return repack_layers(cfg, dense, ragged, 0, cfg->n_layers, stream);
 }
 
 hkv_status hkv_export_state(const hkv_config *cfg, const hkv_cache *cache, int layer,

@@ -30,11 +30,24 @@
 namespace hkv {
 namespace {
 
-constexpr int NT = kCacheThreads;
-// update kernels resident per SM that the register budget allows (48
-// registers a thread, no spills): a layer of many short heads (one CTA each)
-// then runs in fewer waves; shared memory may allow fewer
-constexpr int kUpdCtasPerSm = 5;
+// threads of the update kernels, and of the identification kernels (whose
+// sums' order goes with it)
+#ifndef HKV_UPD_THREADS
+#define HKV_UPD_THREADS 128
+#endif
+constexpr int NT = HKV_UPD_THREADS;
+constexpr int IT = kCacheThreads;
+// Update kernels resident per SM that the register budget allows (48 registers
+// a thread, no spills). An update is a chain of latency-bound phases between
+// block barriers, so what counts is how many run at once: CTAs of four warps,
+// up to ten on an SM, rather than eight warps staging whole rows of keys in 70
+// KB, two or three on an SM. Lumina-mGPT 1024, 8 sequences, all layers: 475 ->
+// 327 us (of 264 at the measured bandwidth); with 256 threads and four CTAs
+// 339. LlamaGen-XL's 92160 heads of up to 121 rows: 1.34 -> 0.9 ms a period.
+#ifndef HKV_UPD_CTAS
+#define HKV_UPD_CTAS 10
+#endif
+constexpr int kUpdCtasPerSm = HKV_UPD_CTAS;
 
 // Phase timestamps per head of the update for latency studies; compiled out
 // by default.
@@ -79,47 +92,61 @@ struct UpdShared {
 
 // Shared-memory work area of one update (dynamic).
 struct UpdSmem {
-  unsigned char *ring;       // [P][D] the buffered queries (<= 4 B each)
-  unsigned long long *keys;  // [max_len]
-  int *ps;                   // [max_len] positions of the source rows
-  int *aux;                  // [max_len] class, then keep flag, then rank
-  float *qbar;               // [D]
-  int *hist;                 // [512]
-  int stage_rows;            // rows a warp stages per pass of the score phase
+  unsigned char *ring;  // [P][D] the buffered queries (<= 4 B each); then the score stages
+  uint32_t *kh;         // [max_len] high words of the selection keys (the low ones: positions)
+  int *ps;              // [max_len] positions of the source rows
+  int16_t *aux;         // [max_len] class, then keep flag, then rank
+  float *qbar;          // [D]
+  int *hist;            // [512]
+  int stage_rows;       // rows a warp stages at a time in the score phase
 };
 
-// Rows a warp stages per pass of the score phase: 32, or fewer when every
+// Rows a warp stages at a time in the score phase: 32, or fewer when every
 // warp's share of the longest segment is smaller (short segments then leave
 // room for more CTAs per SM).
 __host__ __device__ constexpr int stage_rows(int max_len) {
   return max_len >= NT ? 32 : (max_len + NT / 32 - 1) / (NT / 32) < 1 ? 1 : (max_len + NT / 32 - 1) / (NT / 32);
 }
 
-// the query ring (P rows of es-byte elements); after q-bar it is the score
-// stage: NT/32 warps x stage_rows rows of D * es + 16 bytes
+// The score phase stages 64 bytes of each row at a time, two such pieces in
+// flight per warp, at a row stride of 80 bytes (lanes that read the same
+// 16-byte column of consecutive rows hit distinct banks).
+constexpr int kChunk = 64, kChunkStride = kChunk + 16, kChunkStages = 2;
+__host__ __device__ constexpr size_t stage_bytes_of(int rows) {
+  return (size_t)rows * kChunkStride * kChunkStages;
+}
+__host__ __device__ constexpr size_t stage_bytes(int max_len) {
+  return stage_bytes_of(stage_rows(max_len));
+}
+
+// the query ring (P rows of es-byte elements); after q-bar the score stages,
+// and at the end the list of the rows that fill holes
 __host__ __device__ constexpr size_t ring_bytes(int P, int D, int es, int max_len) {
-  return (size_t)P * D * es > (size_t)(NT / 32) * stage_rows(max_len) * (D * es + 16)
-             ? (size_t)P * D * es
-             : (size_t)(NT / 32) * stage_rows(max_len) * (D * es + 16);
+  size_t b = (size_t)P * D * es;
+  if (b < (size_t)(NT / 32) * stage_bytes(max_len)) b = (size_t)(NT / 32) * stage_bytes(max_len);
+  if (b < (size_t)max_len * 4) b = (size_t)max_len * 4;
+  return (b + 15) / 16 * 16;
 }
 
 __device__ __forceinline__ UpdSmem carve(unsigned char *dyn, int max_len, int D, int P, int es) {
   UpdSmem u;
   u.ring = dyn;
   u.stage_rows = stage_rows(max_len);
-  u.keys = reinterpret_cast<unsigned long long *>(dyn + ring_bytes(P, D, es, max_len));
-  u.ps = reinterpret_cast<int *>(u.keys + max_len);
-  u.aux = u.ps + max_len;
-  u.qbar = reinterpret_cast<float *>(u.aux + max_len);
+  u.qbar = reinterpret_cast<float *>(dyn + ring_bytes(P, D, es, max_len));
   u.hist = reinterpret_cast<int *>(u.qbar + D);
+  u.kh = reinterpret_cast<uint32_t *>(u.hist + 512);
+  u.ps = reinterpret_cast<int *>(u.kh + max_len);
+  u.aux = reinterpret_cast<int16_t *>(u.ps + max_len);
   return u;
 }
 
 // The k0-th smallest key among rows of class 0 and the k1-th among rows of
 // class 1 (1-based; 0 = not needed; other classes ignored), by MSD radix
-// select on bytes from `top_shift` down. Keys are unique within a class, so
-// each result bounds exactly k keys of its class from above.
-__device__ void radix_select2(const unsigned long long *keys, const int *cls, int n, int k0,
+// select on bytes from `top_shift` down. A key is (kh[j], ps[j]), or ps[j]
+// alone. Keys are unique within a class, so each result bounds exactly k keys
+// of its class from above.
+template <bool HIGH>
+__device__ void radix_select2(const uint32_t *kh, const int *ps, const int16_t *cls, int n, int k0,
                               int k1, int top_shift, int *hist, UpdShared &sh) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {
@@ -137,7 +164,7 @@ __device__ void radix_select2(const unsigned long long *keys, const int *cls, in
     for (int j = tid; j < n; j += NT) {
       const int s = cls[j];
       if (s != 0 && s != 1) continue;
-      const unsigned long long key = keys[j];
+      const unsigned long long key = (HIGH ? (unsigned long long)kh[j] << 32 : 0ull) | (uint32_t)ps[j];
       if ((s ? r1 : r0) > 0 && (key & hi) == (s ? p1 : p0))
         atomicAdd(&hist[s * 256 + (int)((key >> shift) & 255ull)], 1);
     }
@@ -198,9 +225,22 @@ __device__ int select_evictions(const SegRef &sg, int label, const MethodArgs &m
                                 UpdShared &sh) {
   constexpr int RB = D * (int)sizeof(T);
   constexpr int EPL = Elem<T>::kPerPiece;
-  constexpr int LPR = RB / 16;
   const int tid = threadIdx.x;
-  const int C = m.C;
+  const int C = m.C, P = m.P;
+  // the head's history budget, B_g - w with the paper's budgets, from the
+  // capacity its segment was given (C + budget + P)
+  const int hist_budget = sg.dst_cap - C - P - m.w > 0 ? sg.dst_cap - C - P - m.w : 0;
+  // The queries of a head that will score its history come in with one bulk
+  // copy, on its way while the history is counted and split.
+  auto fetch_ring = [&]() {
+    mbar_init(&sh.ring_bar, 1);
+    fence_barrier_init();
+    const uint32_t bytes = (uint32_t)P * RB;
+    mbar_arrive_expect_tx(&sh.ring_bar, bytes);
+    bulk_g2s(u.ring, qring, bytes, &sh.ring_bar);
+  };
+  const bool early = label == HKV_GLOBAL && sg.len - C - (ntok < m.w ? ntok : m.w) > hist_budget;
+  if (early && tid == 0) fetch_ring();
   const int recent_from = C + (ntok > m.w ? ntok - m.w : 0);   // newest w image tokens
   int nh = 0;
   for (int r = tid; r < sg.len; r += NT) {
@@ -212,14 +252,12 @@ __device__ int select_evictions(const SegRef &sg, int label, const MethodArgs &m
   }
   const int NH = block_sum(nh, sh);  // history candidates (Eq. 2)
   HKV_UTRACE(1);
-  // the head's history budget, B_g - w with the paper's budgets, from the
-  // capacity its segment was given (C + budget + P)
-  const int hist_budget = sg.dst_cap - C - m.P - m.w > 0 ? sg.dst_cap - C - m.P - m.w : 0;
   int M = 0;
   if (label == HKV_LOCAL) M = NH;    // Eq. 3: no history
   else if (NH > hist_budget) M = NH - hist_budget;
 
   if (label == HKV_GLOBAL && M > 0) {
+    auto key_of = [&](int r) { return ((unsigned long long)u.kh[r] << 32) | (uint32_t)u.ps[r]; };
     // Eq. 5: the floor(NH r_s) oldest history tokens are long-range (or,
     // in the grid-distance variant, the farthest from the newest image
     // token, equal distances older first)
@@ -229,18 +267,16 @@ __device__ int select_evictions(const SegRef &sg, int label, const MethodArgs &m
       for (int r = tid; r < sg.len; r += NT) {
         const int i = u.ps[r] - C;
         const long long dr = i / m.row_len - ref / m.row_len, dc = i % m.row_len - ref % m.row_len;
-        const unsigned long long far = 0x7FFFFFFFull - (unsigned long long)(dr * dr + dc * dc);
-        u.keys[r] = (far << 32) | (uint32_t)u.ps[r];
+        u.kh[r] = 0x7FFFFFFFu - (uint32_t)(dr * dr + dc * dc);
       }
-      radix_select2(u.keys, u.aux, sg.len, n_long, 0, 56, u.hist, sh);
+      radix_select2<true>(u.kh, u.ps, u.aux, sg.len, n_long, 0, 56, u.hist, sh);
       const unsigned long long k_long = sh.prefix[0];
       for (int r = tid; r < sg.len; r += NT)
-        if (u.aux[r] == 0) u.aux[r] = u.keys[r] <= k_long ? 0 : 1;
+        if (u.aux[r] == 0) u.aux[r] = key_of(r) <= k_long ? 0 : 1;
     } else if (n_long > 0 && n_long < NH) {
-      for (int r = tid; r < sg.len; r += NT) u.keys[r] = (unsigned long long)(uint32_t)u.ps[r];
       const int maxp = C + ntok;  // positions are below it: start at its top byte
       const int top = maxp < (1 << 8) ? 0 : maxp < (1 << 16) ? 8 : maxp < (1 << 24) ? 16 : 24;
-      radix_select2(u.keys, u.aux, sg.len, n_long, 0, top, u.hist, sh);
+      radix_select2<false>(u.kh, u.ps, u.aux, sg.len, n_long, 0, top, u.hist, sh);
       const int p_long = (int)sh.prefix[0];
       for (int r = tid; r < sg.len; r += NT)
         if (u.aux[r] == 0) u.aux[r] = u.ps[r] <= p_long ? 0 : 1;
@@ -249,64 +285,73 @@ __device__ int select_evictions(const SegRef &sg, int label, const MethodArgs &m
         if (u.aux[r] == 0) u.aux[r] = n_long == NH ? 0 : 1;
     }
     HKV_UTRACE(2);
-    // Eq. 6 scores: q-bar = the P buffered queries, oldest first. The ring
-    // comes in with one bulk copy; the sums keep their order.
-    const int P = m.P;
-    if (tid == 0) {
-      mbar_init(&sh.ring_bar, 1);
-      fence_barrier_init();
-    }
+    // Eq. 6 scores: q-bar = the P buffered queries, oldest first (image token
+    // t in slot t mod P); the sums keep their order.
+    if (!early && tid == 0) fetch_ring();
     __syncthreads();
-    if (tid == 0) {
-      const uint32_t bytes = (uint32_t)P * RB;
-      mbar_arrive_expect_tx(&sh.ring_bar, bytes);
-      bulk_g2s(u.ring, qring, bytes, &sh.ring_bar);
-    }
     if (!mbar_wait(&sh.ring_bar, 0) && tid == 0) set_err(sg.err, HKV_ERR_TIMEOUT);
     for (int d = tid; d < D; d += NT) {
       float acc = 0.f;
-      for (int pp = 0; pp < P; ++pp) {
-        int slot = (ntok - P + pp) % P;
-        if (slot < 0) slot += P;
+      const int oldest = ntok % P;
+#pragma unroll 8
+      for (int slot = oldest; slot < P; ++slot)
         acc = __fadd_rn(acc, Elem<T>::load1(u.ring, (size_t)slot * D + d));
-      }
+#pragma unroll 8
+      for (int slot = 0; slot < oldest; ++slot)
+        acc = __fadd_rn(acc, Elem<T>::load1(u.ring, (size_t)slot * D + d));
       u.qbar[d] = acc;
     }
     __syncthreads();
     HKV_UTRACE(3);
-    // Each warp stages 32 rows at a time in the (now free) ring area with
-    // coalesced 16-byte async copies, at a row stride of LPR + 1 pieces so
-    // that lane l reading row l, piece j, hits distinct banks; then lane l
-    // sums its row in the fixed order.
-    constexpr int RS = LPR + 1;  // row stride in 16-byte pieces
+    // Each warp takes blocks of stage_rows rows and stages 64 bytes of every
+    // candidate row at a time in the (now free) ring area with 16-byte async
+    // copies, the next piece on its way while lane l sums row l's in the fixed
+    // order of channels.
     const int warp = tid >> 5, lane = tid & 31;
     const int SR = u.stage_rows;
-    unsigned char *stage = u.ring + (size_t)warp * SR * RS * 16;
-    for (int base = warp * SR; base < sg.len; base += (NT / 32) * SR) {
-      const int nrows = sg.len - base < SR ? sg.len - base : SR;
-      for (int w = lane; w < nrows * LPR; w += 32) {
-        const int rr = w / LPR, pc = w % LPR;
-        cp_async16(stage + (rr * RS + pc) * 16, sg.sk + (size_t)(base + rr) * RB + pc * 16);
-      }
-      cp_async_wait_all();
-      __syncwarp();
-      const int r = base + lane;
-      if (lane < nrows && u.aux[r] >= 0) {
-        const unsigned char *krow = stage + lane * RS * 16;
-        float s = 0.f;
+    constexpr int NCH = RB / kChunk, PPC = kChunk / 16;  // pieces of a row, 16-byte columns of one
+    static_assert(RB % kChunk == 0, "whole pieces");
+    unsigned char *stage = u.ring + (size_t)warp * stage_bytes_of(SR);
+    const int blocks = (sg.len + SR - 1) / SR;
+    const int mine = blocks > warp ? (blocks - warp + NT / 32 - 1) / (NT / 32) : 0;
+    auto issue = [&](int step) {
+      const int base = (warp + step / NCH * (NT / 32)) * SR;
+      unsigned char *dst = stage + (step & 1) * SR * kChunkStride;
+      const unsigned char *src = sg.sk + (size_t)base * RB + (step % NCH) * kChunk;
 #pragma unroll 4
-        for (int pc = 0; pc < LPR; ++pc) {
+      for (int w = lane; w < SR * PPC; w += 32) {
+        const int rr = w / PPC, pc = w % PPC;
+        if (base + rr < sg.len && u.aux[base + rr] >= 0)
+          cp_async16(dst + rr * kChunkStride + pc * 16, src + (size_t)rr * RB + pc * 16);
+      }
+    };
+    if (mine > 0) issue(0);
+    cp_async_commit();
+    float s = 0.f;
+    for (int step = 0; step < mine * NCH; ++step) {
+      if (step + 1 < mine * NCH) issue(step + 1);
+      cp_async_commit();
+      cp_async_wait<1>();
+      __syncwarp();
+      const int r = (warp + step / NCH * (NT / 32)) * SR + lane;
+      if (lane < SR && r < sg.len && u.aux[r] >= 0) {
+        if (step % NCH == 0) s = 0.f;
+        const unsigned char *krow = stage + (step & 1) * SR * kChunkStride + lane * kChunkStride;
+        const float *qb = u.qbar + (step % NCH) * PPC * EPL;
+#pragma unroll
+        for (int pc = 0; pc < PPC; ++pc) {
           float kf[EPL];
           Elem<T>::unpack(*reinterpret_cast<const uint4 *>(krow + pc * 16), kf);
 #pragma unroll
-          for (int e = 0; e < EPL; ++e) s = __fadd_rn(s, __fmul_rn(u.qbar[pc * EPL + e], kf[e]));
+          for (int e = 0; e < EPL; ++e) s = __fadd_rn(s, __fmul_rn(qb[pc * EPL + e], kf[e]));
         }
-        s = __fadd_rn(s, 0.f);  // -0 reads as +0
-        uint32_t bits = __float_as_uint(s);
-        bits = (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);  // order-preserving
-        u.keys[r] = ((unsigned long long)bits << 32) | (uint32_t)u.ps[r];
+        if (step % NCH == NCH - 1) {
+          const float z = __fadd_rn(s, 0.f);  // -0 reads as +0
+          const uint32_t bits = __float_as_uint(z);
+          u.kh[r] = (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);  // order-preserving
+        }
       }
-      __syncwarp();  // the stage is rewritten next round
+      __syncwarp();  // the stage is rewritten by the next piece but one
     }
     __syncthreads();
     HKV_UTRACE(4);
@@ -320,30 +365,24 @@ __device__ int select_evictions(const SegRef &sg, int label, const MethodArgs &m
       m_long += m_near - (NH - n_long);
       m_near = NH - n_long;
     }
-    radix_select2(u.keys, u.aux, sg.len, m_long, m_near, 56, u.hist, sh);
+    radix_select2<true>(u.kh, u.ps, u.aux, sg.len, m_long, m_near, 56, u.hist, sh);
     const unsigned long long thr0 = sh.prefix[0], thr1 = sh.prefix[1];
     for (int r = tid; r < sg.len; r += NT) {
       const int c = u.aux[r];
-      const bool ev = c == 0 ? (m_long > 0 && u.keys[r] <= thr0)
-                             : c == 1 ? (m_near > 0 && u.keys[r] <= thr1) : false;
+      const bool ev = c == 0 ? (m_long > 0 && key_of(r) <= thr0)
+                             : c == 1 ? (m_near > 0 && key_of(r) <= thr1) : false;
       u.aux[r] = ev ? 0 : 1;
     }
     HKV_UTRACE(5);
   } else {
+    if (early) {  // fetched for nothing: it must have landed before the CTA ends
+      __syncthreads();
+      if (!mbar_wait(&sh.ring_bar, 0) && tid == 0) set_err(sg.err, HKV_ERR_TIMEOUT);
+    }
     for (int r = tid; r < sg.len; r += NT) u.aux[r] = (u.aux[r] == 0 && M > 0) ? 0 : 1;
   }
   __syncthreads();
   return M;
-}
-
-template <int D, typename T>
-__device__ __forceinline__ void copy_piece(unsigned char *dk, unsigned char *dv,
-                                           const unsigned char *sk, const unsigned char *sv,
-                                           int piece) {
-  *reinterpret_cast<uint4 *>(dk + piece * 16) =
-      __ldcg(reinterpret_cast<const uint4 *>(sk + piece * 16));
-  *reinterpret_cast<uint4 *>(dv + piece * 16) =
-      __ldcg(reinterpret_cast<const uint4 *>(sv + piece * 16));
 }
 
 // In place: the new length is len - M; every evicted row below it takes a
@@ -360,9 +399,9 @@ __device__ int fill_holes(const SegRef &sg, int M, const UpdSmem &u, UpdShared &
   const int tid = threadIdx.x;
   const int len = sg.len, new_len = len - M;
   if (M == 0) return len;
-  // the keys area is free now and holds the two index lists
-  int *hole = reinterpret_cast<int *>(u.keys);  // [M]
-  int *fill = hole + M;                          // [M]
+  // the key and stage areas are free now and hold the two index lists
+  int *hole = reinterpret_cast<int *>(u.kh);    // [M]
+  int *fill = reinterpret_cast<int *>(u.ring);  // [M]
   const int per = (len + NT - 1) / NT;
   const int r0 = tid * per < len ? tid * per : len;
   const int r1 = r0 + per < len ? r0 + per : len;
@@ -426,12 +465,27 @@ __device__ int copy_kept(const SegRef &sg, const UpdSmem &u, UpdShared &sh) {
     run += tot;
   }
   __syncthreads();
-  for (int w = tid; w < sg.len * LPR; w += NT) {
-    const int r = w / LPR, pc = w % LPR;
-    const int d = u.aux[r];
-    if (d >= 0)
-      copy_piece<D, T>(sg.dk + (size_t)d * RB, sg.dv + (size_t)d * RB, sg.sk + (size_t)r * RB,
-                       sg.sv + (size_t)r * RB, pc);
+  // each batch issues all of its loads before its stores
+  constexpr int B = 4;
+  for (int w0 = 0; w0 < sg.len * LPR; w0 += NT * B) {
+    uint4 kb[B], vb[B];
+    int d[B];
+#pragma unroll
+    for (int x = 0; x < B; ++x) {
+      const int w = w0 + x * NT + tid;
+      d[x] = w < sg.len * LPR ? u.aux[w / LPR] : -1;
+      if (d[x] >= 0) {
+        kb[x] = __ldcg(reinterpret_cast<const uint4 *>(sg.sk + (size_t)w * 16));
+        vb[x] = __ldcg(reinterpret_cast<const uint4 *>(sg.sv + (size_t)w * 16));
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < B; ++x)
+      if (d[x] >= 0) {
+        const size_t at = (size_t)d[x] * RB + (w0 + x * NT + tid) % LPR * 16;
+        *reinterpret_cast<uint4 *>(sg.dk + at) = kb[x];
+        *reinterpret_cast<uint4 *>(sg.dv + at) = vb[x];
+      }
   }
   for (int r = tid; r < sg.len; r += NT)
     if (u.aux[r] >= 0) sg.dpos[u.aux[r]] = u.ps[r];
@@ -675,7 +729,7 @@ __host__ __device__ constexpr size_t id_smem(size_t floats, int max_len, bool gr
 // of the j-th token counted. Image tokens by squared grid distance from image
 // token ref, nearest first, equal distances newer first; then the
 // conditioning tokens, newest first. Keys are unique (positions are); each
-// row's rank is the number of smaller keys (len^2 / NT comparisons per
+// row's rank is the number of smaller keys (len^2 / IT comparisons per
 // thread, once per head and generation). Block-uniform.
 __device__ void grid_count_order(const int32_t *pos, int len, int C, int row_len, int ref,
                                  unsigned long long *keys, int *perm) {
@@ -706,14 +760,14 @@ __device__ void grid_count_order(const int32_t *pos, int len, int C, int row_len
 // grid-distance variant); local iff fewer than w_loc tokens were needed.
 // The dense cache holds its tokens in position order.
 template <int D, typename T, int U>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(IT)
     identify_kernel(const CacheArgs c, const MethodArgs m, int layer_base, const void *q,
                     uint8_t *label_out, int32_t *nh_out, float qscale, int max_len) {
   constexpr int RB = D * (int)sizeof(T);
   constexpr int EPL = Elem<T>::kPerPiece;
   constexpr int LPR = RB / 16;
   constexpr int RPW = 32 / LPR;
-  constexpr int NW = NT / 32;
+  constexpr int NW = IT / 32;
   extern __shared__ float e[];
   __shared__ float red[NW];
   __shared__ float s_bcast;
@@ -769,7 +823,7 @@ __global__ void __launch_bounds__(NT)
   }
   __syncthreads();
   float mx = -INFINITY;
-  for (int r = tid; r < len; r += NT) mx = fmaxf(mx, e[r]);
+  for (int r = tid; r < len; r += IT) mx = fmaxf(mx, e[r]);
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
   if (lane == 0) red[warp] = mx;
@@ -782,7 +836,7 @@ __global__ void __launch_bounds__(NT)
   __syncthreads();
   mx = s_bcast;
   float sum = 0.f;
-  for (int r = tid; r < len; r += NT) {
+  for (int r = tid; r < len; r += IT) {
     const float x = exp2f(e[r] - mx);
     e[r] = x;
     sum += x;
@@ -808,7 +862,7 @@ __global__ void __launch_bounds__(NT)
                      reinterpret_cast<unsigned long long *>(base), perm);
   }
   float running = 0.f;  // cumulative mass from the newest token
-  for (int base = 0; base < len; base += NT) {
+  for (int base = 0; base < len; base += IT) {
     const int jb = base + tid;  // jb-th token counted (0 = current)
     const float x = jb < len ? e[perm ? perm[jb] : len - 1 - jb] : 0.f;
     float tot;
@@ -870,14 +924,14 @@ __host__ __device__ constexpr int id_qb(int P) { return P >= kIdQB8From ? 8 : 4;
 // identify_kernel. One CTA per head; each pass over the keys serves QB
 // queries (every key row loaded once per pass, dotted with all of them).
 template <int D, typename T, int QB, int U>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(IT)
     identify_multi_kernel(const CacheArgs c, const MethodArgs m, int layer_base,
                           uint8_t *label_out, int32_t *nh_out, float qscale, int max_len) {
   constexpr int RB = D * (int)sizeof(T);
   constexpr int EPL = Elem<T>::kPerPiece;
   constexpr int LPR = RB / 16;
   constexpr int RPW = 32 / LPR;
-  constexpr int NW = NT / 32;
+  constexpr int NW = IT / 32;
   extern __shared__ float e[];      // [QB][max_len] the pass's logits, then weights
   float *pbar = e + QB * max_len;  // [max_len] summed weights of all queries
   __shared__ float red[QB * NW];
@@ -907,7 +961,7 @@ __global__ void __launch_bounds__(NT)
   const int grp = lane / LPR, col = lane % LPR;
   const unsigned char *K = static_cast<const unsigned char *>(c.K) + off * RB;
   const unsigned char *ring = static_cast<const unsigned char *>(c.qbuf) + (size_t)i * m.P * RB;
-  for (int r = tid; r < len; r += NT) pbar[r] = 0.f;
+  for (int r = tid; r < len; r += IT) pbar[r] = 0.f;
   for (int p0 = 0; p0 < Pe; p0 += QB) {
     // query p0 + b sees mq[b] keys (0 past the newest query)
     int mq[QB];
@@ -960,7 +1014,7 @@ __global__ void __launch_bounds__(NT)
     float acc[QB];
 #pragma unroll
     for (int b = 0; b < QB; ++b) acc[b] = -INFINITY;
-    for (int r = tid; r < mmax; r += NT)
+    for (int r = tid; r < mmax; r += IT)
 #pragma unroll
       for (int b = 0; b < QB; ++b)
         if (r < mq[b]) acc[b] = fmaxf(acc[b], e[b * max_len + r]);
@@ -971,7 +1025,7 @@ __global__ void __launch_bounds__(NT)
       mx[b] = acc[b];
       acc[b] = 0.f;
     }
-    for (int r = tid; r < mmax; r += NT)
+    for (int r = tid; r < mmax; r += IT)
 #pragma unroll
       for (int b = 0; b < QB; ++b)
         if (r < mq[b]) {
@@ -982,7 +1036,7 @@ __global__ void __launch_bounds__(NT)
     block_all<false, QB>(acc, red, s_b);
 #pragma unroll
     for (int b = 0; b < QB; ++b) acc[b] = 1.f / acc[b];  // unused past the newest query
-    for (int r = tid; r < mmax; r += NT) {
+    for (int r = tid; r < mmax; r += IT) {
       float s = pbar[r];
 #pragma unroll
       for (int b = 0; b < QB; ++b)
@@ -992,7 +1046,7 @@ __global__ void __launch_bounds__(NT)
     __syncthreads();  // e is rewritten by the next pass
   }
   float tot[1] = {0.f};
-  for (int r = tid; r < len; r += NT) tot[0] += pbar[r];
+  for (int r = tid; r < len; r += IT) tot[0] += pbar[r];
   block_all<false, 1>(tot, red, s_b);
   const float thr = tot[0] * m.tau;
   if (tid == 0) s_nh = len;
@@ -1006,7 +1060,7 @@ __global__ void __launch_bounds__(NT)
                      reinterpret_cast<unsigned long long *>(base), perm);
   }
   float running = 0.f;  // cumulative mass from the newest token
-  for (int base = 0; base < len; base += NT) {
+  for (int base = 0; base < len; base += IT) {
     const int jb = base + tid;  // jb-th token counted (0 = current)
     const float x = jb < len ? pbar[perm ? perm[jb] : len - 1 - jb] : 0.f;
     float t;
@@ -1065,6 +1119,61 @@ __global__ void budgets_kernel(const uint8_t *label, int32_t *budget, int32_t *c
   if (__syncthreads_or(bad) && threadIdx.x == 0) off[n - 1] = -1;  // reported as a state error
 }
 
+// The same without groups, over several CTAs of kBudgetHeads heads each: a
+// CTA counts the global heads before its own from the labels (n bytes out of
+// L2, at most 1 MB, see launch_budgets), so that none waits for another. One
+// CTA looping over blocks of heads took a load and a scan of 1.3 us for every
+// 1024 heads.
+constexpr int kBudgetHeads = 4096, kBudgetThreads = 256;
+constexpr int kBudgetMost = 1 << 20;
+__global__ void __launch_bounds__(kBudgetThreads)
+    budgets_plain_kernel(const uint8_t *label, int32_t *budget, int32_t *cap, int64_t *off, int n,
+                         int C, int B_g, int w, int P) {
+  constexpr int NW = kBudgetThreads / 32, PER = kBudgetHeads / NW;
+  __shared__ int s_before[NW], s_own[NW];
+  pdl_wait();
+  pdl_launch_dependents();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int first = blockIdx.x * kBudgetHeads;
+  int bad = 0, count = 0;
+  auto tally = [&](int i) {
+    const int lb = label[i];
+    bad |= lb != HKV_GLOBAL && lb != HKV_LOCAL;
+    return lb == HKV_GLOBAL ? 1 : 0;
+  };
+#pragma unroll 16
+  for (int i = tid; i < first; i += kBudgetThreads) count += tally(i);
+  count = __reduce_add_sync(0xFFFFFFFFu, (unsigned)count);
+  const int w0 = first + warp * PER;  // this warp's heads
+  int own = 0;
+#pragma unroll 16
+  for (int i = w0 + lane; i < w0 + PER; i += 32) own += i < n ? tally(i) : 0;
+  own = __reduce_add_sync(0xFFFFFFFFu, (unsigned)own);
+  if (lane == 0) {
+    s_before[warp] = count;
+    s_own[warp] = own;
+  }
+  const bool any_bad = __syncthreads_or(bad);
+  int g = 0;  // global heads before this warp's
+  for (int x = 0; x < NW; ++x) g += s_before[x] + (x < warp ? s_own[x] : 0);
+  const long long cl = (long long)C + w + P, cg = (long long)C + B_g + P;
+#pragma unroll 4
+  for (int i0 = w0; i0 < w0 + PER && i0 < n; i0 += 32) {
+    const int i = i0 + lane;
+    const bool gl = i < n && label[i] == HKV_GLOBAL;
+    const unsigned m = __ballot_sync(0xFFFFFFFFu, gl);
+    if (i < n) {
+      const int rank = g + __popc(m & ((1u << lane) - 1u));
+      budget[i] = gl ? B_g : w;
+      cap[i] = (int32_t)(gl ? cg : cl);
+      // (the CTA of the last head has seen every label: a bad one is
+      // reported as a state error)
+      off[i] = i == n - 1 && any_bad ? -1 : rank * cg + (i - rank) * cl;
+    }
+    g += __popc(m);
+  }
+}
+
 }  // namespace
 
 #ifdef HKV_UPD_TRACE
@@ -1103,6 +1212,9 @@ cudaError_t prepare_t(size_t smem) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(append_evict_kernel<D, T>,
                              cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(repack_kernel<D, T>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             100);
   return e;
 }
 
@@ -1151,27 +1263,22 @@ cudaError_t pdl_launch(void (*kernel)(KArgs...), int grid, int block, size_t sme
 }
 
 size_t smem_of(int max_len, int D, int P, int es) {
-  // the query ring / score stage; keys (8 B), positions (4 B), class/flag/
-  // rank (4 B) per row; q-bar; two 256-bin histograms
-  return ring_bytes(P, D, es, max_len) + (size_t)max_len * 16 + (size_t)D * 4 + 512 * 4 + 64;
-}
-
-// the longest segment a launch with `smem` bytes takes (the inverse of
-// smem_of, which grows with max_len)
-int max_len_of(size_t smem, int D, int P, int es) {
-  int lo = 0, hi = 1 << 20;
-  while (lo < hi) {
-    const int mid = lo + (hi - lo + 1) / 2;
-    if (smem_of(mid, D, P, es) <= smem) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
+  // the query ring / score stages; key words, positions (4 B each) and
+  // class/flag/rank (2 B) per row; q-bar; two 256-bin histograms
+  return ring_bytes(P, D, es, max_len) + (size_t)D * 4 + 512 * 4 + (size_t)max_len * 10 + 16;
 }
 
 }  // namespace
 
 size_t update_smem_bytes(int max_len, int D, int P, int dtype) {
   return smem_of(max_len, D, P, dtype == HKV_BF16 ? 2 : 4);
+}
+
+size_t update_limit_bytes(int max_len, int D, int P, int dtype) {
+  const size_t es = dtype == HKV_BF16 ? 2 : 4;
+  const size_t ring = (size_t)P * D * es;
+  const size_t rows = (size_t)(NT / 32) * stage_rows(max_len) * (D * es + 16);
+  return (ring > rows ? ring : rows) + (size_t)max_len * 16 + (size_t)D * 4 + 512 * 4 + 64;
 }
 
 cudaError_t update_prepare(int D, int dtype, size_t smem) {
@@ -1181,8 +1288,7 @@ cudaError_t update_prepare(int D, int dtype, size_t smem) {
 
 cudaError_t launch_append_evict(const CacheArgs &c, const MethodArgs &m, int layer_base,
                                 int nheads, const void *q, const void *k, const void *v, int D,
-                                int dtype, size_t smem, cudaStream_t s) {
-  const int max_len = max_len_of(smem, D, m.P, dtype == HKV_BF16 ? 2 : 4);
+                                int dtype, int max_len, size_t smem, cudaStream_t s) {
   HKV_DISPATCH(D, dtype,
                return pdl_launch(append_evict_kernel<kD, kT>, nheads, NT, smem, s, c, m,
                                  layer_base, q, k, v, max_len));
@@ -1190,8 +1296,7 @@ cudaError_t launch_append_evict(const CacheArgs &c, const MethodArgs &m, int lay
 }
 
 cudaError_t launch_evict(const CacheArgs &c, const MethodArgs &m, int layer_base, int nheads,
-                         int D, int dtype, size_t smem, cudaStream_t s) {
-  const int max_len = max_len_of(smem, D, m.P, dtype == HKV_BF16 ? 2 : 4);
+                         int D, int dtype, int max_len, size_t smem, cudaStream_t s) {
   HKV_DISPATCH(D, dtype,
                return pdl_launch(evict_kernel<kD, kT>, nheads, NT, smem, s, c, m, layer_base,
                                  max_len));
@@ -1199,9 +1304,8 @@ cudaError_t launch_evict(const CacheArgs &c, const MethodArgs &m, int layer_base
 }
 
 cudaError_t launch_repack(const CacheArgs &dense, const CacheArgs &ragged, const MethodArgs &m,
-                          int layer_base, int nheads, int D, int dtype, size_t smem,
+                          int layer_base, int nheads, int D, int dtype, int max_len, size_t smem,
                           cudaStream_t s) {
-  const int max_len = max_len_of(smem, D, m.P, dtype == HKV_BF16 ? 2 : 4);
   HKV_DISPATCH(D, dtype,
                return pdl_launch(repack_kernel<kD, kT>, nheads, NT, smem, s, dense, ragged, m,
                                  layer_base, max_len));
@@ -1230,11 +1334,11 @@ cudaError_t launch_identify(const CacheArgs &c, const MethodArgs &m, int layer_b
   const size_t smem = identify_smem_bytes(max_len, m.P, m.grid2d != 0, false);
   if (id_rows_in_flight(max_len, false) == 8) {
     HKV_DISPATCH(D, dtype,
-                 return pdl_launch(identify_kernel<kD, kT, 8>, nheads, NT, smem, s, c, m,
+                 return pdl_launch(identify_kernel<kD, kT, 8>, nheads, IT, smem, s, c, m,
                                    layer_base, q, label_out, nh_out, qscale, max_len));
   }
   HKV_DISPATCH(D, dtype,
-               return pdl_launch(identify_kernel<kD, kT, 2>, nheads, NT, smem, s, c, m, layer_base,
+               return pdl_launch(identify_kernel<kD, kT, 2>, nheads, IT, smem, s, c, m, layer_base,
                                  q, label_out, nh_out, qscale, max_len));
   return cudaErrorInvalidValue;
 }
@@ -1247,7 +1351,7 @@ cudaError_t launch_identify_multi(const CacheArgs &c, const MethodArgs &m, int l
   const bool q8 = id_qb(m.P) == 8, u4 = id_rows_in_flight(max_len, true) == 4;
 #define HKV_ID_MULTI(QB_, U_)                                                                  \
   HKV_DISPATCH(D, dtype,                                                                       \
-               return pdl_launch(identify_multi_kernel<kD, kT, QB_, U_>, nheads, NT, smem, s, c, \
+               return pdl_launch(identify_multi_kernel<kD, kT, QB_, U_>, nheads, IT, smem, s, c, \
                                  m, layer_base, label_out, nh_out, qscale, max_len))
   if (q8 && u4) HKV_ID_MULTI(8, 4);
   if (q8) HKV_ID_MULTI(8, 2);
@@ -1264,6 +1368,9 @@ size_t identify_smem_bytes(int max_len, int P, bool grid2d, bool multi) {
 
 cudaError_t launch_budgets(const uint8_t *label, int32_t *budget, int32_t *cap, int64_t *off,
                            int n, int C, int B_g, int w, int P, int group, cudaStream_t s) {
+  if (group == 0 && n <= kBudgetMost)
+    return pdl_launch(budgets_plain_kernel, (n + kBudgetHeads - 1) / kBudgetHeads, kBudgetThreads, 0,
+                      s, label, budget, cap, off, n, C, B_g, w, P);
   return pdl_launch(budgets_kernel, 1, 1024, 0, s, label, budget, cap, off, n, C, B_g, w, P, group);
 }
 

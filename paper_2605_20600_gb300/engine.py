@@ -131,8 +131,7 @@ class Engine:
                                                    self.off, self.stream())
         self.ragged = CacheBuffers(self.cfg, self.total_tokens, dev, qbuf=self.dense.qbuf,
                                    label=self.labels, off=self.off, cap=self.cap)
-        for layer in range(self.cfg.n_layers):
-            H.hkv_repack(self.cfg, self.dense.c, self.ragged.c, layer, self.stream())
+        H.hkv_repack_all(self.cfg, self.dense.c, self.ragged.c, self.stream())
         self.cache = self.ragged
 
     def release_dense(self) -> None:

@@ -1,4 +1,4 @@
-"""ctypes binding of the HeadKV C-ABI (include/hkv.h).
+"""ctypes binding of the HeadKV C-ABI (include/hkv.h, include/hkv_layers.h).
 
 Argument marshalling only: every function has the name of the C entry point
 it forwards to, accepts integers (device addresses) or objects with a
@@ -87,6 +87,7 @@ _SIGNATURES = {
     "hkv_allocate_budgets": ([POINTER(hkv_config), c_void_p, c_void_p, c_void_p, c_void_p,
                               POINTER(c_int64), c_void_p], c_int),
     "hkv_repack": ([POINTER(hkv_config), POINTER(hkv_cache), POINTER(hkv_cache), c_int, c_void_p], c_int),
+    "hkv_repack_all": ([POINTER(hkv_config), POINTER(hkv_cache), POINTER(hkv_cache), c_void_p], c_int),
     "hkv_check": ([POINTER(hkv_cache), c_void_p], c_int),
     "hkv_export_state": ([POINTER(hkv_config), POINTER(hkv_cache), c_int, c_void_p, c_void_p, c_void_p,
                           c_void_p, c_void_p, c_int64, POINTER(c_int64), c_void_p], c_int),
@@ -229,6 +230,10 @@ def hkv_allocate_budgets(cfg, label, budget, cap, off, stream=0) -> int:
 
 def hkv_repack(cfg, dense, ragged, layer, stream=0) -> None:
     _call("repack", ctypes.byref(cfg), ctypes.byref(dense), ctypes.byref(ragged), layer, stream)
+
+
+def hkv_repack_all(cfg, dense, ragged, stream=0) -> None:
+    _call("repack_all", ctypes.byref(cfg), ctypes.byref(dense), ctypes.byref(ragged), stream)
 
 
 def hkv_check(cache, stream=0) -> None:
