@@ -415,10 +415,10 @@ hkv_status hkv_decode_attention(const hkv_config *cfg, const hkv_cache *cache, i
 
 namespace {
 
-hkv_status decode_step(const char *name, const hkv_config *cfg, const hkv_cache *cache, int layer,
-                       const void *q, const void *k, const void *v, float *out,
-                       uint8_t *label_out, void *workspace, size_t ws_bytes, int flags,
-                       hkv_stream_t stream) {
+// the checks of a decode step of `layer` and its launch plan
+hkv_status step_checks(const char *name, const hkv_config *cfg, const hkv_cache *cache, int layer,
+                       const void *q, const void *k, const void *v, const float *out,
+                       const void *workspace, size_t ws_bytes, int flags, int *grid) {
   HKV_TRY(injected(name));
   HKV_TRY(hkv_validate_config(cfg));
   HKV_TRY(check_cache(cache));
@@ -426,8 +426,16 @@ hkv_status decode_step(const char *name, const hkv_config *cfg, const hkv_cache 
   if (!q || !k || !v || !out || !workspace) return HKV_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out) || !aligned16(workspace))
     return HKV_ERR_ALIGN;
-  if (ws_bytes < hkv_workspace_size(cfg)) return HKV_ERR_CAPACITY;
+  if (ws_bytes < ws_layout(cfg).total) return HKV_ERR_CAPACITY;
   if (flags & ~HKV_STEP_PREFETCH) return HKV_ERR_INVALID_ARG;
+  return one_launch_grid(cfg, true, grid);
+}
+
+// the launch, after those checks; grid 0: the two-kernel design
+hkv_status launch_checked_step(const hkv_config *cfg, const hkv_cache *cache, int layer,
+                               const void *q, const void *k, const void *v, float *out,
+                               uint8_t *label_out, void *workspace, int flags, int grid,
+                               hkv_stream_t stream) {
   AttnArgs a = attn_args(cfg, cache, layer, q, out, workspace);
   a.k_new = k;
   a.v_new = v;
@@ -435,13 +443,21 @@ hkv_status decode_step(const char *name, const hkv_config *cfg, const hkv_cache 
   a.label_out = label_out;
   a.w_loc = cfg->local_w;
   a.tau = (float)cfg->tau;
-  int grid = 0;
-  HKV_TRY(one_launch_grid(cfg, true, &grid));
   if (grid > 0)
     return cuda_status(launch_step(a, cfg->head_dim, cfg->dtype, grid, true, (cudaStream_t)stream));
   HKV_TRY(attn_grid(cfg, &grid));
   return cuda_status(launch_attention(a, cfg->head_dim, cfg->dtype, grid, true,
                                       label_out != nullptr, (cudaStream_t)stream));
+}
+
+hkv_status decode_step(const char *name, const hkv_config *cfg, const hkv_cache *cache, int layer,
+                       const void *q, const void *k, const void *v, float *out,
+                       uint8_t *label_out, void *workspace, size_t ws_bytes, int flags,
+                       hkv_stream_t stream) {
+  int grid = 0;
+  HKV_TRY(step_checks(name, cfg, cache, layer, q, k, v, out, workspace, ws_bytes, flags, &grid));
+  return launch_checked_step(cfg, cache, layer, q, k, v, out, label_out, workspace, flags, grid,
+                             stream);
 }
 
 }  // namespace
@@ -469,6 +485,28 @@ hkv_status hkv_decode_step_identify(const hkv_config *cfg, const hkv_cache *cach
   if (cfg && cfg->distance_mode != HKV_DIST_RASTER) return HKV_ERR_INVALID_ARG;
   return decode_step("decode_step_identify", cfg, cache, layer, q, k, v, out, label_out,
                      workspace, ws_bytes, flags, stream);
+}
+
+hkv_status hkv_decode_step_layers(const hkv_config *cfg, const hkv_cache *cache, const void *q,
+                                  const void *k, const void *v, float *out, uint8_t *label_out,
+                                  void *workspace, size_t ws_bytes, int flags,
+                                  hkv_stream_t stream) {
+  HKV_TRY(injected("decode_step_layers"));
+  if (label_out && cfg && cfg->distance_mode != HKV_DIST_RASTER) return HKV_ERR_INVALID_ARG;
+  int grid = 0;
+  HKV_TRY(step_checks(label_out ? "decode_step_identify" : "decode_step", cfg, cache, 0, q, k, v,
+                      out, workspace, ws_bytes, flags, &grid));
+  // (a layer's rows are a multiple of 128 bytes: every layer is as aligned as the first)
+  const size_t rows = (size_t)heads_per_layer(cfg) * cfg->head_dim;
+  const size_t in = rows * (cfg->dtype == HKV_BF16 ? 2 : 4);
+  for (int layer = 0; layer < cfg->n_layers; ++layer) {
+    const size_t at = layer * in;
+    HKV_TRY(launch_checked_step(cfg, cache, layer, static_cast<const char *>(q) + at,
+                                static_cast<const char *>(k) + at,
+                                static_cast<const char *>(v) + at, out + layer * rows, label_out,
+                                workspace, flags, grid, stream));
+  }
+  return HKV_OK;
 }
 
 namespace {

@@ -98,6 +98,14 @@ class Engine:
         H.hkv_decode_step(self.cfg, self.cache.c, layer, q, k, v, out, self.ws, self.ws_bytes,
                           flags, self.stream())
 
+    def step_layers(self, q, k, v, out, identify: bool = False) -> None:
+        """step (or step_identify) of every layer in order, in one call;
+        q, k, v, out: [L][S][H][D], contiguous."""
+        flags = H.HKV_STEP_PREFETCH if self.cfg.n_layers >= 2 else 0
+        H.hkv_decode_step_layers(self.cfg, self.cache.c, q, k, v, out,
+                                 self.labels if identify else None, self.ws, self.ws_bytes, flags,
+                                 self.stream())
+
     def update_due(self, t: int) -> bool:
         """Whether image token t's step starts with the periodic update
         (decided by the library, hkv_update_due)."""

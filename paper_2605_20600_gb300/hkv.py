@@ -75,6 +75,8 @@ _SIGNATURES = {
     "hkv_decode_step_identify": ([POINTER(hkv_config), POINTER(hkv_cache), c_int, c_void_p, c_void_p,
                                   c_void_p, c_void_p, c_void_p, c_void_p, c_size_t, c_int, c_void_p],
                                  c_int),
+    "hkv_decode_step_layers": ([POINTER(hkv_config), POINTER(hkv_cache), c_void_p, c_void_p, c_void_p,
+                                c_void_p, c_void_p, c_void_p, c_size_t, c_int, c_void_p], c_int),
     "hkv_decode_step_launches": ([POINTER(hkv_config)], c_int),
     "hkv_global_budget": ([c_int64, c_int64, c_int32, POINTER(c_int32)], c_int),
     "hkv_update_due": ([POINTER(hkv_config), c_int32, POINTER(c_int32)], c_int),
@@ -186,6 +188,14 @@ def hkv_decode_step(cfg, cache, layer, q, k, v, out, workspace, ws_bytes, flags=
                     stream=0) -> None:
     _call("decode_step", ctypes.byref(cfg), ctypes.byref(cache), layer, _p(q), _p(k), _p(v), _p(out),
           _p(workspace), ws_bytes, flags, stream)
+
+
+def hkv_decode_step_layers(cfg, cache, q, k, v, out, label_out, workspace, ws_bytes, flags=0,
+                           stream=0) -> None:
+    """hkv_decode_step (label_out None) or hkv_decode_step_identify of every
+    layer; q, k, v, out: [L][S][H][D]."""
+    _call("decode_step_layers", ctypes.byref(cfg), ctypes.byref(cache), _p(q), _p(k), _p(v), _p(out),
+          _p(label_out), _p(workspace), ws_bytes, flags, stream)
 
 
 def hkv_decode_step_launches(cfg) -> int:

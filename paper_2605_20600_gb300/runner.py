@@ -19,7 +19,7 @@ def generate(engine: Engine, provider, *, last_step: int | None = None, on_step=
     """Runs image tokens first_step..last_step (default N-1) for every layer.
 
     fused: hkv_evict_all (every layer in one launch) when the update is due,
-    then hkv_decode_step per layer; otherwise hkv_append_evict then
+    then hkv_decode_step of every layer in one call; otherwise hkv_append_evict then
     hkv_decode_attention per layer.
     on_step(t, out) receives out [L][S][H][D] (fp32, device) after step t.
     before_compress(engine) runs after grouping, before budgets and repack.
@@ -57,19 +57,21 @@ def generate(engine: Engine, provider, *, last_step: int | None = None, on_step=
         due = engine.update_due(t)
         if fused and due:
             engine.evict_all()       # every layer's buffer fills at the same token
-        for layer in range(L):
-            if fused:
-                if t == E - 1 and identify == "fused":
-                    engine.step_identify(layer, q[layer], k[layer], v[layer], out[layer])
-                else:
+        # a separate identification of a layer follows its own step
+        after = t == E - 1 and identify in ("separate", "multi")
+        if fused and not after:
+            engine.step_layers(q, k, v, out, identify=t == E - 1)
+        else:
+            for layer in range(L):
+                if fused:
                     engine.step(layer, q[layer], k[layer], v[layer], out[layer])
-            else:
-                engine.append(layer, q[layer], k[layer], v[layer])
-                engine.attend(layer, q[layer], out[layer])
-            if t == E - 1 and identify == "separate":
-                engine.identify(layer, q[layer])
-            elif t == E - 1 and identify == "multi":
-                engine.identify_multi(layer)
+                else:
+                    engine.append(layer, q[layer], k[layer], v[layer])
+                    engine.attend(layer, q[layer], out[layer])
+                if after and identify == "separate":
+                    engine.identify(layer, q[layer])
+                elif after:
+                    engine.identify_multi(layer)
         if on_step is not None:
             on_step(t, out)
         if t == E - 1:
