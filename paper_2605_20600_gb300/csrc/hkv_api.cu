@@ -231,14 +231,14 @@ hkv_status step_ctas(DeviceState *st, int D, int dtype, int *ctas) {
   return HKV_OK;
 }
 
-// The grid of a one-launch step (fused) or attention of this config, or 0
-// where the two-kernel design runs: a CTA's range could then hold more heads
+// The plan of a one-launch step (fused) or attention of this config, or no
+// CTAs where the two-kernel design runs: a CTA's range could then hold more heads
 // than the one-launch kernel's table (bounded from the longest segment the
 // config allows). Where it fits, one launch is the faster design on every
 // model shape measured. HKV_STEP_TWO_KERNELS in the environment forces the
 // two-kernel design (tests of both).
-hkv_status one_launch_grid(const hkv_config *cfg, bool fused, int *grid) {
-  *grid = 0;
+hkv_status one_launch_plan(const hkv_config *cfg, bool fused, StepPlan *plan) {
+  *plan = {0, false};
   if (getenv("HKV_STEP_TWO_KERNELS")) return HKV_OK;
   DeviceState *st;
   hkv_status s = device_state(&st);
@@ -248,7 +248,7 @@ hkv_status one_launch_grid(const hkv_config *cfg, bool fused, int *grid) {
   if (s != HKV_OK) return s;
   int full = st->sms.load(std::memory_order_acquire) * ctas;
   if (full > kAttnMaxGrid) full = kAttnMaxGrid;
-  *grid = step_grid(cfg->head_dim, cfg->dtype, heads_per_layer(cfg), max_segment(*cfg), full, fused);
+  *plan = step_plan(cfg->head_dim, cfg->dtype, heads_per_layer(cfg), max_segment(*cfg), full, fused);
   return HKV_OK;
 }
 
@@ -404,10 +404,11 @@ hkv_status hkv_decode_attention(const hkv_config *cfg, const hkv_cache *cache, i
   if (!aligned16(q) || !aligned16(out) || !aligned16(workspace)) return HKV_ERR_ALIGN;
   if (ws_bytes < hkv_workspace_size(cfg)) return HKV_ERR_CAPACITY;
   const AttnArgs a = attn_args(cfg, cache, layer, q, out, workspace);
+  StepPlan plan;
+  HKV_TRY(one_launch_plan(cfg, false, &plan));
+  if (plan.grid > 0)
+    return cuda_status(launch_step(a, cfg->head_dim, cfg->dtype, plan, false, (cudaStream_t)stream));
   int grid = 0;
-  HKV_TRY(one_launch_grid(cfg, false, &grid));
-  if (grid > 0)
-    return cuda_status(launch_step(a, cfg->head_dim, cfg->dtype, grid, false, (cudaStream_t)stream));
   HKV_TRY(attn_grid(cfg, &grid));
   return cuda_status(
       launch_attention(a, cfg->head_dim, cfg->dtype, grid, false, false, (cudaStream_t)stream));
@@ -418,7 +419,7 @@ namespace {
 // the checks of a decode step of `layer` and its launch plan
 hkv_status step_checks(const char *name, const hkv_config *cfg, const hkv_cache *cache, int layer,
                        const void *q, const void *k, const void *v, const float *out,
-                       const void *workspace, size_t ws_bytes, int flags, int *grid) {
+                       const void *workspace, size_t ws_bytes, int flags, StepPlan *plan) {
   HKV_TRY(injected(name));
   HKV_TRY(hkv_validate_config(cfg));
   HKV_TRY(check_cache(cache));
@@ -428,13 +429,13 @@ hkv_status step_checks(const char *name, const hkv_config *cfg, const hkv_cache 
     return HKV_ERR_ALIGN;
   if (ws_bytes < ws_layout(cfg).total) return HKV_ERR_CAPACITY;
   if (flags & ~HKV_STEP_PREFETCH) return HKV_ERR_INVALID_ARG;
-  return one_launch_grid(cfg, true, grid);
+  return one_launch_plan(cfg, true, plan);
 }
 
-// the launch, after those checks; grid 0: the two-kernel design
+// the launch, after those checks; no CTAs planned: the two-kernel design
 hkv_status launch_checked_step(const hkv_config *cfg, const hkv_cache *cache, int layer,
                                const void *q, const void *k, const void *v, float *out,
-                               uint8_t *label_out, void *workspace, int flags, int grid,
+                               uint8_t *label_out, void *workspace, int flags, StepPlan plan,
                                hkv_stream_t stream) {
   AttnArgs a = attn_args(cfg, cache, layer, q, out, workspace);
   a.k_new = k;
@@ -443,8 +444,9 @@ hkv_status launch_checked_step(const hkv_config *cfg, const hkv_cache *cache, in
   a.label_out = label_out;
   a.w_loc = cfg->local_w;
   a.tau = (float)cfg->tau;
-  if (grid > 0)
-    return cuda_status(launch_step(a, cfg->head_dim, cfg->dtype, grid, true, (cudaStream_t)stream));
+  if (plan.grid > 0)
+    return cuda_status(launch_step(a, cfg->head_dim, cfg->dtype, plan, true, (cudaStream_t)stream));
+  int grid = 0;
   HKV_TRY(attn_grid(cfg, &grid));
   return cuda_status(launch_attention(a, cfg->head_dim, cfg->dtype, grid, true,
                                       label_out != nullptr, (cudaStream_t)stream));
@@ -454,9 +456,9 @@ hkv_status decode_step(const char *name, const hkv_config *cfg, const hkv_cache 
                        const void *q, const void *k, const void *v, float *out,
                        uint8_t *label_out, void *workspace, size_t ws_bytes, int flags,
                        hkv_stream_t stream) {
-  int grid = 0;
-  HKV_TRY(step_checks(name, cfg, cache, layer, q, k, v, out, workspace, ws_bytes, flags, &grid));
-  return launch_checked_step(cfg, cache, layer, q, k, v, out, label_out, workspace, flags, grid,
+  StepPlan plan;
+  HKV_TRY(step_checks(name, cfg, cache, layer, q, k, v, out, workspace, ws_bytes, flags, &plan));
+  return launch_checked_step(cfg, cache, layer, q, k, v, out, label_out, workspace, flags, plan,
                              stream);
 }
 
@@ -471,9 +473,9 @@ hkv_status hkv_decode_step(const hkv_config *cfg, const hkv_cache *cache, int la
 
 int hkv_decode_step_launches(const hkv_config *cfg) {
   if (hkv_validate_config(cfg) != HKV_OK) return 0;
-  int grid = 0;
-  if (one_launch_grid(cfg, true, &grid) != HKV_OK) return 0;
-  return grid > 0 ? 1 : 2;
+  StepPlan plan;
+  if (one_launch_plan(cfg, true, &plan) != HKV_OK) return 0;
+  return plan.grid > 0 ? 1 : 2;
 }
 
 hkv_status hkv_decode_step_identify(const hkv_config *cfg, const hkv_cache *cache, int layer,
@@ -493,9 +495,9 @@ hkv_status hkv_decode_step_layers(const hkv_config *cfg, const hkv_cache *cache,
                                   hkv_stream_t stream) {
   HKV_TRY(injected("decode_step_layers"));
   if (label_out && cfg && cfg->distance_mode != HKV_DIST_RASTER) return HKV_ERR_INVALID_ARG;
-  int grid = 0;
+  StepPlan plan;
   HKV_TRY(step_checks(label_out ? "decode_step_identify" : "decode_step", cfg, cache, 0, q, k, v,
-                      out, workspace, ws_bytes, flags, &grid));
+                      out, workspace, ws_bytes, flags, &plan));
   // (a layer's rows are a multiple of 128 bytes: every layer is as aligned as the first)
   const size_t rows = (size_t)heads_per_layer(cfg) * cfg->head_dim;
   const size_t in = rows * (cfg->dtype == HKV_BF16 ? 2 : 4);
@@ -504,7 +506,7 @@ hkv_status hkv_decode_step_layers(const hkv_config *cfg, const hkv_cache *cache,
     HKV_TRY(launch_checked_step(cfg, cache, layer, static_cast<const char *>(q) + at,
                                 static_cast<const char *>(k) + at,
                                 static_cast<const char *>(v) + at, out + layer * rows, label_out,
-                                workspace, flags, grid, stream));
+                                workspace, flags, plan, stream));
   }
   return HKV_OK;
 }

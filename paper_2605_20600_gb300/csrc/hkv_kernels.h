@@ -120,15 +120,21 @@ size_t attention_smem_bytes(int D, int dtype);
 constexpr int kStepActivePerSm = HKV_STEP_ACTIVE_PER_SM;
 
 cudaError_t step_prepare(int D, int dtype, int *ctas_per_sm);
-// CTAs of a one-launch step (fused) or attention (not fused) over nheads
-// heads of at most max_rows rows, out of a grid of `full`; 0: a range could
-// hold more heads than the kernel's table, so the two-kernel design runs
-int step_grid(int D, int dtype, int nheads, int max_rows, int full, bool fused);
+// The launch of a one-launch step (fused) or attention (not fused) over nheads
+// heads of at most max_rows rows, out of a grid of `full`: its CTAs, and
+// whether it takes the shape for heads that fit one stage. 0 CTAs: a range
+// could hold more heads than the kernel's table, so the two-kernel design runs.
+struct StepPlan {
+  int grid;
+  bool whole;
+};
+StepPlan step_plan(int D, int dtype, int nheads, int max_rows, int full, bool fused);
 // one layer in one launch: the decode step (append + attention, merges of
 // split heads and counters in the same kernel), with the head types decided
-// where a.label_out is set, or attention alone (not fused); `grid` CTAs, at
-// most kAttnMaxGrid and at most what is resident at once
-cudaError_t launch_step(const AttnArgs &a, int D, int dtype, int grid, bool fused, cudaStream_t s);
+// where a.label_out is set, or attention alone (not fused); at most
+// kAttnMaxGrid CTAs and at most what is resident at once
+cudaError_t launch_step(const AttnArgs &a, int D, int dtype, StepPlan plan, bool fused,
+                        cudaStream_t s);
 cudaError_t attention_prepare(int D, int dtype, int *ctas_per_sm);
 // launches the attention kernel on `grid` CTAs (at most kAttnMaxGrid) and the
 // finishing kernel behind it; identify (fused only): also the Step 2 label of

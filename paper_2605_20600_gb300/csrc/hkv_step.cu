@@ -137,34 +137,41 @@ constexpr int step_cw(int D, int es) {
   return es == 4 ? 8 : D == 64 ? HKV_STEP_CW_D64 : HKV_STEP_CW_D128;
 }
 
-template <int D, typename T>
-using StepTile = TileShape<D, T, step_cw(D, sizeof(T)),
-                           D == 64 ? HKV_STEP_TILE_BYTES_D64 : HKV_STEP_TILE_BYTES_D128,
-                           D == 64 ? HKV_STEP_STAGES_D64 : HKV_STEP_STAGES_D128,
-                           D == 64 ? HKV_STEP_PRE_D64 : HKV_STEP_PRE_D128>;
+// Heads of at most this many grains (96 KB of K and V) are not split when
+// every head can have a CTA of its own: the exchange of partial results
+// costs more than the tiles it saves.
+constexpr int kAlignedGrains = 12;
 
-template <int D, typename T>
-struct StepShape : StepTile<D, T> {
-  using Tile = StepTile<D, T>;
+constexpr int step_grain(int row_bytes) { return row_bytes == 512 ? 8 : 16; }  // rows
+
+// SHORT: the shape for layers whose every head fits kAlignedGrains: one stage
+// that holds a whole head, so that the consumers pass over it once.
+template <int D, typename T, bool SHORT>
+using StepTile = TileShape<
+    D, T, step_cw(D, sizeof(T)),
+    SHORT     ? kAlignedGrains * step_grain(D * sizeof(T)) * D * (int)sizeof(T)
+    : D == 64 ? HKV_STEP_TILE_BYTES_D64
+              : HKV_STEP_TILE_BYTES_D128,
+    SHORT ? 1 : D == 64 ? HKV_STEP_STAGES_D64 : HKV_STEP_STAGES_D128,
+    SHORT ? 1 : D == 64 ? HKV_STEP_PRE_D64 : HKV_STEP_PRE_D128>;
+
+template <int D, typename T, bool SHORT = false>
+struct StepShape : StepTile<D, T, SHORT> {
+  using Tile = StepTile<D, T, SHORT>;
   // states a segment hands over: one per consumer warp, or (fp32) per row group
   static constexpr int kNST = sizeof(T) == 2 ? Tile::kCW : Tile::kCW * Tile::kRPW;
   // The split counts in grains of kGR rows (4 or 8 KB of K and V). A head of
   // g grains takes g + 1 slots, at least kMinCost: the extra one stands for
   // what a head costs beyond its rows (a hand-over, a partial tile), and the
   // minimum bounds the heads of a range (step_max_heads).
-  static constexpr int kGR = Tile::kRB == 512 ? 8 : 16;
-  static constexpr int kMinCost = Tile::kRB == 128 ? 5 : Tile::kTT / kGR > 3 ? 3 : 2;
-  static constexpr int kMinChunk = 2 * Tile::kTT / kGR;  // fewest slots per CTA range
+  static constexpr int kGR = step_grain(Tile::kRB);
+  static constexpr int kMinCost = Tile::kRB == 128 ? 5 : 3;
+  static constexpr int kMinChunk = SHORT ? kAlignedGrains : 2 * Tile::kTT / kGR;  // fewest slots per CTA range
   __host__ __device__ static constexpr int grains(int rows) {
     return (int)(((unsigned)rows + kGR - 1) / kGR);
   }
   __host__ __device__ static constexpr int cost(int g) { return g + 1 > kMinCost ? g + 1 : kMinCost; }
 };
-
-// Heads of at most this many grains (96 KB of K and V) are not split when
-// every head can have a CTA of its own: the exchange of partial results
-// costs more than the tiles it saves.
-constexpr int kAlignedGrains = 12;
 
 // A boundary between ranges that falls within 1/kSnapDiv of a range of a
 // head's first or last row moves there.
@@ -264,10 +271,10 @@ __host__ __device__ constexpr int step_threads() {
 // the pass (Sec. 4, Step 2), or attention alone (no append, no counters).
 enum StepMode { kModeStep = 0, kModeIdentify = 1, kModeAttend = 2 };
 
-template <int D, typename T, int MODE>
+template <int D, typename T, int MODE, bool SHORT>
 __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM)
     step_kernel(const AttnArgs p) {
-  using S = StepShape<D, T>;
+  using S = StepShape<D, T, SHORT>;
   constexpr bool FUSED = MODE != kModeAttend, IDENT = MODE == kModeIdentify;
   constexpr int kCW = S::kCW, kThr = step_threads<D, T>(), NW = kThr / 32;
   constexpr int LPR = S::kLPR, EPL = S::kEPL, RPW = S::kRPW, TT = S::kTT;
@@ -285,7 +292,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   __shared__ uint64_t full[NS], empty[NS];
   __shared__ uint64_t epi_full[2], epi_free[2];  // two hand-over buffers
   __shared__ __align__(16) float red_acc[2][NST][D];
-  __shared__ float red_m[2][NST], red_l[2][NST], red_r[IDENT ? 2 : 1][IDENT ? NST : 1];
+  __shared__ __align__(16) float red_m[2][NST], red_l[2][NST], red_r[IDENT ? 2 : 1][IDENT ? NST : 1];
   __shared__ TileMeta meta[NS];
   __shared__ SegMeta seg[2];
   __shared__ StepTable<kThr> tab;
@@ -775,7 +782,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         issue_old(st_i);
         issue_extra(st_i);
         ++armed;
-        if (++st_i == NS) {
+        if (NS == 1 || ++st_i == NS) {
           st_i = 0;
           st_ph ^= 1u;
         }
@@ -877,6 +884,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     constexpr int NJ = MMA ? D / 32 : 1;          // 16-byte pieces of a row per lane
     constexpr int NB = MMA ? TT / (kCW * 8) : 1;  // 8-row blocks per warp and tile
     constexpr int VS = MMA ? 8 / RPW : 1;         // row steps of a block's V
+    constexpr bool kEarlyV = NB * VS <= 8;        // V is loaded with K while registers last
     static_assert(!MMA || TT % (kCW * 8) == 0, "blocks of 8 rows");
     uint32_t qb[NJ][2];
     typename M::Q q;
@@ -924,7 +932,14 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
           // g + 8. The even columns of B hold the query's channels of x and
           // z, the odd ones those of y and w, so the row's dot product is
           // C[g][even] + C[g + 8][odd]: c[0] + c[3] in all lanes of quad g.
-          uint4 vf[NB][VS];
+          uint4 vf[kEarlyV ? NB : 1][VS];
+          // V: whole rows by groups of lanes, RPW rows a step; rows past the
+          // tile's are not read (they may hold anything)
+          auto load_v = [&](int rb, int st) {
+            return rb + st * RPW + grp < nr
+                       ? *reinterpret_cast<const uint4 *>(Vs + (rb + st * RPW + grp) * RB + col * 16)
+                       : make_uint4(0u, 0u, 0u, 0u);
+          };
           float dots[NB];
           float mt = -INFINITY;
 #pragma unroll
@@ -936,14 +951,10 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
               uint4 kf[NJ];
 #pragma unroll
               for (int j = 0; j < NJ; ++j) kf[j] = *reinterpret_cast<const uint4 *>(kr + j * 64);
-              // V: whole rows by groups of lanes, RPW rows a step; rows past
-              // the tile's are not read (they may hold anything)
-              const unsigned char *vr = Vs + (rb + grp) * RB + col * 16;
+              if (kEarlyV) {
 #pragma unroll
-              for (int st = 0; st < VS; ++st)
-                vf[b8][st] = rb + st * RPW + grp < nr
-                                 ? *reinterpret_cast<const uint4 *>(vr + st * RPW * RB)
-                                 : make_uint4(0u, 0u, 0u, 0u);
+                for (int st = 0; st < VS; ++st) vf[kEarlyV ? b8 : 0][st] = load_v(rb, st);
+              }
               float c[2][4] = {};
 #pragma unroll
               for (int j = 0; j < NJ; ++j) mma_bf16(c[j & 1], kf[j], qb[j][0], qb[j][1]);
@@ -971,7 +982,8 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
                 if (IDENT && rb + (lane >> 2) >= mt4.recent0) lr += pr;
 #pragma unroll
                 for (int st = 0; st < VS; ++st)
-                  M::add_v(acc, vf[b8][st], __shfl_sync(0xFFFFFFFFu, pr, (st * RPW + grp) * 4));
+                  M::add_v(acc, kEarlyV ? vf[kEarlyV ? b8 : 0][st] : load_v(rb, st),
+                           __shfl_sync(0xFFFFFFFFu, pr, (st * RPW + grp) * 4));
               }
             }
           }
@@ -1011,9 +1023,9 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         }
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[stage]);
+      mbar_arrive_if(&empty[stage], lane == 0);
       if (flags & kLast) hand_over(mt4.h, flags);  // last tile of this head in this piece
-      if (++stage == NS) {
+      if (NS == 1 || ++stage == NS) {
         stage = 0;
         fph ^= 1u;
       }
@@ -1040,29 +1052,25 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       const SegMeta sg = seg[bb];
       if (sg.h < 0) break;
       const int h = sg.h;
-      // lane s < NST weighs state s
-      const float ms = lane < NST ? red_m[bb][lane] : -INFINITY;
-      float mx = ms;
+      // every lane weighs every state itself: no exchange between lanes
+      float ws[NST];
 #pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-      const float ws = ms == -INFINITY ? 0.f : exp2f(ms - mx);
-      float L = lane < NST ? red_l[bb][lane] * ws : 0.f;
-      float LR = IDENT && lane < NST ? red_r[bb][lane] * ws : 0.f;
+      for (int si = 0; si < NST; ++si) ws[si] = red_m[bb][si];
+      float mx = ws[0];
 #pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) {
-        L += __shfl_xor_sync(0xFFFFFFFFu, L, o);
-        if (IDENT) LR += __shfl_xor_sync(0xFFFFFFFFu, LR, o);
-      }
-      float A[CPL];
+      for (int si = 1; si < NST; ++si) mx = fmaxf(mx, ws[si]);
+      float L = 0.f, LR = 0.f, A[CPL];
 #pragma unroll
       for (int c = 0; c < CPL; ++c) A[c] = 0.f;
 #pragma unroll
       for (int si = 0; si < NST; ++si) {
-        const float sw = __shfl_sync(0xFFFFFFFFu, ws, si);
+        ws[si] = ws[si] == -INFINITY ? 0.f : exp2f(ws[si] - mx);
+        L = fmaf(red_l[bb][si], ws[si], L);
+        if (IDENT) LR = fmaf(red_r[bb][si], ws[si], LR);
         float r[CPL];
         V::lds(&red_acc[bb][si][CPL * lane], r);
 #pragma unroll
-        for (int c = 0; c < CPL; ++c) A[c] = fmaf(r[c], sw, A[c]);
+        for (int c = 0; c < CPL; ++c) A[c] = fmaf(r[c], ws[si], A[c]);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&epi_free[bb]);  // the consumers may reuse the buffer
@@ -1319,19 +1327,19 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   }
 }
 
-template <int D, typename T>
+template <int D, typename T, bool SHORT>
 size_t step_smem() {
-  return (size_t)StepShape<D, T>::kNS * StepShape<D, T>::kStageBytes;
+  return (size_t)StepShape<D, T, SHORT>::kNS * StepShape<D, T, SHORT>::kStageBytes;
 }
 
-template <int D, typename T, int MODE>
+template <int D, typename T, int MODE, bool SHORT>
 cudaError_t step_prepare_m(int *ctas) {
-  const size_t smem = step_smem<D, T>();
-  cudaError_t e = cudaFuncSetAttribute(step_kernel<D, T, MODE>,
+  const size_t smem = step_smem<D, T, SHORT>();
+  cudaError_t e = cudaFuncSetAttribute(step_kernel<D, T, MODE, SHORT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int n = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_kernel<D, T, MODE>,
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_kernel<D, T, MODE, SHORT>,
                                                     step_threads<D, T>(), smem);
   if (n < *ctas) *ctas = n;
   return e;
@@ -1340,20 +1348,20 @@ cudaError_t step_prepare_m(int *ctas) {
 template <int D, typename T>
 cudaError_t step_prepare_t(int *ctas) {
   *ctas = kStepActivePerSm;
-  cudaError_t e = step_prepare_m<D, T, kModeStep>(ctas);
-  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeIdentify>(ctas);
-  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeAttend>(ctas);
+  cudaError_t e = step_prepare_m<D, T, kModeStep, false>(ctas);
+  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeStep, true>(ctas);
+  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeIdentify, false>(ctas);
+  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeAttend, false>(ctas);
   return e;
 }
 
-template <int D, typename T>
-cudaError_t step_launch_t(AttnArgs a, int grid, bool fused, cudaStream_t s) {
-  a.grid_recip = (uint32_t)(((1ull << 32) + grid - 1) / grid);  // (not used for a grid of one)
+template <int D, typename T, int MODE, bool SHORT>
+cudaError_t step_launch_m(const AttnArgs &a, int grid, cudaStream_t s) {
   static const bool pdl = getenv("HKV_NO_PDL") == nullptr;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(step_threads<D, T>());
-  cfg.dynamicSmemBytes = step_smem<D, T>();
+  cfg.dynamicSmemBytes = step_smem<D, T, SHORT>();
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   int na = 0;
@@ -1364,25 +1372,31 @@ cudaError_t step_launch_t(AttnArgs a, int grid, bool fused, cudaStream_t s) {
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  if (!fused) return cudaLaunchKernelEx(&cfg, step_kernel<D, T, kModeAttend>, a);
-  if (a.label_out) return cudaLaunchKernelEx(&cfg, step_kernel<D, T, kModeIdentify>, a);
-  return cudaLaunchKernelEx(&cfg, step_kernel<D, T, kModeStep>, a);
+  return cudaLaunchKernelEx(&cfg, step_kernel<D, T, MODE, SHORT>, a);
 }
 
-// The CTAs a layer of n heads gets out of a full grid, and whether the
-// launch fits: see launch_step.
 template <int D, typename T>
-int step_grid_t(long long n, long long max_rows, int full, bool fused) {
+cudaError_t step_launch_t(AttnArgs a, int grid, bool fused, bool whole, cudaStream_t s) {
+  a.grid_recip = (uint32_t)(((1ull << 32) + grid - 1) / grid);  // (not used for a grid of one)
+  if (!fused) return step_launch_m<D, T, kModeAttend, false>(a, grid, s);
+  if (a.label_out) return step_launch_m<D, T, kModeIdentify, false>(a, grid, s);
+  return whole ? step_launch_m<D, T, kModeStep, true>(a, grid, s)
+               : step_launch_m<D, T, kModeStep, false>(a, grid, s);
+}
+
+// The CTAs a layer of n heads gets out of a full grid: see step_plan.
+template <int D, typename T>
+StepPlan step_plan_t(long long n, long long max_rows, int full, bool fused) {
   using S = StepShape<D, T>;
   const long long g = (max_rows + S::kGR - 1) / S::kGR;
   const long long total = n * (g + 1 > S::kMinCost ? g + 1 : S::kMinCost);
   long long chunk = (total + full - 1) / full;
   if (chunk < S::kMinChunk) chunk = S::kMinChunk;
-  if (n > kStepTable && chunk / S::kMinCost + 2 > kStepTable) return 0;
-  if (!fused) return full;
-  if (n <= full && n <= kStepTable && g <= kAlignedGrains) return (int)n;
+  if (n > kStepTable && chunk / S::kMinCost + 2 > kStepTable) return {0, false};
+  if (!fused) return {full, false};
+  if (n <= full && n <= kStepTable && g <= kAlignedGrains) return {(int)n, true};
   const long long need = (total + S::kMinChunk - 1) / S::kMinChunk;
-  return need < full ? (int)need : full;
+  return {need < full ? (int)need : full, false};
 }
 
 }  // namespace
@@ -1393,12 +1407,12 @@ extern "C" int hkv_debug_set_step_trace(unsigned long long *buf) {
 }
 #endif
 
-int step_grid(int D, int dtype, int nheads, int max_rows, int full, bool fused) {
+StepPlan step_plan(int D, int dtype, int nheads, int max_rows, int full, bool fused) {
   if (dtype == HKV_BF16)
-    return D == 64 ? step_grid_t<64, __nv_bfloat16>(nheads, max_rows, full, fused)
-                   : step_grid_t<128, __nv_bfloat16>(nheads, max_rows, full, fused);
-  return D == 64 ? step_grid_t<64, float>(nheads, max_rows, full, fused)
-                 : step_grid_t<128, float>(nheads, max_rows, full, fused);
+    return D == 64 ? step_plan_t<64, __nv_bfloat16>(nheads, max_rows, full, fused)
+                   : step_plan_t<128, __nv_bfloat16>(nheads, max_rows, full, fused);
+  return D == 64 ? step_plan_t<64, float>(nheads, max_rows, full, fused)
+                 : step_plan_t<128, float>(nheads, max_rows, full, fused);
 }
 
 cudaError_t step_prepare(int D, int dtype, int *ctas) {
@@ -1407,13 +1421,15 @@ cudaError_t step_prepare(int D, int dtype, int *ctas) {
   return D == 64 ? step_prepare_t<64, float>(ctas) : step_prepare_t<128, float>(ctas);
 }
 
-cudaError_t launch_step(const AttnArgs &a, int D, int dtype, int grid, bool fused, cudaStream_t s) {
+cudaError_t launch_step(const AttnArgs &a, int D, int dtype, StepPlan plan, bool fused,
+                        cudaStream_t s) {
+  const int grid = plan.grid;
   if (grid < 1 || grid > kAttnMaxGrid) return cudaErrorInvalidValue;
   if (dtype == HKV_BF16)
-    return D == 64 ? step_launch_t<64, __nv_bfloat16>(a, grid, fused, s)
-                   : step_launch_t<128, __nv_bfloat16>(a, grid, fused, s);
-  return D == 64 ? step_launch_t<64, float>(a, grid, fused, s)
-                 : step_launch_t<128, float>(a, grid, fused, s);
+    return D == 64 ? step_launch_t<64, __nv_bfloat16>(a, grid, fused, plan.whole, s)
+                   : step_launch_t<128, __nv_bfloat16>(a, grid, fused, plan.whole, s);
+  return D == 64 ? step_launch_t<64, float>(a, grid, fused, plan.whole, s)
+                 : step_launch_t<128, float>(a, grid, fused, plan.whole, s);
 }
 
 }  // namespace hkv
