@@ -734,6 +734,8 @@ __global__ void init_dense_kernel(const CacheArgs c, int n, int seg) {
 // with one; segments of 101-164 tokens go best with 2, where more loads in
 // flight cost registers and resident CTAs.
 constexpr int kIdLongSegment = 512;
+// stages of the single-query kernel's keys for such segments
+constexpr int kIdStageBytes = 32768, kIdStages = 3;
 __host__ __device__ constexpr int id_rows_in_flight(int max_len, bool multi) {
   return max_len >= kIdLongSegment ? (multi ? 4 : 8) : 2;
 }
@@ -747,6 +749,8 @@ __host__ __device__ constexpr size_t id_order_offset(size_t floats) {
 __host__ __device__ constexpr size_t id_smem(size_t floats, int max_len, bool grid2d) {
   return grid2d ? id_order_offset(floats) + (size_t)max_len * 12 : floats * 4;
 }
+__host__ __device__ constexpr size_t id_stage_at(size_t smem) { return (smem + 127) / 128 * 128; }
+constexpr size_t kIdMostSmem = 226 * 1024;  // dynamic, beside the kernels' static part
 
 // The count order of the grid-distance variant of Step 2: perm[j] = the row
 // of the j-th token counted. Image tokens by squared grid distance from image
@@ -785,12 +789,21 @@ __device__ void grid_count_order(const int32_t *pos, int len, int C, int row_len
 // One CTA per head, one and a half on an SM for 256 heads: beside the keys'
 // bytes it is a chain of phases, so each phase is one block barrier: every
 // warp combines the warps' maxima, sums and scan totals itself, in the order
-// in which one warp did (the counts depend on it). 12.1 -> 11.8 us for 256
-// heads of 628 tokens (6.1 at the measured bandwidth); 512 threads 12.3.
-template <int D, typename T, int U>
+// in which one warp did (the counts depend on it). 256 heads of 628 tokens
+// (6.1 us at the measured bandwidth): 12.1 us; with those barriers 11.8, with
+// the staged keys below 10.4 (512 threads without them 12.3).
+//
+// The logits: short segments (STAGED = false) load U row steps at a time into
+// registers; longer ones come through kIdStages stages of 32 KB filled by
+// bulk copies, so that a head's keys are on their way before the first
+// product, and a warp takes eight row steps of a stage at once: pairs of rows
+// share FMAs, and the eight sums are exchanged by halves (8 shuffles instead
+// of 32). Products and sums are the same operations in the same order.
+template <int D, typename T, int U, bool STAGED>
 __global__ void __launch_bounds__(IT)
     identify_kernel(const CacheArgs c, const MethodArgs m, int layer_base, const void *q,
-                    uint8_t *label_out, int32_t *nh_out, float qscale, int max_len) {
+                    uint8_t *label_out, int32_t *nh_out, float qscale, int max_len,
+                    int stage_at) {
   constexpr int RB = D * (int)sizeof(T);
   constexpr int EPL = Elem<T>::kPerPiece;
   constexpr int LPR = RB / 16;
@@ -799,6 +812,7 @@ __global__ void __launch_bounds__(IT)
   extern __shared__ float e[];
   __shared__ float s_max[NW], s_sum[NW], s_tot[2][NW];
   __shared__ int s_nh;
+  __shared__ uint64_t s_full[kIdStages], s_empty[kIdStages];
   pdl_wait();
   pdl_launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -826,27 +840,99 @@ __global__ void __launch_bounds__(IT)
 #pragma unroll
   for (int x = 0; x < EPL; ++x) qf[x] *= qscale;
   const unsigned char *K = static_cast<const unsigned char *>(c.K) + off * RB;
-  // logits (log2 units); U row steps load before any is used
+  // logits (log2 units)
   float mx = -INFINITY;
-  for (int r0 = warp * RPW; r0 < len; r0 += U * NW * RPW) {
-    uint4 kr[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int r = r0 + u * NW * RPW + grp;
-      kr[u] = r < len ? *reinterpret_cast<const uint4 *>(K + (size_t)r * RB + col * 16)
-                      : make_uint4(0u, 0u, 0u, 0u);
+  if constexpr (STAGED) {
+    constexpr int ROWS = kIdStageBytes / RB;  // of a stage: eight row steps of every warp
+    static_assert(ROWS == 8 * NW * RPW, "a stage is eight row steps");
+    unsigned char *stage = reinterpret_cast<unsigned char *>(e) + stage_at;
+    const int fills = (len + ROWS - 1) / ROWS;
+    auto fill = [&](int f) {  // thread 0
+      const int rows = len - f * ROWS < ROWS ? len - f * ROWS : ROWS;
+      const uint32_t bytes = (uint32_t)rows * RB;
+      mbar_arrive_expect_tx(&s_full[f % kIdStages], bytes);
+      bulk_g2s(stage + (f % kIdStages) * kIdStageBytes, K + (size_t)f * ROWS * RB, bytes,
+               &s_full[f % kIdStages]);
+    };
+    if (tid == 0) {
+      for (int x = 0; x < kIdStages; ++x) {
+        mbar_init(&s_full[x], 1);
+        mbar_init(&s_empty[x], NW);
+      }
+      fence_barrier_init();
+      for (int f = 0; f < fills && f < kIdStages; ++f) fill(f);
     }
+    __syncthreads();
+    float2 q2[EPL];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int r = r0 + u * NW * RPW + grp;
-      float kf[EPL];
-      Elem<T>::unpack(kr[u], kf);
-      float dot = 0.f;
+    for (int x = 0; x < EPL; ++x) q2[x] = make_float2(qf[x], qf[x]);
+#pragma unroll 1
+    for (int f = 0; f < fills; ++f) {
+      const int sg = f % kIdStages;
+      if (!mbar_wait(&s_full[sg], (uint32_t)(f / kIdStages) & 1u) && tid == 0)
+        set_err(c.err, HKV_ERR_TIMEOUT);
+      const unsigned char *src = stage + sg * kIdStageBytes + (warp * RPW + grp) * RB + col * 16;
+      float v[8];
 #pragma unroll
-      for (int x = 0; x < EPL; ++x) dot = fmaf(qf[x], kf[x], dot);
+      for (int u = 0; u < 8; u += 2) {
+        float ka[EPL], kb[EPL];
+        Elem<T>::unpack(*reinterpret_cast<const uint4 *>(src + u * NW * RPW * RB), ka);
+        Elem<T>::unpack(*reinterpret_cast<const uint4 *>(src + (u + 1) * NW * RPW * RB), kb);
+        float2 dot = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int o = LPR / 2; o >= 1; o >>= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, o);
-      if (r < len && col == 0) e[r] = dot;
+        for (int x = 0; x < EPL; ++x) dot = __ffma2_rn(q2[x], make_float2(ka[x], kb[x]), dot);
+        v[u] = dot.x;
+        v[u + 1] = dot.y;
+      }
+      __syncwarp();
+      mbar_arrive_if(&s_empty[sg], lane == 0);
+      // the sum over a row's lanes: halves of the values change hands at the
+      // first three levels, so lane bits choose the row step that is left
+      int step = 0;
+      int o = LPR / 2;
+#pragma unroll
+      for (int n = 4; n >= 1; n >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int x = 0; x < n; ++x) {
+          const float give = up ? v[x] : v[x + n], keep = up ? v[x + n] : v[x];
+          v[x] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+        }
+        step += up ? n : 0;
+      }
+#pragma unroll
+      for (int l = LPR / 16; l >= 1; l >>= 1)
+        v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], l);
+      const int r = f * ROWS + step * NW * RPW + warp * RPW + grp;
+      if (r < len) e[r] = v[0];  // (the lanes that share a row step store the same value)
+      if (tid == 0 && f + kIdStages < fills) {
+        if (!mbar_wait(&s_empty[sg], (uint32_t)(f / kIdStages) & 1u))
+          set_err(c.err, HKV_ERR_TIMEOUT);
+        fill(f + kIdStages);
+      }
+    }
+  } else {
+    // U row steps load before any is used
+    for (int r0 = warp * RPW; r0 < len; r0 += U * NW * RPW) {
+      uint4 kr[U];
+  #pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int r = r0 + u * NW * RPW + grp;
+        kr[u] = r < len ? *reinterpret_cast<const uint4 *>(K + (size_t)r * RB + col * 16)
+                        : make_uint4(0u, 0u, 0u, 0u);
+      }
+  #pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int r = r0 + u * NW * RPW + grp;
+        float kf[EPL];
+        Elem<T>::unpack(kr[u], kf);
+        float dot = 0.f;
+  #pragma unroll
+        for (int x = 0; x < EPL; ++x) dot = fmaf(qf[x], kf[x], dot);
+  #pragma unroll
+        for (int o = LPR / 2; o >= 1; o >>= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, o);
+        if (r < len && col == 0) e[r] = dot;
+      }
     }
   }
   __syncthreads();
@@ -1218,8 +1304,9 @@ cudaError_t prepare_t(size_t smem) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(repack_kernel<D, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-  const void *ident[] = {(const void *)identify_kernel<D, T, 2>,
-                         (const void *)identify_kernel<D, T, 8>,
+  const void *ident[] = {(const void *)identify_kernel<D, T, 2, false>,
+                         (const void *)identify_kernel<D, T, 8, false>,
+                         (const void *)identify_kernel<D, T, 8, true>,
                          (const void *)identify_multi_kernel<D, T, 4, 2>,
                          (const void *)identify_multi_kernel<D, T, 4, 4>,
                          (const void *)identify_multi_kernel<D, T, 8, 2>,
@@ -1359,14 +1446,22 @@ cudaError_t launch_identify(const CacheArgs &c, const MethodArgs &m, int layer_b
                             int max_len, cudaStream_t s) {
   const float qscale = (float)(1.4426950408889634 / sqrt((double)D));
   const size_t smem = identify_smem_bytes(max_len, m.P, m.grid2d != 0, false);
+  // the stages lie behind the rest, where both fit (identify_stage_bytes)
+  const size_t staged = identify_stage_bytes(max_len, m.grid2d != 0);
+  if (staged > 0) {
+    HKV_DISPATCH(D, dtype,
+                 return pdl_launch(identify_kernel<kD, kT, 8, true>, nheads, IT, staged, s, c, m,
+                                   layer_base, q, label_out, nh_out, qscale, max_len,
+                                   (int)id_stage_at(smem)));
+  }
   if (id_rows_in_flight(max_len, false) == 8) {
     HKV_DISPATCH(D, dtype,
-                 return pdl_launch(identify_kernel<kD, kT, 8>, nheads, IT, smem, s, c, m,
-                                   layer_base, q, label_out, nh_out, qscale, max_len));
+                 return pdl_launch(identify_kernel<kD, kT, 8, false>, nheads, IT, smem, s, c, m,
+                                   layer_base, q, label_out, nh_out, qscale, max_len, 0));
   }
   HKV_DISPATCH(D, dtype,
-               return pdl_launch(identify_kernel<kD, kT, 2>, nheads, IT, smem, s, c, m, layer_base,
-                                 q, label_out, nh_out, qscale, max_len));
+               return pdl_launch(identify_kernel<kD, kT, 2, false>, nheads, IT, smem, s, c, m,
+                                 layer_base, q, label_out, nh_out, qscale, max_len, 0));
   return cudaErrorInvalidValue;
 }
 
@@ -1386,6 +1481,13 @@ cudaError_t launch_identify_multi(const CacheArgs &c, const MethodArgs &m, int l
   HKV_ID_MULTI(4, 2);
 #undef HKV_ID_MULTI
   return cudaErrorInvalidValue;
+}
+
+size_t identify_stage_bytes(int max_len, bool grid2d) {
+  if (max_len < kIdLongSegment) return 0;
+  const size_t b = id_stage_at(identify_smem_bytes(max_len, 1, grid2d, false)) +
+                   (size_t)kIdStages * kIdStageBytes;
+  return b <= kIdMostSmem ? b : 0;
 }
 
 size_t identify_smem_bytes(int max_len, int P, bool grid2d, bool multi) {
