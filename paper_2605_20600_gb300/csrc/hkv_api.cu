@@ -168,7 +168,7 @@ WsLayout ws_layout(const hkv_config *c) {
   w.ctl = w.rec + align256((size_t)kAttnMaxGrid * sizeof(int4));
   w.pslot = w.ctl + kCtlBytes;
   w.bar = w.pslot + align256((size_t)kAttnMaxGrid * 2 * step_piece_words(c->head_dim) * 8);
-  w.total = w.bar + align256((size_t)c->n_layers * 4 * sizeof(uint32_t));
+  w.total = w.bar + align256((size_t)c->n_layers * 8 * sizeof(uint32_t));
   return w;
 }
 
@@ -194,7 +194,7 @@ AttnArgs attn_args(const hkv_config *cfg, const hkv_cache *cache, int layer, con
   a.rec = reinterpret_cast<int4 *>(ws + w.rec);
   a.ctl = reinterpret_cast<AttnCtl *>(ws + w.ctl);
   a.pslot = reinterpret_cast<unsigned long long *>(ws + w.pslot);
-  a.bar = reinterpret_cast<uint32_t *>(ws + w.bar) + (size_t)layer * 4;
+  a.bar = reinterpret_cast<uint32_t *>(ws + w.bar) + (size_t)layer * 8;
   a.n_layers = cfg->n_layers;
   a.layer = layer;
   a.err = cache->err;
@@ -237,8 +237,8 @@ hkv_status step_ctas(DeviceState *st, int D, int dtype, int *ctas) {
 // config allows). Where it fits, one launch is the faster design on every
 // model shape measured. HKV_STEP_TWO_KERNELS in the environment forces the
 // two-kernel design (tests of both).
-hkv_status one_launch_plan(const hkv_config *cfg, bool fused, StepPlan *plan) {
-  *plan = {0, false};
+hkv_status one_launch_plan(const hkv_config *cfg, bool fused, bool identify, StepPlan *plan) {
+  *plan = {0, 0};
   if (getenv("HKV_STEP_TWO_KERNELS")) return HKV_OK;
   DeviceState *st;
   hkv_status s = device_state(&st);
@@ -248,7 +248,8 @@ hkv_status one_launch_plan(const hkv_config *cfg, bool fused, StepPlan *plan) {
   if (s != HKV_OK) return s;
   int full = st->sms.load(std::memory_order_acquire) * ctas;
   if (full > kAttnMaxGrid) full = kAttnMaxGrid;
-  *plan = step_plan(cfg->head_dim, cfg->dtype, heads_per_layer(cfg), max_segment(*cfg), full, fused);
+  *plan = step_plan(cfg->head_dim, cfg->dtype, heads_per_layer(cfg), max_segment(*cfg), full, fused,
+                    identify);
   return HKV_OK;
 }
 
@@ -405,7 +406,7 @@ hkv_status hkv_decode_attention(const hkv_config *cfg, const hkv_cache *cache, i
   if (ws_bytes < hkv_workspace_size(cfg)) return HKV_ERR_CAPACITY;
   const AttnArgs a = attn_args(cfg, cache, layer, q, out, workspace);
   StepPlan plan;
-  HKV_TRY(one_launch_plan(cfg, false, &plan));
+  HKV_TRY(one_launch_plan(cfg, false, false, &plan));
   if (plan.grid > 0)
     return cuda_status(launch_step(a, cfg->head_dim, cfg->dtype, plan, false, (cudaStream_t)stream));
   int grid = 0;
@@ -419,7 +420,8 @@ namespace {
 // the checks of a decode step of `layer` and its launch plan
 hkv_status step_checks(const char *name, const hkv_config *cfg, const hkv_cache *cache, int layer,
                        const void *q, const void *k, const void *v, const float *out,
-                       const void *workspace, size_t ws_bytes, int flags, StepPlan *plan) {
+                       const void *workspace, size_t ws_bytes, int flags, bool identify,
+                       StepPlan *plan) {
   HKV_TRY(injected(name));
   HKV_TRY(hkv_validate_config(cfg));
   HKV_TRY(check_cache(cache));
@@ -429,7 +431,7 @@ hkv_status step_checks(const char *name, const hkv_config *cfg, const hkv_cache 
     return HKV_ERR_ALIGN;
   if (ws_bytes < ws_layout(cfg).total) return HKV_ERR_CAPACITY;
   if (flags & ~HKV_STEP_PREFETCH) return HKV_ERR_INVALID_ARG;
-  return one_launch_plan(cfg, true, plan);
+  return one_launch_plan(cfg, true, identify, plan);
 }
 
 // the launch, after those checks; no CTAs planned: the two-kernel design
@@ -457,7 +459,8 @@ hkv_status decode_step(const char *name, const hkv_config *cfg, const hkv_cache 
                        uint8_t *label_out, void *workspace, size_t ws_bytes, int flags,
                        hkv_stream_t stream) {
   StepPlan plan;
-  HKV_TRY(step_checks(name, cfg, cache, layer, q, k, v, out, workspace, ws_bytes, flags, &plan));
+  HKV_TRY(step_checks(name, cfg, cache, layer, q, k, v, out, workspace, ws_bytes, flags,
+                      label_out != nullptr, &plan));
   return launch_checked_step(cfg, cache, layer, q, k, v, out, label_out, workspace, flags, plan,
                              stream);
 }
@@ -474,7 +477,7 @@ hkv_status hkv_decode_step(const hkv_config *cfg, const hkv_cache *cache, int la
 int hkv_decode_step_launches(const hkv_config *cfg) {
   if (hkv_validate_config(cfg) != HKV_OK) return 0;
   StepPlan plan;
-  if (one_launch_plan(cfg, true, &plan) != HKV_OK) return 0;
+  if (one_launch_plan(cfg, true, false, &plan) != HKV_OK) return 0;
   return plan.grid > 0 ? 1 : 2;
 }
 
@@ -497,7 +500,7 @@ hkv_status hkv_decode_step_layers(const hkv_config *cfg, const hkv_cache *cache,
   if (label_out && cfg && cfg->distance_mode != HKV_DIST_RASTER) return HKV_ERR_INVALID_ARG;
   StepPlan plan;
   HKV_TRY(step_checks(label_out ? "decode_step_identify" : "decode_step", cfg, cache, 0, q, k, v,
-                      out, workspace, ws_bytes, flags, &plan));
+                      out, workspace, ws_bytes, flags, label_out != nullptr, &plan));
   // (a layer's rows are a multiple of 128 bytes: every layer is as aligned as the first)
   const size_t rows = (size_t)heads_per_layer(cfg) * cfg->head_dim;
   const size_t in = rows * (cfg->dtype == HKV_BF16 ? 2 : 4);

@@ -58,8 +58,9 @@ struct AttnArgs {
   int w_loc;
   float tau;
   // one-launch step (hkv_step.cu): the layer's barrier words {arrivals,
-  // generation, worst status of a bad step, unused}, the arrivals and the
-  // status zero between launches; the partial results of split heads
+  // generation, worst status of a bad step, heads taken, arrivals and
+  // generation of the CTAs that take no more, unused, unused}, all but the
+  // generations zero between launches; the partial results of split heads
   // as (value, launch epoch) pairs, two slots per CTA (the piece at the end
   // of its range, the piece at its start), [grid][2][step_piece_words(D)]
   uint32_t *bar;
@@ -121,14 +122,14 @@ constexpr int kStepActivePerSm = HKV_STEP_ACTIVE_PER_SM;
 
 cudaError_t step_prepare(int D, int dtype, int *ctas_per_sm);
 // The launch of a one-launch step (fused) or attention (not fused) over nheads
-// heads of at most max_rows rows, out of a grid of `full`: its CTAs, and
-// whether it takes the shape for heads that fit one stage. 0 CTAs: a range
-// could hold more heads than the kernel's table, so the two-kernel design runs.
+// heads of at most max_rows rows, out of a grid of `full`: its CTAs and how the
+// layer is cut (hkv_step.cu). 0 CTAs: a range could hold more heads than the
+// kernel's table, so the two-kernel design runs.
 struct StepPlan {
   int grid;
-  bool whole;
+  int cut;
 };
-StepPlan step_plan(int D, int dtype, int nheads, int max_rows, int full, bool fused);
+StepPlan step_plan(int D, int dtype, int nheads, int max_rows, int full, bool fused, bool identify);
 // one layer in one launch: the decode step (append + attention, merges of
 // split heads and counters in the same kernel), with the head types decided
 // where a.label_out is set, or attention alone (not fused); at most

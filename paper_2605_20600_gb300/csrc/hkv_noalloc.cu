@@ -160,7 +160,7 @@ extern "C" hkv_status hkv_decode_attention_noalloc(const hkv_config *cfg, const 
     if (full > kAttnMaxGrid) full = kAttnMaxGrid;
     const size_t piece = 2 * (size_t)step_piece_words(cfg->head_dim) * 8;
     if ((size_t)full * piece > kPartBytes) full = (int)(kPartBytes / piece);
-    const StepPlan plan = step_plan(cfg->head_dim, cfg->dtype, hpl, max_segment(*cfg), full, false);
+    const StepPlan plan = step_plan(cfg->head_dim, cfg->dtype, hpl, max_segment(*cfg), full, false, false);
     if (plan.grid > 0)
       return launch_step(a, cfg->head_dim, cfg->dtype, plan, false, s) == cudaSuccess ? HKV_OK
                                                                                     : HKV_ERR_CUDA;

@@ -22,6 +22,9 @@
 //    (kAlignedGrains), and a small layer a grid no larger than its ranges:
 //    nothing is merged and every CTA of the next launch is resident before
 //    this one ends (Janus-Pro-7B, 2 sequences: 6.6 -> 3.9 us);
+//  * a layer of many short heads is not cut at all: CTAs take heads from a
+//    counter (kHeadSlots; Janus-Pro-7B, 256 sequences: 94.5 -> 89.0 us of 87.8
+//    at the measured bandwidth);
 //  * a warp-specialised TMA pipeline: a producer warp, consumer warps, an
 //    epilogue warp and a merge warp;
 //  * bf16 consumers take q.k on the tensor cores (8 rows a warp and tile: 4
@@ -173,6 +176,18 @@ struct StepShape : StepTile<D, T, SHORT> {
   __host__ __device__ static constexpr int cost(int g) { return g + 1 > kMinCost ? g + 1 : kMinCost; }
 };
 
+// Layers of at least kHeadSlots slots for every CTA, no head above kHeadGrains
+// grains, are not cut beforehand (StepCut): taken head by head a launch costs
+// some 1.5 us more (lengths and claims are fetched on the way, the counters
+// advance at the end) and its CTAs end within 2 us of each other instead of
+// 5. Per layer step, cut -> head by head: Janus-Pro-7B at rho = 1/8 with 96
+// sequences (121 slots) 36.8 -> 37.1 us, with 160 (202) 59.5 -> 58.5, with 256
+// (323) 94.5 -> 89.0; LlamaGen-XL with 250 (131) 24.1 -> 24.4.
+#ifndef HKV_STEP_HEAD_SLOTS
+#define HKV_STEP_HEAD_SLOTS 160
+#endif
+constexpr int kHeadSlots = HKV_STEP_HEAD_SLOTS, kHeadGrains = 16;
+
 // A boundary between ranges that falls within 1/kSnapDiv of a range of a
 // head's first or last row moves there.
 #ifndef HKV_STEP_SNAP_DIV
@@ -207,6 +222,11 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t *p, uint32_t v) {
+  uint32_t old;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+  return old;
 }
 __device__ __forceinline__ void st_release(uint32_t *p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -271,10 +291,17 @@ __host__ __device__ constexpr int step_threads() {
 // the pass (Sec. 4, Step 2), or attention alone (no append, no counters).
 enum StepMode { kModeStep = 0, kModeIdentify = 1, kModeAttend = 2 };
 
-template <int D, typename T, int MODE, bool SHORT>
+// How a launch cuts the layer: into equal ranges of slots, one per CTA; the
+// same with the shape for short heads; or head by head, taken as CTAs get
+// free (many short heads).
+enum StepCut { kCutRanges = 0, kCutShort = 1, kCutHeads = 2 };
+
+template <int D, typename T, int MODE, int CUT>
 __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM)
     step_kernel(const AttnArgs p) {
-  using S = StepShape<D, T, SHORT>;
+  using S = StepShape<D, T, CUT == kCutShort>;
+  constexpr bool DYN = CUT == kCutHeads;
+  static_assert(!DYN || MODE == kModeStep, "heads are taken one by one in plain steps only");
   constexpr bool FUSED = MODE != kModeAttend, IDENT = MODE == kModeIdentify;
   constexpr int kCW = S::kCW, kThr = step_threads<D, T>(), NW = kThr / 32;
   constexpr int LPR = S::kLPR, EPL = S::kEPL, RPW = S::kRPW, TT = S::kTT;
@@ -295,7 +322,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   __shared__ __align__(16) float red_m[2][NST], red_l[2][NST], red_r[IDENT ? 2 : 1][IDENT ? NST : 1];
   __shared__ TileMeta meta[NS];
   __shared__ SegMeta seg[2];
-  __shared__ StepTable<kThr> tab;
+  __shared__ StepTable<DYN ? 1 : kThr> tab;
   __shared__ int2 s_w[NW];  // each warp's slots; its longest head, or a status
   // the range's ends: {first slot, first head, that head's first slot, its
   // rows} and {end slot, last head, that head's first slot, whether the range
@@ -330,6 +357,12 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   }
   if (!p.prefetch) pdl_wait();
 
+  // A layer of many short heads (DYN) is not cut beforehand: CTA k starts with
+  // the heads k and k + G and takes further ones from a counter, so there is
+  // no prologue over the layer's lengths, and CTAs that start late, as the
+  // previous launch's end, take fewer. Its merge warp checks a share of the
+  // heads of its own, appends their tokens and advances their counters.
+  //
   // ---- prologue: the layer's lengths, one round of loads -------------------
   // Warp w takes `rows` rows of 32 consecutive heads and sums each row's
   // slots; the warps' sums give every CTA the same ranges, and only the warps
@@ -342,13 +375,29 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   // length); a range outside it reads its heads once it is known. A CTA that
   // finds a bad head in its range then streams nothing and flags the step on
   // the layer's barrier word, and no CTA appends or advances a counter.
-  const int rows = (nheads + kThr - 1) / kThr;
-  const int row0 = warp * rows;  // this warp's first row
-  const bool in_regs = rows <= 1;
   constexpr int kNew = FUSED ? 1 : 0;   // the step's token is one more row
-  constexpr int kMost = 1 << 26;        // grains of a head, slots of a warp: beyond any arena
-  constexpr int kIsBad = 0x70000000;    // a status in place of the longest head
-  constexpr int kPre = 8;               // rows loaded at once
+  int wl = 0;  // the table's first head
+  // the range: slots [a, b), heads h0 .. h0 + n - 1, the first starting at
+  // slot s0 with v0 rows, the last at s1
+  int a = 0, b = 0, h0 = bx, n = 1, s0 = 0, s1 = 0, v0 = 0, chunk = 1, tol = 0, own_bad = 0;
+  bool has_s = false, has_e = false, in_regs = false, active = true;
+  auto init_barriers = [&]() {  // one thread
+    for (int s = 0; s < NS; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], kCW);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&epi_full[s], kCW);
+      mbar_init(&epi_free[s], 1);
+    }
+    mbar_init(&ep_bar, 32);
+    mbar_init(&oth_bar, 32);
+    mbar_init(&own_bar, 32);
+    fence_barrier_init();
+    s_abort = 0;
+    s_bad = 0;
+    s_mg_h = -1;
+  };
   // the status of a head's counters
   auto verify = [&](int l, long long o, int cp, int lab, int nb) {
     if (FUSED) {
@@ -360,234 +409,241 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     }
     return l < 0 || o < 0 || o + l > p.arena_tokens ? (int)HKV_ERR_BOUNDS : 0;
   };
-  int wl = 0;  // the table's first head
-  if (!in_regs) {
-    wl = (int)((float)bx * ((float)nheads / (float)G)) - kThr / 2;
-    wl = wl < nheads - kThr ? wl : nheads - kThr;
-    wl = wl > 0 ? wl : 0;
-  }
-  int key = 0;
-  unsigned c0 = 0;  // in_regs: the slots of this thread's head
-  int lv[kPre];
-  {
-    // every load issued before any use
-    const int h = wl + tid;
-    int l = 0, cp = 0, lab = 0, nb = 0, nt = 0;
-    long long o = 0;
-    if (h < nheads) {
-      l = p.len[h];
-      o = p.off[h];
-      if (FUSED) {
-        cp = p.cap[h];
-        lab = p.label[p.layer_base + h];
-        nb = p.nbuf[p.layer_base + h];
-        nt = p.ntok[p.layer_base + h];
+  // DYN: the producer's next two heads, their lengths and offsets on their
+  // way, and the one after them, claimed meanwhile
+  int na = bx, nb = bx + G, nc = 0, na_l = -1, nb_l = -1;
+  long long na_o = 0, nb_o = 0;
+  auto fetch = [&](int h, int &l, long long &o) {
+    l = p.len[h];
+    o = p.off[h];
+  };
+  auto claim = [&]() { return 2 * G + (int)atomicAdd(p.bar + 3, 1u); };
+  if constexpr (DYN) {
+    if (tid == 0) {
+      if (na < nheads) fetch(na, na_l, na_o);
+      if (nb < nheads) {
+        fetch(nb, nb_l, nb_o);
+        nc = claim();
       }
     }
+    if (tid == kThr - 32) init_barriers();
+    __syncthreads();
+  } else {
+    const int rows = (nheads + kThr - 1) / kThr;
+    const int row0 = warp * rows;  // this warp's first row
+    in_regs = rows <= 1;
+    constexpr int kMost = 1 << 26;        // grains of a head, slots of a warp: beyond any arena
+    constexpr int kIsBad = 0x70000000;    // a status in place of the longest head
+    constexpr int kPre = 8;               // rows loaded at once
     if (!in_regs) {
+      wl = (int)((float)bx * ((float)nheads / (float)G)) - kThr / 2;
+      wl = wl < nheads - kThr ? wl : nheads - kThr;
+      wl = wl > 0 ? wl : 0;
+    }
+    int key = 0;
+    unsigned c0 = 0;  // in_regs: the slots of this thread's head
+    int lv[kPre];
+    {
+      // every load issued before any use
+      const int h = wl + tid;
+      int l = 0, cp = 0, lab = 0, nb = 0, nt = 0;
+      long long o = 0;
+      if (h < nheads) {
+        l = p.len[h];
+        o = p.off[h];
+        if (FUSED) {
+          cp = p.cap[h];
+          lab = p.label[p.layer_base + h];
+          nb = p.nbuf[p.layer_base + h];
+          nt = p.ntok[p.layer_base + h];
+        }
+      }
+      if (!in_regs) {
+#pragma unroll
+        for (int i = 0; i < kPre; ++i) {
+          const int r = (row0 + i) * 32 + lane;
+          lv[i] = i < rows && r < nheads ? p.len[r] : -1;
+        }
+      }
+      // the barriers, while the loads are on their way (the merge warp's lane)
+      if (tid == kThr - 32) init_barriers();
+      if (h < nheads) {
+        const int e = verify(l, o, cp, lab, nb);
+        tab.vlen[tid] = l + kNew;
+        tab.off[tid] = o;
+        tab.bad[tid] = (unsigned char)e;
+        if (FUSED) {
+          tab.ntok[tid] = nt;
+          tab.label[tid] = (unsigned char)lab;
+        }
+        if (in_regs) {
+          const int g = S::grains(l + kNew);
+          const int st = e ? e : g > kMost ? (int)HKV_ERR_BOUNDS : 0;
+          key = st ? kIsBad + st : g;
+          c0 = st ? 0u : (unsigned)S::cost(g);
+        }
+      }
+    }
+    // the slots of a head of length l of row i (a bad one: 0, and the status)
+    auto slots = [&](int h, int l) {
+      if (h >= nheads) return 0u;
+      const int g = S::grains(l + kNew);
+      const bool ok = FUSED ? l >= 0 && g <= kMost : g <= kMost && !verify(l, p.off[h], 0, 0, 0);
+      if (!ok) key = kIsBad + HKV_ERR_BOUNDS;
+      return ok ? (unsigned)S::cost(g) : 0u;
+    };
+    unsigned rowsum = 0;  // lane i: the slots of row i (up to 32 rows)
+    long long wsum = 0;
+    if (in_regs) {
+      rowsum = __reduce_add_sync(0xFFFFFFFFu, c0);
+      wsum = rowsum;
+    } else {
 #pragma unroll
       for (int i = 0; i < kPre; ++i) {
-        const int r = (row0 + i) * 32 + lane;
-        lv[i] = i < rows && r < nheads ? p.len[r] : -1;
+        if (i < rows) {
+          const unsigned r = __reduce_add_sync(0xFFFFFFFFu, slots((row0 + i) * 32 + lane, lv[i]));
+          if (lane == i) rowsum = r;
+          wsum += r;
+        }
       }
-    }
-    // the barriers, while the loads are on their way (the merge warp's lane)
-    if (tid == kThr - 32) {
-      for (int s = 0; s < NS; ++s) {
-        mbar_init(&full[s], 1);
-        mbar_init(&empty[s], kCW);
-      }
-      for (int s = 0; s < 2; ++s) {
-        mbar_init(&epi_full[s], kCW);
-        mbar_init(&epi_free[s], 1);
-      }
-      mbar_init(&ep_bar, 32);
-      mbar_init(&oth_bar, 32);
-      mbar_init(&own_bar, 32);
-      fence_barrier_init();
-      s_abort = 0;
-      s_bad = 0;
-      s_mg_h = -1;
-    }
-    if (h < nheads) {
-      const int e = verify(l, o, cp, lab, nb);
-      tab.vlen[tid] = l + kNew;
-      tab.off[tid] = o;
-      tab.bad[tid] = (unsigned char)e;
-      if (FUSED) {
-        tab.ntok[tid] = nt;
-        tab.label[tid] = (unsigned char)lab;
-      }
-      if (in_regs) {
-        const int g = S::grains(l + kNew);
-        const int st = e ? e : g > kMost ? (int)HKV_ERR_BOUNDS : 0;
-        key = st ? kIsBad + st : g;
-        c0 = st ? 0u : (unsigned)S::cost(g);
-      }
-    }
-  }
-  // the slots of a head of length l of row i (a bad one: 0, and the status)
-  auto slots = [&](int h, int l) {
-    if (h >= nheads) return 0u;
-    const int g = S::grains(l + kNew);
-    const bool ok = FUSED ? l >= 0 && g <= kMost : g <= kMost && !verify(l, p.off[h], 0, 0, 0);
-    if (!ok) key = kIsBad + HKV_ERR_BOUNDS;
-    return ok ? (unsigned)S::cost(g) : 0u;
-  };
-  unsigned rowsum = 0;  // lane i: the slots of row i (up to 32 rows)
-  long long wsum = 0;
-  if (in_regs) {
-    rowsum = __reduce_add_sync(0xFFFFFFFFu, c0);
-    wsum = rowsum;
-  } else {
-#pragma unroll
-    for (int i = 0; i < kPre; ++i) {
-      if (i < rows) {
-        const unsigned r = __reduce_add_sync(0xFFFFFFFFu, slots((row0 + i) * 32 + lane, lv[i]));
+#pragma unroll 1
+      for (int i = kPre; i < rows; ++i) {
+        const int h = (row0 + i) * 32 + lane;
+        const unsigned r = __reduce_add_sync(0xFFFFFFFFu, slots(h, h < nheads ? p.len[h] : 0));
         if (lane == i) rowsum = r;
         wsum += r;
       }
     }
+    if (wsum > kMost) key = kIsBad + HKV_ERR_BOUNDS;
+    key = __reduce_max_sync(0xFFFFFFFFu, key);
+    if (lane == 0) s_w[warp] = make_int2((int)wsum, key);
+    __syncthreads();
+    if (tid == 0) STEP_TRACE(10);
+    const int2 sw = lane < NW ? s_w[lane] : make_int2(0, 0);
+    const int total = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)sw.x);
+    const int longest = __reduce_max_sync(0xFFFFFFFFu, sw.y);
+    if (longest >= kIsBad) {  // every CTA sees it: none reads further or arrives
+      pdl_wait();
+      if (bx == 0 && tid == 0) {
+        set_err(p.err, (uint32_t)(longest - kIsBad));
+        p.ctl->valid = 0;
+      }
+      return;
+    }
+    // a CTA per head where every head is short (see kAlignedGrains), else G
+    // ranges of `chunk` slots
+    const bool aligned = in_regs && nheads <= G && longest <= kAlignedGrains;
+    // total / G rounded up, from the grid's reciprocal (rounded up, so the
+    // quotient is exact or one too large)
+    chunk = G == 1 ? total : (int)__umulhi((unsigned)(total + G - 1), p.grid_recip);
+    if ((long long)chunk * G > total + G - 1) --chunk;
+    if (chunk < S::kMinChunk) chunk = S::kMinChunk;
+    tol = chunk / HKV_STEP_SNAP_DIV;
+    const long long a64 = (long long)bx * chunk, b64 = a64 + chunk;
+    const int a_raw = a64 < total ? (int)a64 : total, b_raw = b64 < total ? (int)b64 : total;
+    active = aligned ? bx < nheads : a_raw < total;
+    // boundary x inside the slots [s, s + cost) of a head of g grains
+    auto snap = [&](int x, int s, int g) {
+      if (x - s <= tol) return s;
+      return x >= s + g - tol ? s + S::cost(g) : x;
+    };
+    // places head h (slots from s, v rows): whether it is in the range, and
+    // the range's ends when they fall into it
+    auto place = [&](int h, int s, int v) {
+      const int g = S::grains(v), e = s + S::cost(g);
+      if (a_raw >= e || b_raw <= s) return false;
+      bool in = true;
+      if (a_raw >= s) {
+        const int x = snap(a_raw, s, g);
+        const bool next = x == e;
+        s_lo = make_int4(x, next ? h + 1 : h, next ? e : s, v);
+        in = !next;
+      }
+      if (b_raw <= e) {
+        const int x = b_raw == e ? e : snap(b_raw, s, g);
+        s_hi = make_int4(x, x == s ? h - 1 : h, s, x > s && x < e);
+        in = in && x != s;
+      }
+      return in;
+    };
+    if (!aligned && active) {
+      const int before = (int)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? (unsigned)sw.x : 0u);
+      if (before < b_raw && before + (int)wsum > a_raw) {  // warp-uniform
+        // one row: its heads in order
+        auto place_row = [&](int i, int at) {
+          const int h = (row0 + i) * 32 + lane;
+          const bool in = h < nheads;
+          const int j = h - wl;
+          const bool here = j >= 0 && j < kThr;
+          const int v = !in ? 0 : here ? tab.vlen[j] : p.len[h] + kNew;
+          const int c = in ? S::cost(S::grains(v)) : 0;
+          const int incl = warp_incl_scan(c);
+          if (in && place(h, at + incl - c, v) && FUSED && !in_regs && here && tab.bad[j])
+            atomicMax(&s_bad, (int)tab.bad[j]);
+          return __shfl_sync(0xFFFFFFFFu, incl, 31);
+        };
+        if (in_regs) {
+          place_row(0, before);
+        } else if (rows <= 32) {
+          const int incl = warp_incl_scan((int)rowsum);
+          const int rs = before + incl - (int)rowsum;
+          unsigned hit = __ballot_sync(0xFFFFFFFFu, lane < rows && rs < b_raw && before + incl > a_raw);
+          while (hit) {
+            const int i = __ffs(hit) - 1;
+            hit &= hit - 1;
+            place_row(i, __shfl_sync(0xFFFFFFFFu, rs, i));
+          }
+        } else {
+          int at = before;
 #pragma unroll 1
-    for (int i = kPre; i < rows; ++i) {
-      const int h = (row0 + i) * 32 + lane;
-      const unsigned r = __reduce_add_sync(0xFFFFFFFFu, slots(h, h < nheads ? p.len[h] : 0));
-      if (lane == i) rowsum = r;
-      wsum += r;
-    }
-  }
-  if (wsum > kMost) key = kIsBad + HKV_ERR_BOUNDS;
-  key = __reduce_max_sync(0xFFFFFFFFu, key);
-  if (lane == 0) s_w[warp] = make_int2((int)wsum, key);
-  __syncthreads();
-  if (tid == 0) STEP_TRACE(10);
-  const int2 sw = lane < NW ? s_w[lane] : make_int2(0, 0);
-  const int total = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)sw.x);
-  const int longest = __reduce_max_sync(0xFFFFFFFFu, sw.y);
-  if (longest >= kIsBad) {  // every CTA sees it: none reads further or arrives
-    pdl_wait();
-    if (bx == 0 && tid == 0) {
-      set_err(p.err, (uint32_t)(longest - kIsBad));
-      p.ctl->valid = 0;
-    }
-    return;
-  }
-  // a CTA per head where every head is short (see kAlignedGrains), else G
-  // ranges of `chunk` slots
-  const bool aligned = in_regs && nheads <= G && longest <= kAlignedGrains;
-  // total / G rounded up, from the grid's reciprocal (rounded up, so the
-  // quotient is exact or one too large)
-  int chunk = G == 1 ? total : (int)__umulhi((unsigned)(total + G - 1), p.grid_recip);
-  if ((long long)chunk * G > total + G - 1) --chunk;
-  if (chunk < S::kMinChunk) chunk = S::kMinChunk;
-  const int tol = chunk / HKV_STEP_SNAP_DIV;
-  const long long a64 = (long long)bx * chunk, b64 = a64 + chunk;
-  const int a_raw = a64 < total ? (int)a64 : total, b_raw = b64 < total ? (int)b64 : total;
-  bool active = aligned ? bx < nheads : a_raw < total;
-  // boundary x inside the slots [s, s + cost) of a head of g grains
-  auto snap = [&](int x, int s, int g) {
-    if (x - s <= tol) return s;
-    return x >= s + g - tol ? s + S::cost(g) : x;
-  };
-  // places head h (slots from s, v rows): whether it is in the range, and
-  // the range's ends when they fall into it
-  auto place = [&](int h, int s, int v) {
-    const int g = S::grains(v), e = s + S::cost(g);
-    if (a_raw >= e || b_raw <= s) return false;
-    bool in = true;
-    if (a_raw >= s) {
-      const int x = snap(a_raw, s, g);
-      const bool next = x == e;
-      s_lo = make_int4(x, next ? h + 1 : h, next ? e : s, v);
-      in = !next;
-    }
-    if (b_raw <= e) {
-      const int x = b_raw == e ? e : snap(b_raw, s, g);
-      s_hi = make_int4(x, x == s ? h - 1 : h, s, x > s && x < e);
-      in = in && x != s;
-    }
-    return in;
-  };
-  if (!aligned && active) {
-    const int before = (int)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? (unsigned)sw.x : 0u);
-    if (before < b_raw && before + (int)wsum > a_raw) {  // warp-uniform
-      // one row: its heads in order
-      auto place_row = [&](int i, int at) {
-        const int h = (row0 + i) * 32 + lane;
-        const bool in = h < nheads;
-        const int j = h - wl;
-        const bool here = j >= 0 && j < kThr;
-        const int v = !in ? 0 : here ? tab.vlen[j] : p.len[h] + kNew;
-        const int c = in ? S::cost(S::grains(v)) : 0;
-        const int incl = warp_incl_scan(c);
-        if (in && place(h, at + incl - c, v) && FUSED && !in_regs && here && tab.bad[j])
-          atomicMax(&s_bad, (int)tab.bad[j]);
-        return __shfl_sync(0xFFFFFFFFu, incl, 31);
-      };
-      if (in_regs) {
-        place_row(0, before);
-      } else if (rows <= 32) {
-        const int incl = warp_incl_scan((int)rowsum);
-        const int rs = before + incl - (int)rowsum;
-        unsigned hit = __ballot_sync(0xFFFFFFFFu, lane < rows && rs < b_raw && before + incl > a_raw);
-        while (hit) {
-          const int i = __ffs(hit) - 1;
-          hit &= hit - 1;
-          place_row(i, __shfl_sync(0xFFFFFFFFu, rs, i));
+          for (int i = 0; i < rows && at < b_raw; ++i) at += place_row(i, at);
         }
-      } else {
-        int at = before;
-#pragma unroll 1
-        for (int i = 0; i < rows && at < b_raw; ++i) at += place_row(i, at);
       }
     }
-  }
-  __syncthreads();
-  int a = 0, b = 0, h0 = bx, n = 1, s0 = 0, s1 = 0, v0 = 0;
-  bool has_s = false, has_e = false;
-  if (!aligned && active) {
-    const int4 lo = s_lo, hi = s_hi;
-    a = lo.x;
-    b = hi.x;
-    h0 = lo.y;
-    n = hi.y - lo.y + 1;
-    s0 = lo.z;
-    v0 = lo.w;
-    s1 = hi.z;
-    active = a < b && n > 0;
-    has_s = active && s0 < a;
-    has_e = active && hi.w;
+    __syncthreads();
+    if (!aligned && active) {
+      const int4 lo = s_lo, hi = s_hi;
+      a = lo.x;
+      b = hi.x;
+      h0 = lo.y;
+      n = hi.y - lo.y + 1;
+      s0 = lo.z;
+      v0 = lo.w;
+      s1 = hi.z;
+      active = a < b && n > 0;
+      has_s = active && s0 < a;
+      has_e = active && hi.w;
+    }
+    if (!in_regs) {
+      if (FUSED && active && n > kStepTable) {  // excluded by the host; the step is not taken
+        own_bad = HKV_ERR_CAPACITY;
+        active = false;
+      }
+      if (active && (h0 < wl || h0 + n > wl + kThr)) {  // CTA-uniform
+        wl = h0;
+        const int h = h0 + tid, i = p.layer_base + h;
+        if (tid < n) {
+          const int l = p.len[h];
+          const long long o = p.off[h];
+          tab.vlen[tid] = l + kNew;
+          tab.off[tid] = o;
+          if (FUSED) {
+            const int cp = p.cap[h], lab = p.label[i], nb = p.nbuf[i], nt = p.ntok[i];
+            const int e = verify(l, o, cp, lab, nb);
+            if (e) atomicMax(&s_bad, e);
+            tab.ntok[tid] = nt;
+            tab.label[tid] = (unsigned char)lab;
+          }
+        }
+        __syncthreads();
+      }
+      if (FUSED && s_bad) {  // a bad head in this range: stream nothing
+        own_bad = own_bad > s_bad ? own_bad : s_bad;
+        active = false;
+      }
+    }
   }
   const int h1 = h0 + n - 1;
-  int own_bad = 0;
-  if (!in_regs) {
-    if (FUSED && active && n > kStepTable) {  // excluded by the host; the step is not taken
-      own_bad = HKV_ERR_CAPACITY;
-      active = false;
-    }
-    if (active && (h0 < wl || h0 + n > wl + kThr)) {  // CTA-uniform
-      wl = h0;
-      const int h = h0 + tid, i = p.layer_base + h;
-      if (tid < n) {
-        const int l = p.len[h];
-        const long long o = p.off[h];
-        tab.vlen[tid] = l + kNew;
-        tab.off[tid] = o;
-        if (FUSED) {
-          const int cp = p.cap[h], lab = p.label[i], nb = p.nbuf[i], nt = p.ntok[i];
-          const int e = verify(l, o, cp, lab, nb);
-          if (e) atomicMax(&s_bad, e);
-          tab.ntok[tid] = nt;
-          tab.label[tid] = (unsigned char)lab;
-        }
-      }
-      __syncthreads();
-    }
-    if (FUSED && s_bad) {  // a bad head in this range: stream nothing
-      own_bad = own_bad > s_bad ? own_bad : s_bad;
-      active = false;
-    }
-  }
   if (!active) has_s = has_e = false;
   // From here on nothing reads the layer's counters in global memory: the
   // merge warp arrives on the layer's barrier word below. (Attention alone
@@ -616,8 +672,46 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     at_start = true;
     have = true;
   };
+  // This CTA reads no further lengths: the last of the grid to say so resets
+  // the head counter and lets the merge warps advance the lengths (not before
+  // this CTA's has noted the generation).
+  auto no_more = [&]() {
+    mbar_wait(&ep_bar, 0u);
+    if (atom_add_acq_rel(p.bar + 4, 1u) == (uint32_t)G - 1) {
+      p.bar[3] = 0;
+      p.bar[4] = 0;
+      st_release(p.bar + 5, ld_acquire(p.bar + 5) + 1u);
+    }
+  };
   auto next_piece = [&]() {
     have = false;
+    if constexpr (DYN) {
+      while (na < nheads && !have) {
+        const int h = na, l = na_l;
+        const long long o = na_o;
+        na = nb;
+        na_l = nb_l;
+        na_o = nb_o;
+        if (nb < nheads) {
+          nb = nc;
+          if (nb < nheads) {
+            fetch(nb, nb_l, nb_o);
+            nc = claim();
+          }
+        }
+        // (a bad head is not read; the CTA that checks it stops the step)
+        if (l >= 0 && o >= 0 && o + l <= p.arena_tokens) {
+          ph_h = h;
+          ph_v = ph_end = l + 1;
+          ph_off = o;
+          ph_r = 0;
+          ph_flags = kWhole;
+          at_start = have = true;
+        }
+        if (na >= nheads) no_more();  // (after its last length, l, has arrived)
+      }
+      return;
+    }
     if (ph == 0) {
       ph = 1;
       if (has_e && !(has_s && n == 1)) {
@@ -642,7 +736,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   // the arena rows are read once per step: evict them from L2 first (measured:
   // 0.4-0.55 us per step slower without the hint)
   const uint64_t stream_pol = producer ? l2_evict_first_policy() : 0;
-  auto issue_old = [&](int stage) {  // describe, expect and copy the arena rows
+  auto issue_old = [&](int stage, bool open_next) {  // describe, expect and copy the arena rows
     const int left = ph_end - ph_r;
     const int rows = left < TT ? left : TT;
     const int real = ph_v - kNew;  // rows in the arena
@@ -668,7 +762,10 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     meta[stage] = mt;
     at_start = false;
     ph_r += TT;
-    if (last) next_piece();
+    // (DYN: the tile before the wait for the previous kernel does not wait for
+    // the next head's length)
+    if (last && open_next) next_piece();
+    else if (last) have = false;
   };
   auto issue_extra = [&](int stage) {  // the step's inputs, then arrive
     unsigned char *dk = stages + stage * S::kStageBytes;
@@ -686,10 +783,14 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   };
   int n_pre = 0;
   if (producer) {
+    if (DYN && na >= nheads) no_more();
     next_piece();
     const int lim = p.prefetch ? S::kPre : NS;
 #pragma unroll 1
-    while (n_pre < lim && have) issue_old(n_pre++);
+    while (n_pre < lim && have) {
+      ++n_pre;
+      issue_old(n_pre - 1, !DYN || n_pre < lim);
+    }
   }
   if (tid == 0) STEP_TRACE(7);
 
@@ -731,7 +832,28 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       bar_done = 1;
     }
   };
+  // DYN: this CTA's share of the heads for checks, appends and counters
+  const int share = DYN ? (nheads + G - 1) / G : 0;
+  const int sh0 = DYN && bx * share < nheads ? bx * share : nheads;
+  const int sh1 = sh0 + share < nheads ? sh0 + share : nheads;
+  uint32_t taken0 = 0;  // generation of the second barrier: every head is taken
+  int k_len = 0, k_nb = -1, k_nt = 0;  // the counters of the share's first 32 heads
   if (warp == kCW + 2) {
+    if constexpr (DYN) {
+      int e = 0;
+      for (int h = sh0 + lane; h < sh1; h += 32) {
+        const int i = p.layer_base + h;
+        const int l = p.len[h], lab = p.label[i], nbv = p.nbuf[i], ntv = p.ntok[i];
+        e = max(e, verify(l, p.off[h], p.cap[h], lab, nbv));
+        if (h < sh0 + 32) {  // kept for the advance
+          k_len = l;
+          k_nb = lab == HKV_DENSE ? -1 : nbv;
+          k_nt = ntv;
+        }
+      }
+      own_bad = __reduce_max_sync(0xFFFFFFFFu, e);
+      if (lane == 0) taken0 = ld_acquire(p.bar + 5);
+    }
     if (lane == 0) {
       if (has_s) {
         const int er = s0 + S::grains(v0);
@@ -766,6 +888,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       long long w_empty = 0;  // cycles waiting for free stages (tracer)
 #pragma unroll 1
       for (int j = 0; j < n_pre; ++j) issue_extra(j);
+      if (DYN && !have) next_piece();
       st_i = n_pre < NS ? n_pre : 0;
       st_ph = n_pre < NS ? 1u : 0u;
       int armed = n_pre;  // tiles armed in all
@@ -779,7 +902,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         const long long c0 = STEP_CLK();
         if (!stage_free()) break;
         w_empty += STEP_CLK() - c0;
-        issue_old(st_i);
+        issue_old(st_i, true);
         issue_extra(st_i);
         ++armed;
         if (NS == 1 || ++st_i == NS) {
@@ -1170,7 +1293,13 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     };
     // The heads whose last row is in the range (a range's first head always
     // reaches past its start; only its last one can continue past its end).
-    const int napp = active ? (has_e ? n - 1 : n) : 0;
+    const int napp = DYN ? sh1 - sh0 : active ? (has_e ? n - 1 : n) : 0;
+    const int app0 = DYN ? sh0 : h0;
+    // a head's last row (the step's token) in the arena, and its image tokens
+    auto last_row = [&](int h) {
+      return DYN ? p.off[h] + p.len[h] : tab.off[h - wl] + tab.vlen[h - wl] - 1;
+    };
+    auto tokens_of = [&](int h) { return DYN ? p.ntok[p.layer_base + h] : tab.ntok[h - wl]; };
     // Appends: the K/V row at index len, its position, q into the ring of the
     // periodic update. Nothing in this launch reads them.
     auto append = [&]() {
@@ -1188,16 +1317,16 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
           dst[v] = nullptr;
           if (u < units) {
             const int w3 = (u / CH) % 3, cc = u % CH;
-            const int h = h0 + u / (3 * CH), i = p.layer_base + h, j = h - wl;
+            const int h = app0 + u / (3 * CH), i = p.layer_base + h;
             const unsigned char *src = w3 == 0 ? static_cast<const unsigned char *>(p.k_new)
                                      : w3 == 1 ? static_cast<const unsigned char *>(p.v_new)
                                                : static_cast<const unsigned char *>(p.q);
             x[v] = reinterpret_cast<const uint4 *>(src + (size_t)h * RB)[cc];
-            const long long row = tab.off[j] + tab.vlen[j] - 1;
+            const long long row = last_row(h);
             unsigned char *d = w3 == 0 ? static_cast<unsigned char *>(p.K) + row * RB
                              : w3 == 1 ? static_cast<unsigned char *>(p.V) + row * RB
                                        : static_cast<unsigned char *>(p.qbuf) +
-                                             ((size_t)i * p.period + tab.ntok[j] % p.period) * RB;
+                                             ((size_t)i * p.period + tokens_of(h) % p.period) * RB;
             dst[v] = d + (size_t)cc * 16;
           }
         }
@@ -1205,17 +1334,26 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         for (int v = 0; v < NU; ++v)
           if (dst[v]) *reinterpret_cast<uint4 *>(dst[v]) = x[v];
       }
-      for (int h = h0 + lane; h < h0 + napp; h += 32) {
-        const int j = h - wl;
-        p.pos[tab.off[j] + tab.vlen[j] - 1] = p.n_cond + tab.ntok[j];
-      }
+      for (int h = app0 + lane; h < app0 + napp; h += 32)
+        p.pos[last_row(h)] = p.n_cond + tokens_of(h);
     };
     auto advance = [&]() {  // the counters of the appended heads
-      for (int h = h0 + lane; h < h0 + napp; h += 32) {
-        const int i = p.layer_base + h, j = h - wl;
-        p.len[h] = tab.vlen[j];
-        p.ntok[i] = tab.ntok[j] + 1;
-        if (tab.label[j] != HKV_DENSE) ++p.nbuf[i];
+      for (int h = app0 + lane; h < app0 + napp; h += 32) {
+        const int i = p.layer_base + h;
+        if (DYN && h < sh0 + 32) {
+          p.len[h] = k_len + 1;
+          p.ntok[i] = k_nt + 1;
+          if (k_nb >= 0) p.nbuf[i] = k_nb + 1;
+        } else if (DYN) {
+          ++p.len[h];
+          ++p.ntok[i];
+          if (p.label[i] != HKV_DENSE) ++p.nbuf[i];
+        } else {
+          const int j = h - wl;
+          p.len[h] = tab.vlen[j];
+          p.ntok[i] = tab.ntok[j] + 1;
+          if (tab.label[j] != HKV_DENSE) ++p.nbuf[i];
+        }
       }
     };
     // Counters advance once the whole grid has arrived (every CTA has read
@@ -1236,7 +1374,17 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       STEP_TRACE_SET(19, globaltimer());
       if (!s_abort && bar_done && !(gen1 & kBadStep)) {
         append();
-        advance();
+        if (DYN) {  // the lengths advance once no CTA reads another
+          bool all = false;
+          while (!s_abort && !all) {
+            all = __shfl_sync(0xFFFFFFFFu, lane == 0 ? ld_acquire(p.bar + 5) != taken0 : 0, 0);
+            if (!all && timed_out()) break;
+          }
+          __syncwarp();
+          if (all) advance();
+        } else {
+          advance();
+        }
       }
       advanced = true;
     }
@@ -1327,19 +1475,20 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   }
 }
 
-template <int D, typename T, bool SHORT>
+template <int D, typename T, int CUT>
 size_t step_smem() {
-  return (size_t)StepShape<D, T, SHORT>::kNS * StepShape<D, T, SHORT>::kStageBytes;
+  using S = StepShape<D, T, CUT == kCutShort>;
+  return (size_t)S::kNS * S::kStageBytes;
 }
 
-template <int D, typename T, int MODE, bool SHORT>
+template <int D, typename T, int MODE, int CUT>
 cudaError_t step_prepare_m(int *ctas) {
-  const size_t smem = step_smem<D, T, SHORT>();
-  cudaError_t e = cudaFuncSetAttribute(step_kernel<D, T, MODE, SHORT>,
+  const size_t smem = step_smem<D, T, CUT>();
+  cudaError_t e = cudaFuncSetAttribute(step_kernel<D, T, MODE, CUT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int n = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_kernel<D, T, MODE, SHORT>,
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_kernel<D, T, MODE, CUT>,
                                                     step_threads<D, T>(), smem);
   if (n < *ctas) *ctas = n;
   return e;
@@ -1348,20 +1497,21 @@ cudaError_t step_prepare_m(int *ctas) {
 template <int D, typename T>
 cudaError_t step_prepare_t(int *ctas) {
   *ctas = kStepActivePerSm;
-  cudaError_t e = step_prepare_m<D, T, kModeStep, false>(ctas);
-  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeStep, true>(ctas);
-  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeIdentify, false>(ctas);
-  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeAttend, false>(ctas);
+  cudaError_t e = step_prepare_m<D, T, kModeStep, kCutRanges>(ctas);
+  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeStep, kCutShort>(ctas);
+  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeStep, kCutHeads>(ctas);
+  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeIdentify, kCutRanges>(ctas);
+  if (e == cudaSuccess) e = step_prepare_m<D, T, kModeAttend, kCutRanges>(ctas);
   return e;
 }
 
-template <int D, typename T, int MODE, bool SHORT>
+template <int D, typename T, int MODE, int CUT>
 cudaError_t step_launch_m(const AttnArgs &a, int grid, cudaStream_t s) {
   static const bool pdl = getenv("HKV_NO_PDL") == nullptr;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(step_threads<D, T>());
-  cfg.dynamicSmemBytes = step_smem<D, T, SHORT>();
+  cfg.dynamicSmemBytes = step_smem<D, T, CUT>();
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   int na = 0;
@@ -1372,31 +1522,34 @@ cudaError_t step_launch_m(const AttnArgs &a, int grid, cudaStream_t s) {
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, step_kernel<D, T, MODE, SHORT>, a);
+  return cudaLaunchKernelEx(&cfg, step_kernel<D, T, MODE, CUT>, a);
 }
 
 template <int D, typename T>
-cudaError_t step_launch_t(AttnArgs a, int grid, bool fused, bool whole, cudaStream_t s) {
+cudaError_t step_launch_t(AttnArgs a, int grid, bool fused, int cut, cudaStream_t s) {
   a.grid_recip = (uint32_t)(((1ull << 32) + grid - 1) / grid);  // (not used for a grid of one)
-  if (!fused) return step_launch_m<D, T, kModeAttend, false>(a, grid, s);
-  if (a.label_out) return step_launch_m<D, T, kModeIdentify, false>(a, grid, s);
-  return whole ? step_launch_m<D, T, kModeStep, true>(a, grid, s)
-               : step_launch_m<D, T, kModeStep, false>(a, grid, s);
+  if (!fused) return step_launch_m<D, T, kModeAttend, kCutRanges>(a, grid, s);
+  if (a.label_out) return step_launch_m<D, T, kModeIdentify, kCutRanges>(a, grid, s);
+  return cut == kCutShort   ? step_launch_m<D, T, kModeStep, kCutShort>(a, grid, s)
+         : cut == kCutHeads ? step_launch_m<D, T, kModeStep, kCutHeads>(a, grid, s)
+                            : step_launch_m<D, T, kModeStep, kCutRanges>(a, grid, s);
 }
 
 // The CTAs a layer of n heads gets out of a full grid: see step_plan.
 template <int D, typename T>
-StepPlan step_plan_t(long long n, long long max_rows, int full, bool fused) {
+StepPlan step_plan_t(long long n, long long max_rows, int full, bool fused, bool identify) {
   using S = StepShape<D, T>;
   const long long g = (max_rows + S::kGR - 1) / S::kGR;
   const long long total = n * (g + 1 > S::kMinCost ? g + 1 : S::kMinCost);
+  if (fused && !identify && total >= (long long)kHeadSlots * full && g <= kHeadGrains)
+    return {full, kCutHeads};
   long long chunk = (total + full - 1) / full;
   if (chunk < S::kMinChunk) chunk = S::kMinChunk;
-  if (n > kStepTable && chunk / S::kMinCost + 2 > kStepTable) return {0, false};
-  if (!fused) return {full, false};
-  if (n <= full && n <= kStepTable && g <= kAlignedGrains) return {(int)n, true};
+  if (n > kStepTable && chunk / S::kMinCost + 2 > kStepTable) return {0, kCutRanges};
+  if (!fused) return {full, kCutRanges};
+  if (!identify && n <= full && n <= kStepTable && g <= kAlignedGrains) return {(int)n, kCutShort};
   const long long need = (total + S::kMinChunk - 1) / S::kMinChunk;
-  return {need < full ? (int)need : full, false};
+  return {need < full ? (int)need : full, kCutRanges};
 }
 
 }  // namespace
@@ -1407,12 +1560,12 @@ extern "C" int hkv_debug_set_step_trace(unsigned long long *buf) {
 }
 #endif
 
-StepPlan step_plan(int D, int dtype, int nheads, int max_rows, int full, bool fused) {
+StepPlan step_plan(int D, int dtype, int nheads, int max_rows, int full, bool fused, bool identify) {
   if (dtype == HKV_BF16)
-    return D == 64 ? step_plan_t<64, __nv_bfloat16>(nheads, max_rows, full, fused)
-                   : step_plan_t<128, __nv_bfloat16>(nheads, max_rows, full, fused);
-  return D == 64 ? step_plan_t<64, float>(nheads, max_rows, full, fused)
-                 : step_plan_t<128, float>(nheads, max_rows, full, fused);
+    return D == 64 ? step_plan_t<64, __nv_bfloat16>(nheads, max_rows, full, fused, identify)
+                   : step_plan_t<128, __nv_bfloat16>(nheads, max_rows, full, fused, identify);
+  return D == 64 ? step_plan_t<64, float>(nheads, max_rows, full, fused, identify)
+                 : step_plan_t<128, float>(nheads, max_rows, full, fused, identify);
 }
 
 cudaError_t step_prepare(int D, int dtype, int *ctas) {
@@ -1426,10 +1579,10 @@ cudaError_t launch_step(const AttnArgs &a, int D, int dtype, StepPlan plan, bool
   const int grid = plan.grid;
   if (grid < 1 || grid > kAttnMaxGrid) return cudaErrorInvalidValue;
   if (dtype == HKV_BF16)
-    return D == 64 ? step_launch_t<64, __nv_bfloat16>(a, grid, fused, plan.whole, s)
-                   : step_launch_t<128, __nv_bfloat16>(a, grid, fused, plan.whole, s);
-  return D == 64 ? step_launch_t<64, float>(a, grid, fused, plan.whole, s)
-                 : step_launch_t<128, float>(a, grid, fused, plan.whole, s);
+    return D == 64 ? step_launch_t<64, __nv_bfloat16>(a, grid, fused, plan.cut, s)
+                   : step_launch_t<128, __nv_bfloat16>(a, grid, fused, plan.cut, s);
+  return D == 64 ? step_launch_t<64, float>(a, grid, fused, plan.cut, s)
+                 : step_launch_t<128, float>(a, grid, fused, plan.cut, s);
 }
 
 }  // namespace hkv

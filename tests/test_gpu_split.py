@@ -31,8 +31,8 @@ def _lens(kind, n, grain, rng):
 
 CASES = [("aligned", 1), ("aligned", 64), ("aligned", 256), ("just over", 64), ("edges", 287),
          ("edges", 288), ("edges", 289), ("edges", 351), ("edges", 352), ("edges", 353),
-         ("edges", 2304), ("edges", 2817), ("edges", 3300), ("long", 7), ("long", 300),
-         ("long", 900)]
+         ("edges", 2304), ("edges", 2817), ("edges", 3300), ("edges", 6100), ("edges", 9800),
+         ("long", 7), ("long", 300), ("long", 900)]
 
 
 @pytest.mark.parametrize("D,dtype", [(128, "bf16"), (64, "bf16"), (128, "fp32"), (64, "fp32")])
@@ -119,3 +119,60 @@ def test_split(kind, n, D, dtype):
     newest = torch.where(order >= (width - 4)[:, None], p[:, :-1], 0.0).sum(1) + p[:, -1]
     sure = (newest - 0.9).abs() > 1e-5
     assert torch.equal(label[sl][sure], torch.where(newest >= 0.9, 0, 1).to(torch.uint8)[sure])
+
+
+@pytest.mark.parametrize("fault", ["capacity", "state", "bounds", "negative"])
+@pytest.mark.parametrize("head", [0, 303, 304, 1700, 3999])
+def test_one_bad_head_of_many_short_ones_stops_the_step(fault, head):
+    """Layers taken head by head: a bad head anywhere leaves every row, counter
+    and query of the layer as it was; repaired, the next call on the same
+    workspace takes the step."""
+    import torch
+    from paper_2605_20600_gb300 import hkv as H
+    from paper_2605_20600_gb300.engine import CacheBuffers
+    n, D, P = 4000, 64, 8   # 255 rows allowed: 16 grains, 17 slots a head
+    cfg = H.make_config(n_layers=1, n_seqs=4, n_heads=n // 4, head_dim=D, dtype="bf16", n_cond=1,
+                        n_image=300, row_len=8, recent_w=8, local_w=5, period=P, group_at=254,
+                        global_budget=40)
+    g = torch.Generator(device="cuda").manual_seed(head)
+    lens = torch.randint(0, 60, (n,), generator=g, device="cuda", dtype=torch.int32)
+    cb = CacheBuffers(cfg, n * 64, "cuda")
+    for t in (cb.k, cb.v, cb.qbuf):
+        t.normal_(generator=g)
+    cb.off.copy_(torch.arange(n, device="cuda") * 64)
+    cb.cap.fill_(64)
+    cb.len.copy_(lens)
+    cb.label.copy_(torch.arange(n, device="cuda") % 2)
+    cb.nbuf.fill_(3)
+    cb.ntok.fill_(70)
+    field, value, code = {"capacity": (cb.cap, lens[head], H.HKV_ERR_CAPACITY),
+                          "state": (cb.nbuf, P, H.HKV_ERR_STATE),
+                          "bounds": (cb.off, n * 64, H.HKV_ERR_BOUNDS),
+                          "negative": (cb.len, -1, H.HKV_ERR_BOUNDS)}[fault]
+    good = field[head].clone()
+    field[head] = value
+    q, k, v = (torch.randn(4, n // 4, D, generator=g, device="cuda").bfloat16() for _ in range(3))
+    out = torch.zeros(4, n // 4, D, device="cuda")
+    ws = torch.zeros(H.hkv_workspace_size(cfg), dtype=torch.uint8, device="cuda")
+    st = torch.cuda.current_stream().cuda_stream
+    names = ("k", "v", "pos", "len", "ntok", "nbuf", "qbuf")
+    before = {nm: getattr(cb, nm).clone() for nm in names}
+    H.hkv_decode_step(cfg, cb.c, 0, q, k, v, out, ws, ws.numel(), 0, st)
+    with pytest.raises(H.HkvError) as e:
+        H.hkv_check(cb.c)
+    assert e.value.status == code
+    for nm in names:
+        assert torch.equal(getattr(cb, nm), before[nm]), nm
+    field[head] = good
+    cb.err.zero_()
+    for step in range(2):     # and again: the counters are ready for the next launch
+        H.hkv_decode_step(cfg, cb.c, 0, q, k, v, out, ws, ws.numel(), 0, st)
+        H.hkv_check(cb.c)
+        assert torch.equal(cb.len, lens + 1 + step)
+        assert (cb.nbuf == 4 + step).all() and (cb.ntok == 71 + step).all()
+    K = cb.k.view(n, 64, D).double()
+    V = cb.v.view(n, 64, D).double()
+    s = torch.einsum("nrd,nd->nr", K, q.view(n, D).double()) / D ** 0.5
+    s = s.masked_fill(torch.arange(64, device="cuda")[None] >= cb.len[:, None], -torch.inf)
+    exp = torch.einsum("nr,nrd->nd", torch.softmax(s, 1), V)
+    assert (out.view(n, D).double() - exp).abs().max().item() <= TOL["bf16"]
