@@ -169,7 +169,15 @@ struct StepShape : StepTile<D, T, SHORT> {
   // minimum bounds the heads of a range (step_max_heads).
   static constexpr int kGR = step_grain(Tile::kRB);
   static constexpr int kMinCost = Tile::kRB == 128 ? 5 : 3;
-  static constexpr int kMinChunk = SHORT ? kAlignedGrains : 2 * Tile::kTT / kGR;  // fewest slots per CTA range
+  // Fewest slots of a CTA's range: on small layers a longer range costs less
+  // than one more piece to combine. Periods of steps over 12 layers of
+  // Lumina-mGPT 1024 at rho = 1/6, ms with 2, 3, 4, 5, 6 and 8 tiles: one
+  // sequence 5.85, 5.29, 5.05, 5.34, 5.55, 6.27, two sequences 6.66, 6.26,
+  // 6.00, 6.33, 6.45, 6.94. The kernels that stop after the attention or the
+  // grouping are best with 3: attention over one dense sequence 214, 208, 209.
+  static constexpr __host__ __device__ int min_chunk(bool step) {
+    return SHORT ? kAlignedGrains : (step ? 4 : 3) * Tile::kTT / kGR;
+  }
   __host__ __device__ static constexpr int grains(int rows) {
     return (int)(((unsigned)rows + kGR - 1) / kGR);
   }
@@ -537,7 +545,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     // quotient is exact or one too large)
     chunk = G == 1 ? total : (int)__umulhi((unsigned)(total + G - 1), p.grid_recip);
     if ((long long)chunk * G > total + G - 1) --chunk;
-    if (chunk < S::kMinChunk) chunk = S::kMinChunk;
+    if (chunk < S::min_chunk(MODE == kModeStep)) chunk = S::min_chunk(MODE == kModeStep);
     tol = chunk / HKV_STEP_SNAP_DIV;
     const long long a64 = (long long)bx * chunk, b64 = a64 + chunk;
     const int a_raw = a64 < total ? (int)a64 : total, b_raw = b64 < total ? (int)b64 : total;
@@ -1544,11 +1552,12 @@ StepPlan step_plan_t(long long n, long long max_rows, int full, bool fused, bool
   if (fused && !identify && total >= (long long)kHeadSlots * full && g <= kHeadGrains)
     return {full, kCutHeads};
   long long chunk = (total + full - 1) / full;
-  if (chunk < S::kMinChunk) chunk = S::kMinChunk;
+  const int least = S::min_chunk(fused && !identify);
+  if (chunk < least) chunk = least;
   if (n > kStepTable && chunk / S::kMinCost + 2 > kStepTable) return {0, kCutRanges};
   if (!fused) return {full, kCutRanges};
   if (!identify && n <= full && n <= kStepTable && g <= kAlignedGrains) return {(int)n, kCutShort};
-  const long long need = (total + S::kMinChunk - 1) / S::kMinChunk;
+  const long long need = (total + least - 1) / least;
   return {need < full ? (int)need : full, kCutRanges};
 }
 
