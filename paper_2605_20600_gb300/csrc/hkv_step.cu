@@ -41,7 +41,8 @@
 //    never waits for a piece that finishes last in its CTA (measured: 0.3
 //    us per step less than the other order at rho = 1/8);
 //  * merges: a split head is combined by its first middle CTA (whose whole
-//    range lies inside the head), else by the CTA holding its last row. The
+//    range lies inside the head), else (and in the attention alone) by the
+//    CTA holding its last row. The
 //    other pieces write their partial result to the workspace as 64-bit
 //    (value, launch epoch) pairs, which are single-copy atomic, so no fence
 //    or flag is needed: the combining CTA's merge warp reads the pieces until
@@ -62,8 +63,8 @@
 //    arrival and the first tiles of old K/V rows go ahead of the wait for the
 //    previous kernel; the step's inputs (q, the new k and v) are read after
 //    it;
-//  * every wait is bounded (HKV_ERR_TIMEOUT in the error word). The waits on
-//    other CTAs need the whole grid resident: it is at most what fits.
+//  * every wait is bounded (HKV_ERR_TIMEOUT in the error word). A step's waits
+//    on other CTAs need the whole grid resident: it is at most what fits.
 #include <math.h>
 #include <stdlib.h>
 
@@ -805,7 +806,9 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   // ---- merge warp: the launch's epoch and the split head this CTA combines --
   // The split head: the first of the range when this CTA is that head's
   // first middle CTA (its whole range inside the head) or, for a head in two
-  // pieces, holds its last row. The epoch is unique per (layer, launch of
+  // pieces and in the attention alone, holds its last row: CTAs then wait for
+  // lower-numbered ones only, which start before them, so that launches of the
+  // attention that share the GPU never hold each other's places. The epoch is unique per (layer, launch of
   // that layer), from the generation of the layer's barrier word; the
   // epilogue waits for both only when it meets a split head.
   //
@@ -871,7 +874,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         const long long x1 = (long long)k1 * chunk;
         if (x1 > s0 && x1 >= er - tol) --k1;  // that one to its end
         const int np = k1 - k0 + 1;
-        if ((np >= 3 ? k0 + 1 : k1) == bx) {
+        if ((FUSED && np >= 3 ? k0 + 1 : k1) == bx) {
           s_mg_k0 = k0;
           s_mg_np = np;
           s_mg_j = bx - k0;

@@ -176,3 +176,41 @@ def test_one_bad_head_of_many_short_ones_stops_the_step(fault, head):
     s = s.masked_fill(torch.arange(64, device="cuda")[None] >= cb.len[:, None], -torch.inf)
     exp = torch.einsum("nr,nrd->nd", torch.softmax(s, 1), V)
     assert (out.view(n, D).double() - exp).abs().max().item() <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("D,dtype", [(128, "bf16"), (64, "fp32")])
+def test_attention_on_streams_that_share_the_gpu(D, dtype):
+    """The attention alone, a head over many CTAs, on four streams with a
+    workspace each: every call gives the bits of a call on its own."""
+    import torch
+    from paper_2605_20600_gb300 import hkv as H
+    from paper_2605_20600_gb300.engine import CacheBuffers, torch_dtype
+    n, C = 40, 3000
+    cfg = H.make_config(n_layers=1, n_seqs=1, n_heads=n, head_dim=D, dtype=dtype, n_cond=C,
+                        n_image=64, row_len=8, recent_w=8, local_w=5, period=8, group_at=9,
+                        global_budget=16)
+    g = torch.Generator(device="cuda").manual_seed(D)
+    cb = CacheBuffers(cfg, n * C, "cuda")
+    cb.k.normal_(generator=g)
+    cb.v.normal_(generator=g)
+    cb.off.copy_(torch.arange(n, device="cuda") * C)
+    cb.cap.fill_(C)
+    cb.len.copy_(torch.randint(0, C + 1, (n,), generator=g, device="cuda"))
+    q = torch.randn(1, n, D, generator=g, device="cuda").to(torch_dtype(cfg))
+
+    def call(out, ws, stream):
+        H.hkv_decode_attention(cfg, cb.c, 0, q, out, ws, ws.numel(), stream.cuda_stream)
+
+    nbytes = H.hkv_workspace_size(cfg)
+    spaces = [torch.zeros(nbytes, dtype=torch.uint8, device="cuda") for _ in range(4)]
+    outs = torch.full((4, 25, 1, n, D), float("nan"), device="cuda")
+    alone = torch.empty(1, n, D, device="cuda")
+    call(alone, spaces[0], torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(priority=-(i % 2)) for i in range(4)]
+    for i in range(25):
+        for s, ws, o in zip(streams, spaces, outs):
+            call(o[i], ws, s)
+    torch.cuda.synchronize()
+    H.hkv_check(cb.c)
+    assert torch.equal(outs, alone.expand_as(outs))
