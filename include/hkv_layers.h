@@ -14,7 +14,7 @@ extern "C" {
 
 /* hkv_repack for every layer in one launch (one CTA per head of the model):
  * the same results, checks and errors as a call per layer. Asynchronous on
- * `stream`. */
+ * `stream`; a decode step with HKV_STEP_PREFETCH may follow it directly. */
 hkv_status hkv_repack_all(const hkv_config *cfg, const hkv_cache *dense, const hkv_cache *ragged,
                           hkv_stream_t stream);
 

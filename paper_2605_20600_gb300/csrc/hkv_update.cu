@@ -609,8 +609,9 @@ __global__ void __launch_bounds__(NT, kUpdCtasPerSm)
   constexpr int RB = D * (int)sizeof(T);
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ UpdShared sh;
+  // no early launch of the next kernel (as in evict_kernel): this one writes
+  // every layer's cache, which a prefetching decode step reads before its wait
   pdl_wait();
-  pdl_launch_dependents();
   const int tid = threadIdx.x, i = layer_base + blockIdx.x;
   const int slen = dn.len[i];
   const long long soff = dn.off[i];
@@ -713,8 +714,7 @@ __global__ void __launch_bounds__(512) prefill_kernel(const CacheArgs c, int lay
 }
 
 __global__ void init_dense_kernel(const CacheArgs c, int n, int seg) {
-  pdl_wait();
-  pdl_launch_dependents();
+  pdl_wait();  // and no early launch: every layer's counters are written here
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const_cast<int64_t *>(c.off)[i] = (int64_t)i * seg;
     const_cast<int32_t *>(c.cap)[i] = seg;
