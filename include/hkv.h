@@ -63,9 +63,9 @@ enum {
    * rows while that kernel is still finishing (programmatic dependent
    * launch), and waits for it only before touching q, k, v. True when the
    * previous kernel is the decode step or attention of another layer, or
-   * any call of this library other than a decode step, append or prefill of
-   * the same layer (hkv_evict, hkv_repack and hkv_init_dense, which may write
-   * every layer's cache, never let the next kernel start early). */
+   * any call of this library other than a decode step or append of the same
+   * layer (hkv_evict, hkv_repack, hkv_prefill and hkv_init_dense never let
+   * the next kernel start early). */
   HKV_STEP_PREFETCH = 1
 };
 

@@ -93,8 +93,8 @@ class Engine:
     def step(self, layer: int, q, k, v, out) -> None:
         # layers run in order, so with two or more layers the kernel before a
         # decode step belongs to another layer (or is one that never lets its
-        # successor start early: hkv_evict, hkv_repack, hkv_init_dense, alone
-        # or over every layer): the step may prefetch
+        # successor start early: hkv_evict, hkv_repack, hkv_prefill,
+        # hkv_init_dense, of one layer or every one): the step may prefetch
         flags = H.HKV_STEP_PREFETCH if self.cfg.n_layers >= 2 else 0
         H.hkv_decode_step(self.cfg, self.cache.c, layer, q, k, v, out, self.ws, self.ws_bytes,
                           flags, self.stream())

@@ -1,6 +1,6 @@
-"""A decode step with HKV_STEP_PREFETCH directly behind a call that writes the
-cache of every layer (no kernel in between, one graph): it must find what that
-call wrote. On the CPU, the rule that makes it so: such a kernel never lets
+"""A decode step with HKV_STEP_PREFETCH directly behind a call that writes that
+step's cache (no kernel in between, one graph): it must find what that call
+wrote. On the CPU, the rule that makes it so: such a kernel never lets
 the next one start early."""
 import os
 import re
@@ -12,8 +12,9 @@ from conftest import ROOT
 UPDATE = os.path.join(ROOT, "paper_2605_20600_gb300", "csrc", "hkv_update.cu")
 
 
-@pytest.mark.parametrize("kernel", ["evict_kernel", "repack_kernel", "init_dense_kernel"])
-def test_kernels_over_every_layer_do_not_launch_early(kernel):
+@pytest.mark.parametrize("kernel", ["evict_kernel", "repack_kernel", "init_dense_kernel",
+                                    "prefill_kernel"])
+def test_kernels_before_a_step_do_not_launch_early(kernel):
     text = re.sub(r"//.*", "", open(UPDATE).read())
     body = text[re.search(r"\b%s\(const CacheArgs" % kernel, text).start():]
     body = body[:body.index("\n}\n")]
@@ -121,3 +122,50 @@ def test_step_behind_the_set_up_of_the_uncompressed_cache():
         assert (c.len == 1).all() and (c.ntok == 1).all() and (c.nbuf == 0).all()
         at = c.off.long()
         assert torch.equal(c.k[at], k.view(-1, 64)) and (c.pos[at] == 0).all()
+
+
+@pytest.mark.gpu
+def test_step_behind_the_prefill_of_its_layer():
+    import torch
+    from paper_2605_20600_gb300 import hkv as H
+    from paper_2605_20600_gb300.engine import Engine
+    C, n = 40, 20
+    cfg = H.make_config(n_layers=2, n_seqs=1, n_heads=n, head_dim=128, dtype="bf16", n_cond=C,
+                        n_image=64, row_len=8, recent_w=8, local_w=8, period=5, group_at=16,
+                        global_budget=16)
+    eng = Engine(cfg, "cuda")
+    c = eng.dense
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q, k, v = (torch.randn(2, 1, n, 128, generator=g, device="cuda").bfloat16() for _ in range(3))
+    kc, vc = (torch.randn(2, 1, n, C, 128, generator=g, device="cuda").bfloat16() for _ in range(2))
+    out = torch.empty(2, 1, n, 128, device="cuda")
+
+    def both(between):
+        for layer in range(2):
+            eng.prefill(layer, kc[layer], vc[layer])
+            between()
+            eng.step(layer, q[layer], k[layer], v[layer], out[layer])
+
+    def empty():
+        c.len.zero_()
+        c.k.zero_()
+        c.v.zero_()
+        out.fill_(float("nan"))
+
+    empty()
+    both(torch.cuda.synchronize)
+    eng.check()
+    names = ("k", "v", "pos", "len", "nbuf", "ntok", "qbuf")
+    want, want_out = _copy(c, names), out.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        both(lambda: None)
+    for _ in range(20):
+        empty()
+        graph.replay()
+        torch.cuda.synchronize()
+        eng.check()
+        assert torch.equal(out, want_out)
+        assert (c.len == C + 1).all()
+        for nm in names:
+            assert torch.equal(getattr(c, nm), want[nm]), nm
