@@ -198,11 +198,13 @@ hkv_status hkv_update_due(const hkv_config *cfg, int32_t t, int32_t *due_out);
 
 /* Bytes of device workspace hkv_decode_attention and hkv_decode_step need
  * for this config (split-K partial results, records of the heads split
- * between CTAs, a small control block, ready flags of the partial results
- * and eight barrier words per layer). The workspace must be zero-filled before
+ * between CTAs, a small control block, partial results tagged with the launch
+ * that wrote them, and barrier words: eight per layer for the step, one set
+ * for the attention alone). The workspace must be zero-filled before
  * its first use; every call leaves it ready for the next one (after a call
- * that reported an error, zero it again). Concurrent calls must not share a
- * workspace. Host only. */
+ * that reported an error, zero it again). Decode steps of one config only may
+ * share a workspace; hkv_decode_attention may use one workspace for several
+ * configs in turn. Concurrent calls must not share a workspace. Host only. */
 size_t hkv_workspace_size(const hkv_config *cfg);
 
 /* Sets up the uncompressed cache of Step 1 (cache prefilling): every head

@@ -152,21 +152,28 @@ constexpr size_t kCtlBytes = 256;  // AttnCtl, padded
 // Workspace of the decode kernels, in this order: split-K partials
 // (kAttnInlinePieces slots per CTA boundary, one overflow slot per CTA), the
 // record of the head split at each CTA boundary, the control block the
-// two-kernel design's attention kernel leaves for its finishing kernel, the
-// epoch-tagged partial results of the one-launch step (two slots of
-// step_piece_words(D) 8-byte pairs per CTA) and its per-layer barrier words.
+// two-kernel design's attention kernel leaves for its finishing kernel; at the
+// same place for every config (behind the above for the largest head_dim) the
+// barrier words and the epoch-tagged partial results of the attention alone
+// in one launch; then those of the one-launch step (two slots of
+// step_piece_words(D) 8-byte pairs per CTA; barrier words per layer).
 struct WsLayout {
-  size_t part, over, rec, ctl, pslot, bar, total;
+  size_t part, over, rec, ctl, abar, apslot, pslot, bar, total;
 };
 
 WsLayout ws_layout(const hkv_config *c) {
   WsLayout w;
-  const size_t pf = attn_part_floats(c->head_dim) * sizeof(float);
-  w.part = 0;
-  w.over = w.part + align256((size_t)kAttnMaxGrid * kAttnInlinePieces * pf);
-  w.rec = w.over + align256((size_t)kAttnMaxGrid * pf);
-  w.ctl = w.rec + align256((size_t)kAttnMaxGrid * sizeof(int4));
-  w.pslot = w.ctl + kCtlBytes;
+  auto ctl_at = [&](int D) {
+    const size_t pf = attn_part_floats(D) * sizeof(float);
+    w.part = 0;
+    w.over = w.part + align256((size_t)kAttnMaxGrid * kAttnInlinePieces * pf);
+    w.rec = w.over + align256((size_t)kAttnMaxGrid * pf);
+    return w.rec + align256((size_t)kAttnMaxGrid * sizeof(int4));
+  };
+  w.abar = ctl_at(128) + kCtlBytes;
+  w.apslot = w.abar + 256;
+  w.pslot = w.apslot + align256((size_t)kAttnMaxGrid * 2 * step_piece_words(128) * 8);
+  w.ctl = ctl_at(c->head_dim);
   w.bar = w.pslot + align256((size_t)kAttnMaxGrid * 2 * step_piece_words(c->head_dim) * 8);
   w.total = w.bar + align256((size_t)c->n_layers * 8 * sizeof(uint32_t));
   return w;
@@ -404,7 +411,16 @@ hkv_status hkv_decode_attention(const hkv_config *cfg, const hkv_cache *cache, i
   if (!q || !out || !workspace) return HKV_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(out) || !aligned16(workspace)) return HKV_ERR_ALIGN;
   if (ws_bytes < hkv_workspace_size(cfg)) return HKV_ERR_CAPACITY;
-  const AttnArgs a = attn_args(cfg, cache, layer, q, out, workspace);
+  AttnArgs a = attn_args(cfg, cache, layer, q, out, workspace);
+  // One set of words for the attentions of every layer and config: each waits
+  // for the kernel before it, so they never overlap, and an epoch that counts
+  // them all is never met twice. Not the step's words: a step of this layer
+  // that prefetches may arrive on those while this launch is still at work.
+  const WsLayout w = ws_layout(cfg);
+  a.bar = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(workspace) + w.abar);
+  a.pslot = reinterpret_cast<unsigned long long *>(static_cast<unsigned char *>(workspace) + w.apslot);
+  a.n_layers = 1;
+  a.layer = 0;
   StepPlan plan;
   HKV_TRY(one_launch_plan(cfg, false, false, &plan));
   if (plan.grid > 0)

@@ -57,7 +57,8 @@ struct AttnArgs {
   uint8_t *label_out;         // [L*S*H]
   int w_loc;
   float tau;
-  // one-launch step (hkv_step.cu): the layer's barrier words {arrivals,
+  // one-launch step (hkv_step.cu): the layer's barrier words (the attention
+  // alone: its own, for every layer, with n_layers 1 and layer 0) {arrivals,
   // generation, worst status of a bad step, heads taken, arrivals and
   // generation of the CTAs that take no more, unused, unused}, all but the
   // generations zero between launches; the partial results of split heads

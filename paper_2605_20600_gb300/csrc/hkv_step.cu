@@ -808,8 +808,10 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   // first middle CTA (its whole range inside the head) or, for a head in two
   // pieces and in the attention alone, holds its last row: CTAs then wait for
   // lower-numbered ones only, which start before them, so that launches of the
-  // attention that share the GPU never hold each other's places. The epoch is unique per (layer, launch of
-  // that layer), from the generation of the layer's barrier word; the
+  // attention that share the GPU never hold each other's places. The epoch,
+  // from the generation of the barrier word, is unique per (layer, launch of
+  // that layer), or among the attentions alone, which have words and slots of
+  // their own (p.n_layers is 1 there, whatever the layer); the
   // epilogue waits for both only when it meets a split head.
   //
   // Then this CTA arrives on the layer's barrier words {arrivals,
