@@ -243,11 +243,12 @@ hkv_status hkv_append_evict(const hkv_config *cfg, const hkv_cache *cache, int l
  * same update hkv_append_evict runs before its append, without the append.
  * Heads whose buffer is not full are left as they are, so the call is
  * harmless when no update is due; with hkv_decode_step it must run before
- * the step that follows the P-th buffered token. The update stages the P
- * buffered queries, then rows of keys, in shared memory: the larger of
- * P * head_dim * elem and 256 * (head_dim * elem + 16) bytes, plus 16 bytes
- * per token of the longest segment, must fit in 227 KB, else
- * HKV_ERR_CAPACITY (also for hkv_append_evict and hkv_repack). */
+ * the step that follows the P-th buffered token. The P buffered queries and
+ * a record of every row are held in shared memory, so their size is limited:
+ * the larger of P * head_dim * elem and 256 * (head_dim * elem + 16) bytes,
+ * plus 16 bytes per token of the longest segment, plus 4 * head_dim + 2112
+ * bytes, must fit in 227 KB, else HKV_ERR_CAPACITY (also for
+ * hkv_append_evict, hkv_repack and the identification calls). */
 hkv_status hkv_evict(const hkv_config *cfg, const hkv_cache *cache, int layer, hkv_stream_t stream);
 
 /* hkv_evict for every layer in one launch (one CTA per head of the model):

@@ -171,7 +171,7 @@ constexpr int kCacheThreads = 256;
 // tokens and a query ring of P rows
 size_t update_smem_bytes(int max_len, int D, int P, int dtype);
 // the size that the interface promises to refuse above 227 KB (hkv_evict in
-// hkv.h); more than update_smem_bytes
+// hkv.h); near that limit more than update_smem_bytes
 size_t update_limit_bytes(int max_len, int D, int P, int dtype);
 cudaError_t update_prepare(int D, int dtype, size_t smem);
 

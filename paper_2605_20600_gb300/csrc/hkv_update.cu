@@ -1386,9 +1386,10 @@ size_t update_smem_bytes(int max_len, int D, int P, int dtype) {
 }
 
 size_t update_limit_bytes(int max_len, int D, int P, int dtype) {
+  // the interface's own sizes, whatever the kernels' threads and stages are
+  constexpr size_t kRows = 256;
   const size_t es = dtype == HKV_BF16 ? 2 : 4;
-  const size_t ring = (size_t)P * D * es;
-  const size_t rows = (size_t)(NT / 32) * stage_rows(max_len) * (D * es + 16);
+  const size_t ring = (size_t)P * D * es, rows = kRows * (D * es + 16);
   return (ring > rows ? ring : rows) + (size_t)max_len * 16 + (size_t)D * 4 + 512 * 4 + 64;
 }
 
