@@ -274,6 +274,10 @@ hkv_status hkv_evict_all(const hkv_config *cfg, const hkv_cache *cache, hkv_stre
  * hkv_workspace_size bytes. A compressed head whose buffer already holds P
  * tokens (hkv_evict not run) sets HKV_ERR_STATE, a full segment
  * HKV_ERR_CAPACITY, in the error word; the step is then not taken.
+ * In one launch the step's CTAs wait for each other, and all of them have to
+ * be on the GPU at once; there are no more than fit on it. Steps on several
+ * streams that share a GPU can hold each other's places until a wait runs
+ * out (HKV_ERR_TIMEOUT, 2 s)..
  * flags: 0 or HKV_STEP_PREFETCH (see above). */
 hkv_status hkv_decode_step(const hkv_config *cfg, const hkv_cache *cache, int layer,
                            const void *q, const void *k, const void *v, float *out,
@@ -295,7 +299,9 @@ int hkv_decode_step_launches(const hkv_config *cfg);
  * hkv_identify_heads over the same cache (which also reports n_h; this
  * does not). A head of another label than HKV_DENSE sets HKV_ERR_STATE in
  * the error word and the step is not taken; label_out NULL ->
- * HKV_ERR_INVALID_ARG. */
+ * HKV_ERR_INVALID_ARG. label_out is another array than the cache's label,
+ * which is read while it is written. In one launch no CTA waits for one that
+ * starts after it, so the call runs beside others on other streams. */
 hkv_status hkv_decode_step_identify(const hkv_config *cfg, const hkv_cache *cache, int layer,
                                     const void *q, const void *k, const void *v, float *out,
                                     uint8_t *label_out, void *workspace, size_t ws_bytes,

@@ -254,6 +254,11 @@ hkv_status one_launch_plan(const hkv_config *cfg, bool fused, bool identify, Ste
   s = step_ctas(st, cfg->head_dim, cfg->dtype, &ctas);
   if (s != HKV_OK) return s;
   int full = st->sms.load(std::memory_order_acquire) * ctas;
+#ifdef HKV_STEP_TEST_WAVES
+  // test builds only: more CTAs than are resident at once, where none waits
+  // for a higher-numbered one
+  if (!fused || identify) full *= HKV_STEP_TEST_WAVES;
+#endif
   if (full > kAttnMaxGrid) full = kAttnMaxGrid;
   *plan = step_plan(cfg->head_dim, cfg->dtype, heads_per_layer(cfg), max_segment(*cfg), full, fused,
                     identify);

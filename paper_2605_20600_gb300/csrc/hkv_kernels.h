@@ -60,8 +60,9 @@ struct AttnArgs {
   // one-launch step (hkv_step.cu): the layer's barrier words (the attention
   // alone: its own, for every layer, with n_layers 1 and layer 0) {arrivals,
   // generation, worst status of a bad step, heads taken, arrivals and
-  // generation of the CTAs that take no more, unused, unused}, all but the
-  // generations zero between launches; the partial results of split heads
+  // generation of the CTAs that take no more, epoch of a launch with a CTA that
+  // did not wait for the arrivals, unused}, all but the generations and the
+  // epoch zero between launches; the partial results of split heads
   // as (value, launch epoch) pairs, two slots per CTA (the piece at the end
   // of its range, the piece at its start), [grid][2][step_piece_words(D)]
   uint32_t *bar;
@@ -110,7 +111,9 @@ constexpr int kAttnInlinePieces = 4;
 #endif
 constexpr int kStepTable = HKV_STEP_TABLE;
 // 64-bit words of one partial result of the one-launch step: D accumulators,
-// the maximum, the sum and (identification) the newest rows' sum
+// the maximum, the sum and (identification) the newest rows' sum; then
+// identification's word between a CTA and the last one to arrive (slot 0 of
+// the CTA) and the heads the CTA left to that one (slot 1)
 __host__ __device__ constexpr int step_piece_words(int D) { return D + 4; }
 
 size_t attention_smem_bytes(int D, int dtype);

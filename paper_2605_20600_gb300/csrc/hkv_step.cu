@@ -41,9 +41,9 @@
 //    never waits for a piece that finishes last in its CTA (measured: 0.3
 //    us per step less than the other order at rho = 1/8);
 //  * merges: a split head is combined by its first middle CTA (whose whole
-//    range lies inside the head), else (and in the attention alone) by the
-//    CTA holding its last row. The
-//    other pieces write their partial result to the workspace as 64-bit
+//    range lies inside the head), else (and always in the attention alone and
+//    in the step that decides the head types) by the CTA holding its last
+//    row. The other pieces write their partial result to the workspace as 64-bit
 //    (value, launch epoch) pairs, which are single-copy atomic, so no fence
 //    or flag is needed: the combining CTA's merge warp reads the pieces until
 //    every pair carries this launch's epoch, while its consumers stream.
@@ -63,8 +63,12 @@
 //    arrival and the first tiles of old K/V rows go ahead of the wait for the
 //    previous kernel; the step's inputs (q, the new k and v) are read after
 //    it;
-//  * every wait is bounded (HKV_ERR_TIMEOUT in the error word). A step's waits
-//    on other CTAs need the whole grid resident: it is at most what fits.
+//  * every wait is bounded (HKV_ERR_TIMEOUT in the error word). A plain step's
+//    waits on other CTAs need the whole grid resident: it is at most what
+//    fits. In the attention alone and in the step that decides the head types
+//    a CTA waits for lower-numbered ones only, which start before it; what
+//    the latter's barrier holds up is left to the last CTA to arrive (see the
+//    merge warp).
 #include <math.h>
 #include <stdlib.h>
 
@@ -237,6 +241,15 @@ __device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t *p, uint32_t v) {
   asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
   return old;
 }
+__device__ __forceinline__ unsigned long long atom_exch_acq_rel(unsigned long long *p,
+                                                               unsigned long long v) {
+  unsigned long long old;
+  asm volatile("atom.acq_rel.gpu.global.exch.b64 %0, [%1], %2;"
+               : "=l"(old)
+               : "l"(p), "l"(v)
+               : "memory");
+  return old;
+}
 __device__ __forceinline__ void st_release(uint32_t *p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -348,6 +361,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   __shared__ float own_s[NV], oth_s[NV];
   __shared__ int s_own_state;  // 1: combined by the epilogue, 2: own piece handed over
   __shared__ volatile int s_abort;
+  __shared__ volatile int s_streamed;  // (identification) the epilogue is done
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nheads = p.nheads;
@@ -404,6 +418,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     mbar_init(&own_bar, 32);
     fence_barrier_init();
     s_abort = 0;
+    s_streamed = 0;
     s_bad = 0;
     s_mg_h = -1;
   };
@@ -806,9 +821,9 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   // ---- merge warp: the launch's epoch and the split head this CTA combines --
   // The split head: the first of the range when this CTA is that head's
   // first middle CTA (its whole range inside the head) or, for a head in two
-  // pieces and in the attention alone, holds its last row: CTAs then wait for
-  // lower-numbered ones only, which start before them, so that launches of the
-  // attention that share the GPU never hold each other's places. The epoch,
+  // pieces and in all but the plain step, holds its last row: CTAs then wait
+  // for lower-numbered ones only, which start before them, so that launches
+  // that share the GPU never hold each other's places. The epoch,
   // from the generation of the barrier word, is unique per (layer, launch of
   // that layer), or among the attentions alone, which have words and slots of
   // their own (p.n_layers is 1 there, whatever the layer); the
@@ -826,6 +841,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   constexpr uint32_t kBadStep = 0x80000000u;  // in the generation: step not taken
   uint32_t gen0 = 0, gen1 = 0;
   int bar_done = 0;
+  int hinted = 0;  // identification: the last CTA to arrive found the hint (see the merge warp)
   auto arrive = [&]() {  // lane 0 of the merge warp
     const uint32_t inc = own_bad ? 0x10001u : 1u;
     if (own_bad) {
@@ -876,7 +892,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         const long long x1 = (long long)k1 * chunk;
         if (x1 > s0 && x1 >= er - tol) --k1;  // that one to its end
         const int np = k1 - k0 + 1;
-        if ((FUSED && np >= 3 ? k0 + 1 : k1) == bx) {
+        if ((MODE == kModeStep && np >= 3 ? k0 + 1 : k1) == bx) {
           s_mg_k0 = k0;
           s_mg_np = np;
           s_mg_j = bx - k0;
@@ -889,6 +905,10 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     }
     __syncwarp();
     mbar_arrive(&ep_bar);  // all 32 lanes: the epilogue may read s_ep, s_mg_*
+    if (IDENT && lane == 0 && bar_done) {
+      __threadfence();  // the generation before the hint
+      hinted = ld_acquire(p.bar + 6) == s_ep;
+    }
   }
 
   if (p.prefetch) pdl_wait();  // the step's inputs are visible from here on
@@ -1265,6 +1285,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         }
       }
     }
+    if (IDENT && lane == 0) s_streamed = 1;
     if (lane == 0) STEP_TRACE(5);
     STEP_TRACE_SET(9, k);
     if (lane == 0) STEP_TRACE_SET(23, w_epi);
@@ -1309,18 +1330,21 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     const int napp = DYN ? sh1 - sh0 : active ? (has_e ? n - 1 : n) : 0;
     const int app0 = DYN ? sh0 : h0;
     // a head's last row (the step's token) in the arena, and its image tokens
-    auto last_row = [&](int h) {
-      return DYN ? p.off[h] + p.len[h] : tab.off[h - wl] + tab.vlen[h - wl] - 1;
+    // (known: the head is in the table)
+    auto last_row = [&](int h, bool known) {
+      return DYN || !known ? p.off[h] + p.len[h] : tab.off[h - wl] + tab.vlen[h - wl] - 1;
     };
-    auto tokens_of = [&](int h) { return DYN ? p.ntok[p.layer_base + h] : tab.ntok[h - wl]; };
-    // Appends: the K/V row at index len, its position, q into the ring of the
-    // periodic update. Nothing in this launch reads them.
-    auto append = [&]() {
+    auto tokens_of = [&](int h, bool known) {
+      return DYN || !known ? p.ntok[p.layer_base + h] : tab.ntok[h - wl];
+    };
+    // Appends of `count` heads: the K/V row at index len, its position, q into
+    // the ring of the periodic update. Nothing in this launch reads them.
+    auto append = [&](int first, int count, bool known) {
       // the K, V and q rows of every appended head as 16-byte chunks, a
       // lane per chunk, every load of a round issued before its stores
       constexpr int CH = RB / 16;  // chunks of a row
-      constexpr int NU = 8;        // chunks per lane and round
-      const int units = napp * 3 * CH;
+      constexpr int NU = IDENT ? 4 : 8;  // chunks per lane and round (registers)
+      const int units = count * 3 * CH;
       for (int u0 = 0; u0 < units; u0 += 32 * NU) {
         uint4 x[NU];
         unsigned char *dst[NU];
@@ -1330,16 +1354,16 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
           dst[v] = nullptr;
           if (u < units) {
             const int w3 = (u / CH) % 3, cc = u % CH;
-            const int h = app0 + u / (3 * CH), i = p.layer_base + h;
+            const int h = first + u / (3 * CH), i = p.layer_base + h;
             const unsigned char *src = w3 == 0 ? static_cast<const unsigned char *>(p.k_new)
                                      : w3 == 1 ? static_cast<const unsigned char *>(p.v_new)
                                                : static_cast<const unsigned char *>(p.q);
             x[v] = reinterpret_cast<const uint4 *>(src + (size_t)h * RB)[cc];
-            const long long row = last_row(h);
+            const long long row = last_row(h, known);
             unsigned char *d = w3 == 0 ? static_cast<unsigned char *>(p.K) + row * RB
                              : w3 == 1 ? static_cast<unsigned char *>(p.V) + row * RB
                                        : static_cast<unsigned char *>(p.qbuf) +
-                                             ((size_t)i * p.period + tokens_of(h) % p.period) * RB;
+                                             ((size_t)i * p.period + tokens_of(h, known) % p.period) * RB;
             dst[v] = d + (size_t)cc * 16;
           }
         }
@@ -1347,17 +1371,18 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         for (int v = 0; v < NU; ++v)
           if (dst[v]) *reinterpret_cast<uint4 *>(dst[v]) = x[v];
       }
-      for (int h = app0 + lane; h < app0 + napp; h += 32)
-        p.pos[last_row(h)] = p.n_cond + tokens_of(h);
+      for (int h = first + lane; h < first + count; h += 32)
+        p.pos[last_row(h, known)] = p.n_cond + tokens_of(h, known);
     };
-    auto advance = [&]() {  // the counters of the appended heads
-      for (int h = app0 + lane; h < app0 + napp; h += 32) {
+    // the counters of `count` heads whose tokens are appended
+    auto advance = [&](int first, int count, bool known) {
+      for (int h = first + lane; h < first + count; h += 32) {
         const int i = p.layer_base + h;
         if (DYN && h < sh0 + 32) {
           p.len[h] = k_len + 1;
           p.ntok[i] = k_nt + 1;
           if (k_nb >= 0) p.nbuf[i] = k_nb + 1;
-        } else if (DYN) {
+        } else if (DYN || !known) {
           ++p.len[h];
           ++p.ntok[i];
           if (p.label[i] != HKV_DENSE) ++p.nbuf[i];
@@ -1373,11 +1398,35 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     // them). With in_regs every CTA has checked every head, so the step is
     // known to be taken and the appends need not wait for that; otherwise the
     // barrier also tells whether some CTA found a bad head.
-    bool advanced = !FUSED;
+    //
+    // Identification holds no CTA back for that: one that has streamed its
+    // range before the grid has arrived leaves the rest of its share (appends
+    // unless in_regs, counters) to the last CTA to arrive and ends, which may
+    // be what lets that one start (launches on other streams can hold its
+    // place). It says so in the layer's hint word and looks for the arrivals
+    // once more, and the last CTA publishes them before it reads the hint, so
+    // one of the two sees the other. Where both do, they settle it on a word
+    // of the CTA's: whoever exchanges it second sees the other's mark, tagged
+    // with the epoch, and does the share. (Without the hint, the last CTA's
+    // walk over all words cost 3.8 us of a layer step of 9.7.)
+    bool advanced = !FUSED || (IDENT && napp == 0);
+    const unsigned long long tag = (unsigned long long)s_ep << 32;
+    constexpr unsigned kLeft = 1, kArrived = 2;
+    auto hand_word = [&](int k, int sl) { return p.pslot + ((size_t)k * 2 + sl) * PS + D + 3; };
+    auto settle = [&](int first, int count, bool known) {  // once the grid has arrived
+      if (IDENT && (__shfl_sync(0xFFFFFFFFu, gen1, 0) & kBadStep)) return;
+      if (IDENT && !in_regs) append(first, count, known);
+      advance(first, count, known);
+    };
     if (FUSED && in_regs) {
-      append();
+      append(app0, napp, true);
       if (poll()) {
-        advance();
+        advance(app0, napp, true);
+        advanced = true;
+      }
+    } else if (IDENT) {
+      if (!advanced && poll()) {
+        settle(app0, napp, true);
         advanced = true;
       }
     } else if (FUSED) {
@@ -1386,7 +1435,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       gen1 = __shfl_sync(0xFFFFFFFFu, gen1, 0);
       STEP_TRACE_SET(19, globaltimer());
       if (!s_abort && bar_done && !(gen1 & kBadStep)) {
-        append();
+        append(app0, napp, true);
         if (DYN) {  // the lengths advance once no CTA reads another
           bool all = false;
           while (!s_abort && !all) {
@@ -1394,12 +1443,29 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
             if (!all && timed_out()) break;
           }
           __syncwarp();
-          if (all) advance();
+          if (all) advance(app0, napp, true);
         } else {
-          advance();
+          advance(app0, napp, true);
         }
       }
       advanced = true;
+    }
+    if constexpr (IDENT) {
+      if (__shfl_sync(0xFFFFFFFFu, hinted, 0)) {
+        for (int k0 = 0; k0 < G; k0 += 32) {
+          const int k = k0 + lane;
+          unsigned long long share = 0;
+          if (k < G && k != bx &&
+              atom_exch_acq_rel(hand_word(k, 0), tag | kArrived) == (tag | kLeft))
+            share = *hand_word(k, 1);
+          unsigned left = __ballot_sync(0xFFFFFFFFu, share != 0);
+          while (left) {
+            const unsigned long long w = __shfl_sync(0xFFFFFFFFu, share, __ffs(left) - 1);
+            left &= left - 1;
+            settle((int)(w >> 32), (int)(uint32_t)w, false);
+          }
+        }
+      }
     }
     STEP_TRACE_SET(8, globaltimer());
 
@@ -1447,7 +1513,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         }
         if (ready || timed_out()) break;
         if (!advanced && poll()) {
-          advance();
+          settle(app0, napp, true);
           advanced = true;
         }
       }
@@ -1479,10 +1545,30 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       }
     }
     if (!advanced) {
-      while (!s_abort && !poll())
+      while (!s_abort && !poll()) {
+        if (IDENT && __shfl_sync(0xFFFFFFFFu, s_streamed, 0)) break;
         if (timed_out()) break;
+      }
       STEP_TRACE_SET(19, globaltimer());
-      if (!s_abort && bar_done) advance();
+      if (!s_abort && bar_done) {
+        settle(app0, napp, true);
+      } else if (IDENT && !s_abort) {
+        if (lane == 0) {
+          st_release(p.bar + 6, s_ep);
+          __threadfence();  // the hint before the generation
+        }
+        if (!poll()) {
+          if (lane == 0) {
+            *hand_word(bx, 1) = (unsigned long long)app0 << 32 | (uint32_t)napp;
+            if (atom_exch_acq_rel(hand_word(bx, 0), tag | kLeft) == (tag | kArrived)) {
+              gen1 = ld_acquire(p.bar + 1);
+              bar_done = 1;
+            }
+          }
+          bar_done = __shfl_sync(0xFFFFFFFFu, bar_done, 0);
+        }
+        if (bar_done) settle(app0, napp, true);  // the grid has arrived meanwhile
+      }
     }
     if (lane == 0) STEP_TRACE(6);
   }
