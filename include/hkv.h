@@ -325,8 +325,9 @@ hkv_status hkv_decode_attention(const hkv_config *cfg, const hkv_cache *cache, i
  * of heads split between CTAs and the kernels' control block live in a
  * fixed device array inside the library (2.06 MiB: 1 MiB of partials for
  * each of the two designs, 64 KiB of records, 256 bytes), which every GPU
- * that loads the library holds until the process exits. The caller
- * initialises nothing. Same inputs, outputs and results as
+ * that loads the library holds until the process exits. Nothing in it has to
+ * start at zero and nothing is kept from call to call: each call clears or
+ * writes what it reads. Same inputs, outputs and results as
  * hkv_decode_attention; it allocates nothing.
  *  - The first call on a device, with that device current, looks up the
  *    array's device address and prepares the kernel; make that first call
