@@ -1399,19 +1399,23 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
     // known to be taken and the appends need not wait for that; otherwise the
     // barrier also tells whether some CTA found a bad head.
     //
-    // Identification holds no CTA back for that: one that has streamed its
-    // range before the grid has arrived leaves the rest of its share (appends
-    // unless in_regs, counters) to the last CTA to arrive and ends, which may
-    // be what lets that one start (launches on other streams can hold its
-    // place). It says so in the layer's hint word and looks for the arrivals
+    // Identification holds no CTA back for that for long: one that has streamed
+    // its range and sees no end of the arrivals for kHoldNs more leaves the rest
+    // of its share (appends unless in_regs, counters) to the last CTA to arrive
+    // and ends, which may be what lets that one start (launches on other
+    // streams can hold its place). A launch that has the GPU to itself has
+    // arrived by then; without the hold its first CTAs left their shares to one
+    // warp (12 sequences of Janus-Pro-7B: 9.2 us a layer, 17 without). A CTA
+    // that leaves says so in the layer's hint word and looks for the arrivals
     // once more, and the last CTA publishes them before it reads the hint, so
-    // one of the two sees the other. Where both do, they settle it on a word
-    // of the CTA's: whoever exchanges it second sees the other's mark, tagged
-    // with the epoch, and does the share. (Without the hint, the last CTA's
-    // walk over all words cost 3.8 us of a layer step of 9.7.)
+    // one of the two sees the other. Where both do, they settle it on a word of
+    // the CTA's: whoever exchanges it second sees the other's mark, tagged with
+    // the epoch, and does the share. (Without the hint, the last CTA's walk over
+    // all words cost 3.8 us of a layer step of 9.7.)
     bool advanced = !FUSED || (IDENT && napp == 0);
     const unsigned long long tag = (unsigned long long)s_ep << 32;
     constexpr unsigned kLeft = 1, kArrived = 2;
+    constexpr uint64_t kHoldNs = 20000;
     auto hand_word = [&](int k, int sl) { return p.pslot + ((size_t)k * 2 + sl) * PS + D + 3; };
     auto settle = [&](int first, int count, bool known) {  // once the grid has arrived
       if (IDENT && (__shfl_sync(0xFFFFFFFFu, gen1, 0) & kBadStep)) return;
@@ -1545,8 +1549,17 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
       }
     }
     if (!advanced) {
+      uint64_t hold = 0;  // lane 0: the end of the hold
       while (!s_abort && !poll()) {
-        if (IDENT && __shfl_sync(0xFFFFFFFFu, s_streamed, 0)) break;
+        if constexpr (IDENT) {
+          bool leave = false;
+          if (lane == 0 && s_streamed) {
+            const uint64_t now = globaltimer();
+            if (hold == 0) hold = now + kHoldNs;
+            leave = now >= hold;
+          }
+          if (__shfl_sync(0xFFFFFFFFu, leave, 0)) break;
+        }
         if (timed_out()) break;
       }
       STEP_TRACE_SET(19, globaltimer());
