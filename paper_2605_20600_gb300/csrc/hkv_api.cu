@@ -245,7 +245,7 @@ hkv_status step_ctas(DeviceState *st, int D, int dtype, int *ctas) {
 // model shape measured. HKV_STEP_TWO_KERNELS in the environment forces the
 // two-kernel design (tests of both).
 hkv_status one_launch_plan(const hkv_config *cfg, bool fused, bool identify, StepPlan *plan) {
-  *plan = {0, 0};
+  *plan = {0, 0, 0};
   if (getenv("HKV_STEP_TWO_KERNELS")) return HKV_OK;
   DeviceState *st;
   hkv_status s = device_state(&st);

@@ -132,6 +132,7 @@ cudaError_t step_prepare(int D, int dtype, int *ctas_per_sm);
 struct StepPlan {
   int grid;
   int cut;
+  int lone;  // one CTA an SM, which shared memory keeps to itself
 };
 StepPlan step_plan(int D, int dtype, int nheads, int max_rows, int full, bool fused, bool identify);
 // one layer in one launch: the decode step (append + attention, merges of

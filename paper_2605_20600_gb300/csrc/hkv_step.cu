@@ -200,6 +200,23 @@ struct StepShape : StepTile<D, T, SHORT> {
 #define HKV_STEP_HEAD_SLOTS 160
 #endif
 constexpr int kHeadSlots = HKV_STEP_HEAD_SLOTS, kHeadGrains = 16;
+// Rows of 512 bytes (grains of 8) are better cut as long as the table holds
+// every range's heads: heads of up to 112 rows, 3600 of them (177 slots) 44.0
+// us cut and 46.6 head by head, 6000 73.8 and 76.2, 9000 (444) 111.1 and 113.4.
+constexpr int kHeadSlots512 = 3 * (kStepTable - 2);  // of ranges, at 3 slots a head at least
+
+// Rows of 512 bytes: a small layer gets one CTA an SM, which shared memory
+// then keeps to itself, else two. Two halve a range; that loses where a
+// head falls into more than three ranges (fewer heads than a third of the
+// CTAs) or a range is short anyway (fewer than kLoneSlots slots an SM). Per
+// layer step, one -> two: Lumina-mGPT 768 with 1 sequence 6.24 -> 6.78 us, 3
+// (96 heads) 9.08 -> 9.24, 4 11.0 -> 10.3, 12 28.7 -> 23.4; Lumina-mGPT 1024
+// with 1 8.85 -> 9.98, 3 13.9 -> 14.0, 4 17.4 -> 16.7, 10 41.7 -> 35.2;
+// Janus-Pro-7B with 4 (19 slots) 6.08 -> 6.31, 8 (37) 8.3 -> 8.3, 10 (46)
+// 10.7 -> 9.3, 40 30.3 -> 28.2. One CTA an SM beside one of the next launch's
+// is slower than either (Lumina-mGPT 768 with 3: 9.85).
+constexpr int kLoneSlots = 40;
+constexpr size_t kLoneSmem = 104 * 1024;  // dynamic; twice that is more than an SM has
 
 // A boundary between ranges that falls within 1/kSnapDiv of a range of a
 // head's first or last row moves there.
@@ -212,8 +229,9 @@ struct StepTable {  // entry h - s_wl: head h
   long long off[N];  // arena offset
   int vlen[N];       // rows, the new token included
   int ntok[N];
-  unsigned char label[N];
-  unsigned char bad[N];  // status of the head's counters
+  // the status of the head's counters, doubled, and 1 for a compressed head
+  // (one byte: with two, rows of 512 bytes had room for one CTA an SM only)
+  unsigned char state[N];
 };
 
 // kWhole: the piece is its whole head; kTailPiece: the head began in an
@@ -495,11 +513,8 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         const int e = verify(l, o, cp, lab, nb);
         tab.vlen[tid] = l + kNew;
         tab.off[tid] = o;
-        tab.bad[tid] = (unsigned char)e;
-        if (FUSED) {
-          tab.ntok[tid] = nt;
-          tab.label[tid] = (unsigned char)lab;
-        }
+        tab.state[tid] = (unsigned char)(e << 1 | (FUSED && lab != HKV_DENSE));
+        if (FUSED) tab.ntok[tid] = nt;
         if (in_regs) {
           const int g = S::grains(l + kNew);
           const int st = e ? e : g > kMost ? (int)HKV_ERR_BOUNDS : 0;
@@ -602,8 +617,8 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
           const int v = !in ? 0 : here ? tab.vlen[j] : p.len[h] + kNew;
           const int c = in ? S::cost(S::grains(v)) : 0;
           const int incl = warp_incl_scan(c);
-          if (in && place(h, at + incl - c, v) && FUSED && !in_regs && here && tab.bad[j])
-            atomicMax(&s_bad, (int)tab.bad[j]);
+          if (in && place(h, at + incl - c, v) && FUSED && !in_regs && here && tab.state[j] >> 1)
+            atomicMax(&s_bad, tab.state[j] >> 1);
           return __shfl_sync(0xFFFFFFFFu, incl, 31);
         };
         if (in_regs) {
@@ -656,7 +671,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
             const int e = verify(l, o, cp, lab, nb);
             if (e) atomicMax(&s_bad, e);
             tab.ntok[tid] = nt;
-            tab.label[tid] = (unsigned char)lab;
+            tab.state[tid] = lab != HKV_DENSE;
           }
         }
         __syncthreads();
@@ -1390,7 +1405,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
           const int j = h - wl;
           p.len[h] = tab.vlen[j];
           p.ntok[i] = tab.ntok[j] + 1;
-          if (tab.label[j] != HKV_DENSE) ++p.nbuf[i];
+          if (tab.state[j] & 1) ++p.nbuf[i];
         }
       }
     };
@@ -1587,17 +1602,21 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   }
 }
 
-template <int D, typename T, int CUT>
-size_t step_smem() {
-  using S = StepShape<D, T, CUT == kCutShort>;
+template <class S>
+constexpr size_t step_smem_of() {
   return (size_t)S::kNS * S::kStageBytes;
+}
+template <int D, typename T, int CUT>
+constexpr size_t step_smem() {
+  return step_smem_of<StepShape<D, T, CUT == kCutShort>>();
 }
 
 template <int D, typename T, int MODE, int CUT>
 cudaError_t step_prepare_m(int *ctas) {
   const size_t smem = step_smem<D, T, CUT>();
+  const size_t most = smem > kLoneSmem ? smem : kLoneSmem;
   cudaError_t e = cudaFuncSetAttribute(step_kernel<D, T, MODE, CUT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
   if (e != cudaSuccess) return e;
   int n = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_kernel<D, T, MODE, CUT>,
@@ -1618,12 +1637,12 @@ cudaError_t step_prepare_t(int *ctas) {
 }
 
 template <int D, typename T, int MODE, int CUT>
-cudaError_t step_launch_m(const AttnArgs &a, int grid, cudaStream_t s) {
+cudaError_t step_launch_m(const AttnArgs &a, StepPlan plan, cudaStream_t s) {
   static const bool pdl = getenv("HKV_NO_PDL") == nullptr;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = dim3(plan.grid);
   cfg.blockDim = dim3(step_threads<D, T>());
-  cfg.dynamicSmemBytes = step_smem<D, T, CUT>();
+  cfg.dynamicSmemBytes = plan.lone ? kLoneSmem : step_smem<D, T, CUT>();
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   int na = 0;
@@ -1638,31 +1657,36 @@ cudaError_t step_launch_m(const AttnArgs &a, int grid, cudaStream_t s) {
 }
 
 template <int D, typename T>
-cudaError_t step_launch_t(AttnArgs a, int grid, bool fused, int cut, cudaStream_t s) {
-  a.grid_recip = (uint32_t)(((1ull << 32) + grid - 1) / grid);  // (not used for a grid of one)
-  if (!fused) return step_launch_m<D, T, kModeAttend, kCutRanges>(a, grid, s);
-  if (a.label_out) return step_launch_m<D, T, kModeIdentify, kCutRanges>(a, grid, s);
-  return cut == kCutShort   ? step_launch_m<D, T, kModeStep, kCutShort>(a, grid, s)
-         : cut == kCutHeads ? step_launch_m<D, T, kModeStep, kCutHeads>(a, grid, s)
-                            : step_launch_m<D, T, kModeStep, kCutRanges>(a, grid, s);
+cudaError_t step_launch_t(AttnArgs a, StepPlan plan, bool fused, cudaStream_t s) {
+  a.grid_recip = (uint32_t)(((1ull << 32) + plan.grid - 1) / plan.grid);  // (not used for a grid of one)
+  if (!fused) return step_launch_m<D, T, kModeAttend, kCutRanges>(a, plan, s);
+  if (a.label_out) return step_launch_m<D, T, kModeIdentify, kCutRanges>(a, plan, s);
+  return plan.cut == kCutShort   ? step_launch_m<D, T, kModeStep, kCutShort>(a, plan, s)
+         : plan.cut == kCutHeads ? step_launch_m<D, T, kModeStep, kCutHeads>(a, plan, s)
+                                 : step_launch_m<D, T, kModeStep, kCutRanges>(a, plan, s);
 }
 
 // The CTAs a layer of n heads gets out of a full grid: see step_plan.
 template <int D, typename T>
 StepPlan step_plan_t(long long n, long long max_rows, int full, bool fused, bool identify) {
   using S = StepShape<D, T>;
+  static_assert(step_smem_of<S>() <= kLoneSmem, "a lone CTA's shared memory holds its stages");
   const long long g = (max_rows + S::kGR - 1) / S::kGR;
   const long long total = n * (g + 1 > S::kMinCost ? g + 1 : S::kMinCost);
-  if (fused && !identify && total >= (long long)kHeadSlots * full && g <= kHeadGrains)
-    return {full, kCutHeads};
+  const int sms = full / kStepActivePerSm > 1 ? full / kStepActivePerSm : 1;
+  const bool lone = S::kRB == 512 && (total < (long long)kLoneSlots * sms || 3 * n < full);
+  if (lone) full = sms;
+  const int head_slots = S::kRB == 512 ? kHeadSlots512 : kHeadSlots;
+  if (fused && !identify && total >= (long long)head_slots * full && g <= kHeadGrains)
+    return {full, kCutHeads, 0};
   long long chunk = (total + full - 1) / full;
   const int least = S::min_chunk(fused && !identify);
   if (chunk < least) chunk = least;
-  if (n > kStepTable && chunk / S::kMinCost + 2 > kStepTable) return {0, kCutRanges};
-  if (!fused) return {full, kCutRanges};
-  if (!identify && n <= full && n <= kStepTable && g <= kAlignedGrains) return {(int)n, kCutShort};
+  if (n > kStepTable && chunk / S::kMinCost + 2 > kStepTable) return {0, kCutRanges, 0};
+  if (!fused) return {full, kCutRanges, lone};
+  if (!identify && n <= full && n <= kStepTable && g <= kAlignedGrains) return {(int)n, kCutShort, 0};
   const long long need = (total + least - 1) / least;
-  return {need < full ? (int)need : full, kCutRanges};
+  return {need < full ? (int)need : full, kCutRanges, lone};
 }
 
 }  // namespace
@@ -1689,13 +1713,12 @@ cudaError_t step_prepare(int D, int dtype, int *ctas) {
 
 cudaError_t launch_step(const AttnArgs &a, int D, int dtype, StepPlan plan, bool fused,
                         cudaStream_t s) {
-  const int grid = plan.grid;
-  if (grid < 1 || grid > kAttnMaxGrid) return cudaErrorInvalidValue;
+  if (plan.grid < 1 || plan.grid > kAttnMaxGrid) return cudaErrorInvalidValue;
   if (dtype == HKV_BF16)
-    return D == 64 ? step_launch_t<64, __nv_bfloat16>(a, grid, fused, plan.cut, s)
-                   : step_launch_t<128, __nv_bfloat16>(a, grid, fused, plan.cut, s);
-  return D == 64 ? step_launch_t<64, float>(a, grid, fused, plan.cut, s)
-                 : step_launch_t<128, float>(a, grid, fused, plan.cut, s);
+    return D == 64 ? step_launch_t<64, __nv_bfloat16>(a, plan, fused, s)
+                   : step_launch_t<128, __nv_bfloat16>(a, plan, fused, s);
+  return D == 64 ? step_launch_t<64, float>(a, plan, fused, s)
+                 : step_launch_t<128, float>(a, plan, fused, s);
 }
 
 }  // namespace hkv
