@@ -662,9 +662,10 @@ __global__ void __launch_bounds__(NT, kUpdCtasPerSm)
 // of K and V at a time took 20 us for 256 heads of 128 tokens, which 5 us of
 // bandwidth move.
 constexpr int kPrefillBatch = 4;  // 16-byte pieces of K and of V per thread and batch
+
 template <int D, typename T>
-__global__ void __launch_bounds__(512) prefill_kernel(const CacheArgs c, int layer_base, int C, const void *kc,
-                               const void *vc) {
+__global__ void __launch_bounds__(512)
+    prefill_kernel(const CacheArgs c, int layer_base, int C, const void *kc, const void *vc) {
   constexpr int RB = D * (int)sizeof(T);
   // no early launch of the next kernel: a decode step of this layer may be it,
   // and prefetch (48 layers of 256 heads of 128 tokens: 235 us with, 234 without)
@@ -683,8 +684,9 @@ __global__ void __launch_bounds__(512) prefill_kernel(const CacheArgs c, int lay
     return;
   }
   const int pieces = C * (RB / 16);
-  const uint4 *sk = reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(kc) + (size_t)hl * C * RB);
-  const uint4 *sv = reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(vc) + (size_t)hl * C * RB);
+  const size_t src = (size_t)hl * C * RB;
+  const uint4 *sk = reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(kc) + src);
+  const uint4 *sv = reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(vc) + src);
   uint4 *dk = reinterpret_cast<uint4 *>(static_cast<unsigned char *>(c.K) + (size_t)off * RB);
   uint4 *dv = reinterpret_cast<uint4 *>(static_cast<unsigned char *>(c.V) + (size_t)off * RB);
   for (int p0 = 0; p0 < pieces; p0 += blockDim.x * kPrefillBatch) {
@@ -794,6 +796,15 @@ __device__ void grid_count_order(const int32_t *pos, int len, int C, int row_len
 // (6.1 us at the measured bandwidth): 12.1 us; with those barriers 11.8, with
 // the staged keys below 10.4 (512 threads without them 12.3).
 //
+// Two things go by the instantiation, with the same results. Short segments
+// keep the block scan, which leaves the compiler a faster loop over the rows
+// than the scan within the warps: LlamaGen-XL, 2560 heads of 110 tokens, 12.3
+// us, 14.1 with the latter. The query is loaded beside the lengths, but after
+// the checks where bf16 rows of 256 bytes are loaded straight (kLateQ):
+// Lumina-mGPT 768, 256 heads of 428 tokens, 13.5 us, 17.3 when it is early;
+// rows of 128 bytes and fp32 the other way round (14.0 early, 14.9 late;
+// Janus-Pro-7B in fp32, 16 sequences, 10.2 and 10.6).
+//
 // The logits: short segments (STAGED = false) load U row steps at a time into
 // registers; longer ones come through kIdStages stages of 32 KB filled by
 // bulk copies, so that a head's keys are on their way before the first
@@ -810,8 +821,10 @@ __global__ void __launch_bounds__(IT)
   constexpr int LPR = RB / 16;
   constexpr int RPW = 32 / LPR;
   constexpr int NW = IT / 32;
+  constexpr bool kLateQ = !STAGED && sizeof(T) == 2 && D == 128;
   extern __shared__ float e[];
-  __shared__ float s_max[NW], s_sum[NW], s_tot[2][NW];
+  __shared__ __align__(16) float s_max[NW], s_sum[NW];
+  __shared__ float s_tot[2][NW], s_scan[33];
   __shared__ int s_nh;
   __shared__ uint64_t s_full[kIdStages], s_empty[kIdStages];
   pdl_wait();
@@ -819,8 +832,12 @@ __global__ void __launch_bounds__(IT)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int hl = blockIdx.x, i = layer_base + hl;
   const int grp = lane / LPR, col = lane % LPR;
-  const uint4 qraw = *reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(q) +
-                                                      (size_t)hl * RB + col * 16);
+  auto load_q = [&]() {
+    return *reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(q) +
+                                            (size_t)hl * RB + col * 16);
+  };
+  uint4 qraw;
+  if (!kLateQ) qraw = load_q();
   const int len = c.len[i];
   const long long off = c.off[i];
   if (tid == 0) s_nh = len;
@@ -836,6 +853,7 @@ __global__ void __launch_bounds__(IT)
     if (tid == 0) set_err(c.err, HKV_ERR_CAPACITY);
     return;
   }
+  if (kLateQ) qraw = load_q();
   float qf[EPL];
   Elem<T>::unpack(qraw, qf);
 #pragma unroll
@@ -916,21 +934,21 @@ __global__ void __launch_bounds__(IT)
     // U row steps load before any is used
     for (int r0 = warp * RPW; r0 < len; r0 += U * NW * RPW) {
       uint4 kr[U];
-  #pragma unroll
+#pragma unroll
       for (int u = 0; u < U; ++u) {
         const int r = r0 + u * NW * RPW + grp;
         kr[u] = r < len ? *reinterpret_cast<const uint4 *>(K + (size_t)r * RB + col * 16)
                         : make_uint4(0u, 0u, 0u, 0u);
       }
-  #pragma unroll
+#pragma unroll
       for (int u = 0; u < U; ++u) {
         const int r = r0 + u * NW * RPW + grp;
         float kf[EPL];
         Elem<T>::unpack(kr[u], kf);
         float dot = 0.f;
-  #pragma unroll
+#pragma unroll
         for (int x = 0; x < EPL; ++x) dot = fmaf(qf[x], kf[x], dot);
-  #pragma unroll
+#pragma unroll
         for (int o = LPR / 2; o >= 1; o >>= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, o);
         if (r < len && col == 0) e[r] = dot;
       }
@@ -942,8 +960,12 @@ __global__ void __launch_bounds__(IT)
   for (int o = 16; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
   if (lane == 0) s_max[warp] = mx;
   __syncthreads();
+  float all[NW];
 #pragma unroll
-  for (int w = 0; w < NW; ++w) mx = fmaxf(mx, s_max[w]);
+  for (int w = 0; w < NW; w += 4)
+    *reinterpret_cast<float4 *>(all + w) = *reinterpret_cast<const float4 *>(s_max + w);
+#pragma unroll
+  for (int w = 0; w < NW; ++w) mx = fmaxf(mx, all[w]);
   float sum = 0.f;
   for (int r = tid; r < len; r += IT) {
     const float x = exp2f(e[r] - mx);
@@ -956,7 +978,10 @@ __global__ void __launch_bounds__(IT)
   __syncthreads();
   float thr = 0.f;
 #pragma unroll
-  for (int w = 0; w < NW; ++w) thr += s_sum[w];
+  for (int w = 0; w < NW; w += 4)
+    *reinterpret_cast<float4 *>(all + w) = *reinterpret_cast<const float4 *>(s_sum + w);
+#pragma unroll
+  for (int w = 0; w < NW; ++w) thr += all[w];
   thr *= m.tau;
   int *perm = nullptr;
   if (m.grid2d) {
@@ -970,15 +995,26 @@ __global__ void __launch_bounds__(IT)
   for (int base = 0, half = 0; base < len; base += IT, half ^= 1) {
     const int jb = base + tid;  // jb-th token counted (0 = current)
     const float x = jb < len ? e[perm ? perm[jb] : len - 1 - jb] : 0.f;
-    const float incl = warp_incl_scan(x);
-    if (lane == 31) s_tot[half][warp] = incl;
-    __syncthreads();
-    const float wv = lane < NW ? s_tot[half][lane] : 0.f;
-    const float wi = warp_incl_scan(wv);
-    const float before = __shfl_sync(0xFFFFFFFFu, wi - wv, warp);
-    const float cum = running + (before + incl - x) + x;
+    float before, tot;  // the masses before x and of the round
+    if constexpr (STAGED) {
+      const float incl = warp_incl_scan(x);
+      if (lane == 31) s_tot[half][warp] = incl;
+      __syncthreads();
+      const float wv = lane < NW ? s_tot[half][lane] : 0.f;
+      float wi = wv;
+#pragma unroll
+      for (int o = 1; o < NW; o <<= 1) {
+        const float y = __shfl_up_sync(0xFFFFFFFFu, wi, o);
+        if (lane >= o) wi += y;
+      }
+      before = __shfl_sync(0xFFFFFFFFu, wi - wv, warp) + incl - x;
+      tot = __shfl_sync(0xFFFFFFFFu, wi, NW - 1);
+    } else {
+      before = block_excl_scan<float>(x, s_scan, &tot);
+    }
+    const float cum = running + before + x;
     if (jb < len && cum >= thr) atomicMin(&s_nh, jb + 1);
-    running += __shfl_sync(0xFFFFFFFFu, wi, NW - 1);
+    running += tot;
   }
   __syncthreads();
   if (tid == 0) {
