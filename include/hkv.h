@@ -263,7 +263,8 @@ hkv_status hkv_evict_all(const hkv_config *cfg, const hkv_cache *cache, hkv_stre
  * Cache) fused with the attention of Eq. 1 over the cache including that
  * token. One kernel launch when every CTA's share of the layer spans at
  * most 256 heads (bounded from the config: the heads of a layer times the
- * rows of the longest segment it allows, over the grid), else two chained
+ * rows of the longest segment it allows, over the grid) or no segment has
+ * more than 256 rows (128 of 512 bytes), else two chained
  * kernels (attention, then a finishing kernel that combines heads split
  * across CTAs and advances the counters); hkv_decode_step_launches tells
  * which. out[s][h][:] = softmax(q k^T / sqrt(d)) V over the
@@ -277,7 +278,7 @@ hkv_status hkv_evict_all(const hkv_config *cfg, const hkv_cache *cache, hkv_stre
  * In one launch the step's CTAs wait for each other, and all of them have to
  * be on the GPU at once; there are no more than fit on it. Steps on several
  * streams that share a GPU can hold each other's places until a wait runs
- * out (HKV_ERR_TIMEOUT, 2 s)..
+ * out (HKV_ERR_TIMEOUT, 2 s).
  * flags: 0 or HKV_STEP_PREFETCH (see above). */
 hkv_status hkv_decode_step(const hkv_config *cfg, const hkv_cache *cache, int layer,
                            const void *q, const void *k, const void *v, float *out,

@@ -21,17 +21,19 @@
 //  * a layer of short heads, no more than CTAs, gets a CTA per head
 //    (kAlignedGrains), and a small layer a grid no larger than its ranges:
 //    nothing is merged and every CTA of the next launch is resident before
-//    this one ends (Janus-Pro-7B, 2 sequences: 6.6 -> 3.9 us);
+//    this one ends (Janus-Pro-7B, 2 sequences: 6.6 -> 3.4 us);
 //  * a layer of many short heads is not cut at all: CTAs take heads from a
 //    counter (kHeadSlots; Janus-Pro-7B, 256 sequences: 94.5 -> 89.0 us of 87.8
 //    at the measured bandwidth);
 //  * a warp-specialised TMA pipeline: a producer warp, consumer warps, an
 //    epilogue warp and a merge warp;
 //  * bf16 consumers take q.k on the tensor cores (8 rows a warp and tile: 4
-//    mma.sync of D = 128 in place of 64 mixed FMAs and 32 shuffles; the exact
-//    products are summed in fp32 as before) and p.V in fp32 FMAs. The chain
-//    of a tile is what a CTA waits for: 0.8 us less of Lumina-mGPT 1024's
-//    step than with FMAs and shuffles. p.V on the tensor cores too, with the
+//    mma.sync of D = 128 in place of 64 mixed FMAs and 32 shuffles) and p.V in
+//    fp32 FMAs. The products are exact; in which order and with which rounding
+//    mma.sync adds them is not specified. The outputs' error against 64 bits
+//    was 7.5e-7 at most over the timed calls before and is 6.5e-7, mostly since
+//    the exponent is rounded once. The chain of a tile is what a CTA waits for:
+//    0.8 us less of Lumina-mGPT 1024's step than with FMAs and shuffles. p.V on the tensor cores too, with the
 //    weights cut into three bf16 parts and the rows skewed against the banks,
 //    measured 1.7 us slower: the eight small copies a tile then needs;
 //  * tile order: a CTA streams the start of the head that continues into a
@@ -43,8 +45,8 @@
 //  * merges: a split head is combined by its first middle CTA (whose whole
 //    range lies inside the head), else (and always in the attention alone and
 //    in the step that decides the head types) by the CTA holding its last
-//    row. The other pieces write their partial result to the workspace as 64-bit
-//    (value, launch epoch) pairs, which are single-copy atomic, so no fence
+//    row. The other pieces write their partial result to the workspace as
+//    64-bit (value, launch epoch) pairs, which are single-copy atomic, so no fence
 //    or flag is needed: the combining CTA's merge warp reads the pieces until
 //    every pair carries this launch's epoch, while its consumers stream.
 //    Pieces are combined in index order and the CTA's own piece last, so the
@@ -109,6 +111,8 @@ __device__ unsigned long long *g_step_trace = nullptr;  // [layer][kAttnMaxGrid]
 // kStepActivePerSm). Rows of 256 B: 64-row tiles in 3 stages and 48-row ones
 // with 6 warps are within 0.3 % of each other on large layers, 64 rows 2 %
 // faster on small ones (4 stages of 48 rows +0.1 to +1.7 us, 2 stages +0.7).
+// Rows of 512 B: 32-row tiles in 3 stages leave 0 bytes of an SM beside two
+// CTAs; kLoneSlots says where one has the SM.
 // Rows of 128 B (LlamaGen-XL's short heads, many to a CTA): 128-row tiles in
 // 2 stages, 64-row ones in 3 +0.8 us. A third resident CTA per SM, so that
 // the next launch's CTAs start early, leaves some SMs with three CTAs of one
@@ -178,7 +182,10 @@ struct StepShape : StepTile<D, T, SHORT> {
   // than one more piece to combine. Periods of steps over 12 layers of
   // Lumina-mGPT 1024 at rho = 1/6, ms with 2, 3, 4, 5, 6 and 8 tiles: one
   // sequence 5.85, 5.29, 5.05, 5.34, 5.55, 6.27, two sequences 6.66, 6.26,
-  // 6.00, 6.33, 6.45, 6.94. The kernels that stop after the attention or the
+  // 6.00, 6.33, 6.45, 6.94. Other shapes, us per layer step with 3, 4 and 6:
+  // Lumina-mGPT 768 in fp32, one sequence 6.69, 6.25, 6.86, two 7.45, 7.45, 7.51;
+  // LlamaGen-XL with 32 sequences 7.19, 6.97, 7.99, but with 16 5.18, 5.75, 7.50
+  // (fp32 5.69, 6.55, 6.98). The kernels that stop after the attention or the
   // grouping are best with 3: attention over one dense sequence 214, 208, 209.
   static constexpr __host__ __device__ int min_chunk(bool step) {
     return SHORT ? kAlignedGrains : (step ? 4 : 3) * Tile::kTT / kGR;
@@ -194,8 +201,11 @@ struct StepShape : StepTile<D, T, SHORT> {
 // some 1.5 us more (lengths and claims are fetched on the way, the counters
 // advance at the end) and its CTAs end within 2 us of each other instead of
 // 5. Per layer step, cut -> head by head: Janus-Pro-7B at rho = 1/8 with 96
-// sequences (121 slots) 36.8 -> 37.1 us, with 160 (202) 59.5 -> 58.5, with 256
-// (323) 94.5 -> 89.0; LlamaGen-XL with 250 (131) 24.1 -> 24.4.
+// sequences (121 slots) 36.8 -> 37.1 us, with 128 (162) 45.6 -> 44.9, with 160
+// (202) 59.5 -> 58.5, with 256 (323) 94.5 -> 89.0; LlamaGen-XL with 250 (131)
+// 24.1 -> 24.4, with 280 (166) 25.5 -> 24.6, with 400 35.5 -> 33.8; the same in
+// fp32 with 140 (83) 21.0 -> 21.7, with 200 (118) 29.6 -> 29.2, with 280 40.7
+// -> 40.2, with 400 58.2 -> 56.9.
 #ifndef HKV_STEP_HEAD_SLOTS
 #define HKV_STEP_HEAD_SLOTS 160
 #endif
@@ -224,14 +234,28 @@ constexpr size_t kLoneSmem = 104 * 1024;  // dynamic; twice that is more than an
 #define HKV_STEP_SNAP_DIV 4
 #endif
 
-template <int N>
-struct StepTable {  // entry h - s_wl: head h
+// ONE: a head's status and label share a byte, without which rows of 512 bytes
+// had room for one CTA an SM only; elsewhere a byte each is 0.8 % faster on
+// small layers (Janus-Pro-7B, 2 sequences: 2489 and 2512 us a period).
+template <int N, bool ONE>
+struct StepTable {  // entry h - wl: head h
   long long off[N];  // arena offset
   int vlen[N];       // rows, the new token included
   int ntok[N];
-  // the status of the head's counters, doubled, and 1 for a compressed head
-  // (one byte: with two, rows of 512 bytes had room for one CTA an SM only)
-  unsigned char state[N];
+  unsigned char bad[N];  // status of the head's counters (ONE: doubled, 1 for a compressed head)
+  unsigned char label[ONE ? 1 : N];
+  __device__ __forceinline__ void set_label(int j, int lab) {
+    if (ONE) bad[j] = lab != HKV_DENSE;
+    else label[j] = (unsigned char)lab;
+  }
+  __device__ __forceinline__ void set(int j, int status, int lab) {
+    bad[j] = (unsigned char)(ONE ? status << 1 | (lab != HKV_DENSE) : status);
+    if (!ONE) label[j] = (unsigned char)lab;
+  }
+  __device__ __forceinline__ int status(int j) const { return ONE ? bad[j] >> 1 : bad[j]; }
+  __device__ __forceinline__ bool dense(int j) const {
+    return ONE ? !(bad[j] & 1) : label[j] == HKV_DENSE;
+  }
 };
 
 // kWhole: the piece is its whole head; kTailPiece: the head began in an
@@ -285,7 +309,8 @@ __device__ __forceinline__ bool ld_pair(const unsigned long long *p, uint32_t ep
   return (uint32_t)(w >> 32) == ep;
 }
 
-// One bf16 m16n8k16 product added to c. Products are exact, sums in fp32.
+// One bf16 m16n8k16 product added to c in fp32: exact products; the order and
+// rounding of their sums are the hardware's.
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4 &a, uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
       "{%8, %9}, {%0, %1, %2, %3};"
@@ -362,7 +387,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
   __shared__ __align__(16) float red_m[2][NST], red_l[2][NST], red_r[IDENT ? 2 : 1][IDENT ? NST : 1];
   __shared__ TileMeta meta[NS];
   __shared__ SegMeta seg[2];
-  __shared__ StepTable<DYN ? 1 : kThr> tab;
+  __shared__ StepTable<DYN ? 1 : kThr, RB == 512> tab;
   __shared__ int2 s_w[NW];  // each warp's slots; its longest head, or a status
   // the range's ends: {first slot, first head, that head's first slot, its
   // rows} and {end slot, last head, that head's first slot, whether the range
@@ -513,7 +538,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
         const int e = verify(l, o, cp, lab, nb);
         tab.vlen[tid] = l + kNew;
         tab.off[tid] = o;
-        tab.state[tid] = (unsigned char)(e << 1 | (FUSED && lab != HKV_DENSE));
+        tab.set(tid, e, lab);
         if (FUSED) tab.ntok[tid] = nt;
         if (in_regs) {
           const int g = S::grains(l + kNew);
@@ -617,8 +642,8 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
           const int v = !in ? 0 : here ? tab.vlen[j] : p.len[h] + kNew;
           const int c = in ? S::cost(S::grains(v)) : 0;
           const int incl = warp_incl_scan(c);
-          if (in && place(h, at + incl - c, v) && FUSED && !in_regs && here && tab.state[j] >> 1)
-            atomicMax(&s_bad, tab.state[j] >> 1);
+          if (in && place(h, at + incl - c, v) && FUSED && !in_regs && here && tab.status(j))
+            atomicMax(&s_bad, tab.status(j));
           return __shfl_sync(0xFFFFFFFFu, incl, 31);
         };
         if (in_regs) {
@@ -671,7 +696,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
             const int e = verify(l, o, cp, lab, nb);
             if (e) atomicMax(&s_bad, e);
             tab.ntok[tid] = nt;
-            tab.state[tid] = lab != HKV_DENSE;
+            tab.set_label(tid, lab);
           }
         }
         __syncthreads();
@@ -1405,7 +1430,7 @@ __global__ void __launch_bounds__(step_threads<D, T>(), HKV_STEP_RESIDENT_PER_SM
           const int j = h - wl;
           p.len[h] = tab.vlen[j];
           p.ntok[i] = tab.ntok[j] + 1;
-          if (tab.state[j] & 1) ++p.nbuf[i];
+          if (!tab.dense(j)) ++p.nbuf[i];
         }
       }
     };
@@ -1658,7 +1683,8 @@ cudaError_t step_launch_m(const AttnArgs &a, StepPlan plan, cudaStream_t s) {
 
 template <int D, typename T>
 cudaError_t step_launch_t(AttnArgs a, StepPlan plan, bool fused, cudaStream_t s) {
-  a.grid_recip = (uint32_t)(((1ull << 32) + plan.grid - 1) / plan.grid);  // (not used for a grid of one)
+  // (not used for a grid of one)
+  a.grid_recip = (uint32_t)(((1ull << 32) + plan.grid - 1) / plan.grid);
   if (!fused) return step_launch_m<D, T, kModeAttend, kCutRanges>(a, plan, s);
   if (a.label_out) return step_launch_m<D, T, kModeIdentify, kCutRanges>(a, plan, s);
   return plan.cut == kCutShort   ? step_launch_m<D, T, kModeStep, kCutShort>(a, plan, s)
