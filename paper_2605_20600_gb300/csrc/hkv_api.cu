@@ -104,6 +104,19 @@ hkv_status update_ready(DeviceState *st, int D, int dtype, size_t smem, size_t l
   return HKV_OK;
 }
 
+// the threads and shared memory of an update, append or repack over nheads
+// heads, with the kernels prepared for them
+hkv_status update_plan(const hkv_config *cfg, int nheads, int *seg, int *threads, size_t *smem) {
+  DeviceState *st;
+  const hkv_status s = device_state(&st);
+  if (s != HKV_OK) return s;
+  *seg = max_segment(*cfg);
+  *threads = update_threads(nheads, *seg, st->sms.load(std::memory_order_acquire));
+  *smem = update_smem_bytes(*threads, *seg, cfg->head_dim, cfg->period, cfg->dtype);
+  return update_ready(st, cfg->head_dim, cfg->dtype, *smem,
+                      update_limit_bytes(*seg, cfg->head_dim, cfg->period, cfg->dtype));
+}
+
 hkv_status check_cache(const hkv_cache *c) {
   if (!c || !c->k || !c->v || !c->pos || !c->off || !c->cap || !c->len || !c->nbuf || !c->ntok ||
       !c->label || !c->qbuf || !c->err)
@@ -394,15 +407,12 @@ hkv_status hkv_append_evict(const hkv_config *cfg, const hkv_cache *cache, int l
   if (layer < 0 || layer >= cfg->n_layers) return HKV_ERR_INVALID_ARG;
   if (!q || !k || !v) return HKV_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v)) return HKV_ERR_ALIGN;
-  DeviceState *st;
-  HKV_TRY(device_state(&st));
-  const int seg = max_segment(*cfg);
-  const size_t smem = update_smem_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype);
-  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem,
-                       update_limit_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype)));
   const int hpl = heads_per_layer(cfg);
+  int seg, threads;
+  size_t smem;
+  HKV_TRY(update_plan(cfg, hpl, &seg, &threads, &smem));
   return cuda_status(launch_append_evict(cache_args(cache), method_args(cfg), layer * hpl, hpl, q,
-                                         k, v, cfg->head_dim, cfg->dtype, seg, smem,
+                                         k, v, cfg->head_dim, cfg->dtype, seg, threads, smem,
                                          (cudaStream_t)stream));
 }
 
@@ -540,16 +550,13 @@ namespace {
 // the periodic update of the layers [first, first + count) in one launch
 hkv_status evict_layers(const hkv_config *cfg, const hkv_cache *cache, int first, int count,
                         hkv_stream_t stream) {
-  DeviceState *st;
-  HKV_TRY(device_state(&st));
-  const int seg = max_segment(*cfg);
-  const size_t smem = update_smem_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype);
-  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem,
-                       update_limit_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype)));
-  const long long hpl = heads_per_layer(cfg);
-  if (hpl * count > 0x7FFFFFFFLL) return HKV_ERR_SHAPE;  // one CTA per head
-  return cuda_status(launch_evict(cache_args(cache), method_args(cfg), (int)(first * hpl),
-                                  (int)(count * hpl), cfg->head_dim, cfg->dtype, seg, smem,
+  // (a validated config has at most 2^30 heads: one CTA each)
+  const int hpl = heads_per_layer(cfg), n = count * hpl;
+  int seg, threads;
+  size_t smem;
+  HKV_TRY(update_plan(cfg, n, &seg, &threads, &smem));
+  return cuda_status(launch_evict(cache_args(cache), method_args(cfg), first * hpl, n,
+                                  cfg->head_dim, cfg->dtype, seg, threads, smem,
                                   (cudaStream_t)stream));
 }
 
@@ -650,15 +657,12 @@ hkv_status repack_layers(const hkv_config *cfg, const hkv_cache *dense, const hk
   HKV_TRY(check_cache(ragged));
   if (first < 0 || first >= cfg->n_layers) return HKV_ERR_INVALID_ARG;
   if (dense->qbuf != ragged->qbuf) return HKV_ERR_INVALID_ARG;
-  DeviceState *st;
-  HKV_TRY(device_state(&st));
-  const int seg = max_segment(*cfg);
-  const size_t smem = update_smem_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype);
-  HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, smem,
-                       update_limit_bytes(seg, cfg->head_dim, cfg->period, cfg->dtype)));
-  const int hpl = heads_per_layer(cfg);
+  const int hpl = heads_per_layer(cfg), n = count * hpl;
+  int seg, threads;
+  size_t smem;
+  HKV_TRY(update_plan(cfg, n, &seg, &threads, &smem));
   return cuda_status(launch_repack(cache_args(dense), cache_args(ragged), method_args(cfg),
-                                   first * hpl, count * hpl, cfg->head_dim, cfg->dtype, seg, smem,
+                                   first * hpl, n, cfg->head_dim, cfg->dtype, seg, threads, smem,
                                    (cudaStream_t)stream));
 }
 

@@ -173,7 +173,9 @@ constexpr int kCacheThreads = 256;
 
 // dynamic shared memory of the update paths for segments of up to max_len
 // tokens and a query ring of P rows
-size_t update_smem_bytes(int max_len, int D, int P, int dtype);
+size_t update_smem_bytes(int threads, int max_len, int D, int P, int dtype);
+// threads of a CTA for a launch over nheads heads on `sms` SMs
+int update_threads(int nheads, int max_len, int sms);
 // the size that the interface promises to refuse above 227 KB (hkv_evict in
 // hkv.h); near that limit more than update_smem_bytes
 size_t update_limit_bytes(int max_len, int D, int P, int dtype);
@@ -181,12 +183,12 @@ cudaError_t update_prepare(int D, int dtype, size_t smem);
 
 cudaError_t launch_append_evict(const CacheArgs &c, const MethodArgs &m, int layer_base,
                                 int nheads, const void *q, const void *k, const void *v, int D,
-                                int dtype, int max_len, size_t smem, cudaStream_t s);
+                                int dtype, int max_len, int threads, size_t smem, cudaStream_t s);
 cudaError_t launch_evict(const CacheArgs &c, const MethodArgs &m, int layer_base, int nheads,
-                         int D, int dtype, int max_len, size_t smem, cudaStream_t s);
+                         int D, int dtype, int max_len, int threads, size_t smem, cudaStream_t s);
 cudaError_t launch_repack(const CacheArgs &dense, const CacheArgs &ragged, const MethodArgs &m,
-                          int layer_base, int nheads, int D, int dtype, int max_len, size_t smem,
-                          cudaStream_t s);
+                          int layer_base, int nheads, int D, int dtype, int max_len, int threads,
+                          size_t smem, cudaStream_t s);
 cudaError_t launch_prefill(const CacheArgs &c, int layer_base, int nheads, int C, const void *kc,
                            const void *vc, int D, int dtype, cudaStream_t s);
 cudaError_t launch_init_dense(const CacheArgs &c, int nheads_total, int seg_tokens,

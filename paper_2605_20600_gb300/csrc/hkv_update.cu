@@ -30,24 +30,25 @@
 namespace hkv {
 namespace {
 
-// threads of the update kernels, and of the identification kernels (whose
-// sums' order goes with it)
-#ifndef HKV_UPD_THREADS
-#define HKV_UPD_THREADS 128
-#endif
-constexpr int NT = HKV_UPD_THREADS;
-constexpr int IT = kCacheThreads;
-// Update kernels resident per SM that the register budget allows (48 registers
-// a thread, no spills). An update is a chain of latency-bound phases between
-// block barriers, so what counts is how many run at once: CTAs of four warps,
-// up to ten on an SM, rather than eight warps staging whole rows of keys in 70
-// KB, two or three on an SM. Lumina-mGPT 1024, 8 sequences, all layers: 475 ->
-// 327 us (of 264 at the measured bandwidth); with 256 threads and four CTAs
-// 339. LlamaGen-XL's 92160 heads of up to 121 rows: 1.34 -> 0.9 ms a period.
-#ifndef HKV_UPD_CTAS
-#define HKV_UPD_CTAS 10
-#endif
-constexpr int kUpdCtasPerSm = HKV_UPD_CTAS;
+constexpr int IT = kCacheThreads;  // of the identification kernels (their sums' order goes with it)
+
+// Threads of an update CTA (NT below: 128, 256 or 512; the results do not
+// depend on it) and how many CTAs the register budget allows on an SM (48
+// registers a thread, 64 with 512; no spills). An update is a chain of
+// latency-bound phases between block barriers. With many heads for every SM
+// what counts is how many run at once: CTAs of four warps, up to ten on an SM,
+// rather than eight warps staging whole rows of keys in 70 KB, two or three on
+// an SM. Lumina-mGPT 1024, 8 sequences, all layers: 475 -> 327 us (of 264 at
+// the measured bandwidth); with 256 threads and four CTAs 339. LlamaGen-XL's
+// 92160 heads of up to 121 rows: 1.34 -> 0.9 ms a period. With few heads a head
+// has an SM nearly to itself and more warps pass over its rows at once. One
+// launch, us with 128, 256 and 512 threads: segments of 1233 rows, 128 heads
+// 52, 40, 34 (fp32 70, 49, 41), 512 64, 60, 48 (88, 77, 66), 1024 81, 72, 76
+// (112, 100, 104), 2048 116, 110, 122 (187, 160, 174), 8192 319, 321, 399;
+// of 3193 rows, 128 heads 96, 62, 49 (151, 91, 64), 2048 241, 210, 264; of 160
+// rows, 256 heads 27.3, 27.0, 27.4 (30.7, 28.6, 29.6), 1024 29, 34, 44 (34,
+// 37, 49). update_threads draws the lines from these.
+constexpr int upd_ctas(int NT) { return NT == 128 ? 10 : NT == 256 ? 5 : 2; }
 
 // Phase timestamps per head of the update for latency studies; compiled out
 // by default.
@@ -104,8 +105,9 @@ struct UpdSmem {
 // Rows a warp stages at a time in the score phase: 32, or fewer when every
 // warp's share of the longest segment is smaller (short segments then leave
 // room for more CTAs per SM).
-__host__ __device__ constexpr int stage_rows(int max_len) {
-  return max_len >= NT ? 32 : (max_len + NT / 32 - 1) / (NT / 32) < 1 ? 1 : (max_len + NT / 32 - 1) / (NT / 32);
+__host__ __device__ constexpr int stage_rows(int NT, int max_len) {
+  const int share = (max_len + NT / 32 - 1) / (NT / 32);
+  return max_len >= NT ? 32 : share < 1 ? 1 : share;
 }
 
 // The score phase stages 64 bytes of each row at a time, two such pieces in
@@ -115,24 +117,23 @@ constexpr int kChunk = 64, kChunkStride = kChunk + 16, kChunkStages = 2;
 __host__ __device__ constexpr size_t stage_bytes_of(int rows) {
   return (size_t)rows * kChunkStride * kChunkStages;
 }
-__host__ __device__ constexpr size_t stage_bytes(int max_len) {
-  return stage_bytes_of(stage_rows(max_len));
-}
 
 // the query ring (P rows of es-byte elements); after q-bar the score stages,
 // and at the end the list of the rows that fill holes
-__host__ __device__ constexpr size_t ring_bytes(int P, int D, int es, int max_len) {
+__host__ __device__ constexpr size_t ring_bytes(int NT, int P, int D, int es, int max_len) {
+  const size_t stages = (size_t)(NT / 32) * stage_bytes_of(stage_rows(NT, max_len));
   size_t b = (size_t)P * D * es;
-  if (b < (size_t)(NT / 32) * stage_bytes(max_len)) b = (size_t)(NT / 32) * stage_bytes(max_len);
+  if (b < stages) b = stages;
   if (b < (size_t)max_len * 4) b = (size_t)max_len * 4;
   return (b + 15) / 16 * 16;
 }
 
+template <int NT>
 __device__ __forceinline__ UpdSmem carve(unsigned char *dyn, int max_len, int D, int P, int es) {
   UpdSmem u;
   u.ring = dyn;
-  u.stage_rows = stage_rows(max_len);
-  u.qbar = reinterpret_cast<float *>(dyn + ring_bytes(P, D, es, max_len));
+  u.stage_rows = stage_rows(NT, max_len);
+  u.qbar = reinterpret_cast<float *>(dyn + ring_bytes(NT, P, D, es, max_len));
   u.hist = reinterpret_cast<int *>(u.qbar + D);
   u.kh = reinterpret_cast<uint32_t *>(u.hist + 512);
   u.ps = reinterpret_cast<int *>(u.kh + max_len);
@@ -145,7 +146,7 @@ __device__ __forceinline__ UpdSmem carve(unsigned char *dyn, int max_len, int D,
 // select on bytes from `top_shift` down. A key is (kh[j], ps[j]), or ps[j]
 // alone. Keys are unique within a class, so each result bounds exactly k keys
 // of its class from above.
-template <bool HIGH>
+template <int NT, bool HIGH>
 __device__ void radix_select2(const uint32_t *kh, const int *ps, const int16_t *cls, int n, int k0,
                               int k1, int top_shift, int *hist, UpdShared &sh) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -219,7 +220,7 @@ __device__ __forceinline__ int block_sum(int x, UpdShared &sh) {
 // u.aux[r] is 1 for a kept row and 0 for an evicted one (r < len), u.ps
 // holds the rows' positions, and the number of evicted rows is returned.
 // Block-uniform.
-template <int D, typename T>
+template <int NT, int D, typename T>
 __device__ int select_evictions(const SegRef &sg, int label, const MethodArgs &m,
                                 const unsigned char *qring, int ntok, const UpdSmem &u,
                                 UpdShared &sh) {
@@ -269,14 +270,14 @@ __device__ int select_evictions(const SegRef &sg, int label, const MethodArgs &m
         const long long dr = i / m.row_len - ref / m.row_len, dc = i % m.row_len - ref % m.row_len;
         u.kh[r] = 0x7FFFFFFFu - (uint32_t)(dr * dr + dc * dc);
       }
-      radix_select2<true>(u.kh, u.ps, u.aux, sg.len, n_long, 0, 56, u.hist, sh);
+      radix_select2<NT, true>(u.kh, u.ps, u.aux, sg.len, n_long, 0, 56, u.hist, sh);
       const unsigned long long k_long = sh.prefix[0];
       for (int r = tid; r < sg.len; r += NT)
         if (u.aux[r] == 0) u.aux[r] = key_of(r) <= k_long ? 0 : 1;
     } else if (n_long > 0 && n_long < NH) {
       const int maxp = C + ntok;  // positions are below it: start at its top byte
       const int top = maxp < (1 << 8) ? 0 : maxp < (1 << 16) ? 8 : maxp < (1 << 24) ? 16 : 24;
-      radix_select2<false>(u.kh, u.ps, u.aux, sg.len, n_long, 0, top, u.hist, sh);
+      radix_select2<NT, false>(u.kh, u.ps, u.aux, sg.len, n_long, 0, top, u.hist, sh);
       const int p_long = (int)sh.prefix[0];
       for (int r = tid; r < sg.len; r += NT)
         if (u.aux[r] == 0) u.aux[r] = u.ps[r] <= p_long ? 0 : 1;
@@ -365,7 +366,7 @@ __device__ int select_evictions(const SegRef &sg, int label, const MethodArgs &m
       m_long += m_near - (NH - n_long);
       m_near = NH - n_long;
     }
-    radix_select2<true>(u.kh, u.ps, u.aux, sg.len, m_long, m_near, 56, u.hist, sh);
+    radix_select2<NT, true>(u.kh, u.ps, u.aux, sg.len, m_long, m_near, 56, u.hist, sh);
     const unsigned long long thr0 = sh.prefix[0], thr1 = sh.prefix[1];
     for (int r = tid; r < sg.len; r += NT) {
       const int c = u.aux[r];
@@ -391,7 +392,7 @@ __device__ int select_evictions(const SegRef &sg, int label, const MethodArgs &m
 // independent. Each thread ranks a contiguous run of rows (one block scan
 // for holes and fills together), and each copy batch issues all of its
 // loads before its stores. Returns the new length.
-template <int D, typename T>
+template <int NT, int D, typename T>
 __device__ int fill_holes(const SegRef &sg, int M, const UpdSmem &u, UpdShared &sh) {
   constexpr int RB = D * (int)sizeof(T);
   constexpr int LPR = RB / 16;
@@ -450,7 +451,7 @@ __device__ int fill_holes(const SegRef &sg, int M, const UpdSmem &u, UpdShared &
 
 // Out of place, keeping the source order: survivors are packed by a prefix
 // sum of the keep flags. Returns the new length.
-template <int D, typename T>
+template <int NT, int D, typename T>
 __device__ int copy_kept(const SegRef &sg, const UpdSmem &u, UpdShared &sh) {
   constexpr int RB = D * (int)sizeof(T);
   constexpr int LPR = RB / 16;
@@ -494,16 +495,16 @@ __device__ int copy_kept(const SegRef &sg, const UpdSmem &u, UpdShared &sh) {
 }
 
 // The update of one head in place (local: window slide; global: STE).
-template <int D, typename T>
+template <int NT, int D, typename T>
 __device__ int update_in_place(const SegRef &sg, int label, const MethodArgs &m,
                                const unsigned char *qring, int ntok, const UpdSmem &u,
                                UpdShared &sh) {
-  const int M = select_evictions<D, T>(sg, label, m, qring, ntok, u, sh);
-  return fill_holes<D, T>(sg, M, u, sh);
+  const int M = select_evictions<NT, D, T>(sg, label, m, qring, ntok, u, sh);
+  return fill_holes<NT, D, T>(sg, M, u, sh);
 }
 
-template <int D, typename T>
-__global__ void __launch_bounds__(NT, kUpdCtasPerSm)
+template <int NT, int D, typename T>
+__global__ void __launch_bounds__(NT, upd_ctas(NT))
     evict_kernel(const CacheArgs c, const MethodArgs m, int layer_base, int max_len) {
   constexpr int RB = D * (int)sizeof(T);
   extern __shared__ __align__(16) unsigned char dyn[];
@@ -532,7 +533,8 @@ __global__ void __launch_bounds__(NT, kUpdCtasPerSm)
   SegRef sg{K, V, pos, K, V, pos, len, cp, true, c.err};
   HKV_UTRACE(0);
   const int nl =
-      update_in_place<D, T>(sg, lab, m, qring, c.ntok[i], carve(dyn, max_len, D, m.P, (int)sizeof(T)), sh);
+      update_in_place<NT, D, T>(sg, lab, m, qring, c.ntok[i],
+                                carve<NT>(dyn, max_len, D, m.P, (int)sizeof(T)), sh);
   HKV_UTRACE(6);
   if (tid == 0) {
     c.len[i] = nl;
@@ -540,8 +542,8 @@ __global__ void __launch_bounds__(NT, kUpdCtasPerSm)
   }
 }
 
-template <int D, typename T>
-__global__ void __launch_bounds__(NT, kUpdCtasPerSm)
+template <int NT, int D, typename T>
+__global__ void __launch_bounds__(NT, upd_ctas(NT))
     append_evict_kernel(const CacheArgs c, const MethodArgs m, int layer_base, const void *q,
                         const void *k, const void *v, int max_len) {
   constexpr int RB = D * (int)sizeof(T);
@@ -571,7 +573,8 @@ __global__ void __launch_bounds__(NT, kUpdCtasPerSm)
       return;
     }
     SegRef sg{K, V, pos, K, V, pos, len, cp, true, c.err};
-    len = update_in_place<D, T>(sg, lab, m, qring, ntok, carve(dyn, max_len, D, m.P, (int)sizeof(T)), sh);
+    len = update_in_place<NT, D, T>(sg, lab, m, qring, ntok,
+                                    carve<NT>(dyn, max_len, D, m.P, (int)sizeof(T)), sh);
     nbuf = 0;
   }
   if (len >= cp) {
@@ -602,8 +605,8 @@ __global__ void __launch_bounds__(NT, kUpdCtasPerSm)
   }
 }
 
-template <int D, typename T>
-__global__ void __launch_bounds__(NT, kUpdCtasPerSm)
+template <int NT, int D, typename T>
+__global__ void __launch_bounds__(NT, upd_ctas(NT))
     repack_kernel(const CacheArgs dn, const CacheArgs rg, const MethodArgs m, int layer_base,
                   int max_len) {
   constexpr int RB = D * (int)sizeof(T);
@@ -642,13 +645,13 @@ __global__ void __launch_bounds__(NT, kUpdCtasPerSm)
             false,
             rg.err};
   const unsigned char *qring = static_cast<const unsigned char *>(dn.qbuf) + (size_t)i * m.P * RB;
-  const UpdSmem u = carve(dyn, max_len, D, m.P, (int)sizeof(T));
-  const int M = select_evictions<D, T>(sg, lab, m, qring, dn.ntok[i], u, sh);
+  const UpdSmem u = carve<NT>(dyn, max_len, D, m.P, (int)sizeof(T));
+  const int M = select_evictions<NT, D, T>(sg, lab, m, qring, dn.ntok[i], u, sh);
   if (slen - M > dcap) {
     if (tid == 0) set_err(rg.err, HKV_ERR_CAPACITY);
     return;
   }
-  const int nl = copy_kept<D, T>(sg, u, sh);
+  const int nl = copy_kept<NT, D, T>(sg, u, sh);
   if (tid == 0) {
     rg.len[i] = nl;
     rg.nbuf[i] = 0;
@@ -1331,16 +1334,28 @@ extern "C" int hkv_debug_set_utrace(unsigned long long *buf) {
 
 namespace {
 
+// all of an SM's L1 as shared memory, so that every head of a layer (one CTA
+// each) is resident at once
+template <int NT, int D, typename T>
+cudaError_t prepare_update_t(size_t smem) {
+  const void *kernels[] = {(const void *)append_evict_kernel<NT, D, T>,
+                           (const void *)evict_kernel<NT, D, T>,
+                           (const void *)repack_kernel<NT, D, T>};
+  cudaError_t e = cudaSuccess;
+  for (const void *f : kernels) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  }
+  return e;
+}
+
 template <int D, typename T>
 cudaError_t prepare_t(size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(append_evict_kernel<D, T>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(evict_kernel<D, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(repack_kernel<D, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+  cudaError_t e = prepare_update_t<128, D, T>(smem);
+  if (e == cudaSuccess) e = prepare_update_t<256, D, T>(smem);
+  if (e == cudaSuccess) e = prepare_update_t<512, D, T>(smem);
   const void *ident[] = {(const void *)identify_kernel<D, T, 2, false>,
                          (const void *)identify_kernel<D, T, 8, false>,
                          (const void *)identify_kernel<D, T, 8, true>,
@@ -1351,17 +1366,6 @@ cudaError_t prepare_t(size_t smem) {
   for (const void *f : ident)
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  // all of an SM's L1 as shared memory, so that every head of a layer (one
-  // CTA each) is resident at once
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(evict_kernel<D, T>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             100);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(append_evict_kernel<D, T>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(repack_kernel<D, T>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             100);
   return e;
 }
 
@@ -1409,16 +1413,22 @@ cudaError_t pdl_launch(void (*kernel)(KArgs...), int grid, int block, size_t sme
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-size_t smem_of(int max_len, int D, int P, int es) {
+size_t smem_of(int NT, int max_len, int D, int P, int es) {
   // the query ring / score stages; key words, positions (4 B each) and
   // class/flag/rank (2 B) per row; q-bar; two 256-bin histograms
-  return ring_bytes(P, D, es, max_len) + (size_t)D * 4 + 512 * 4 + (size_t)max_len * 10 + 16;
+  return ring_bytes(NT, P, D, es, max_len) + (size_t)D * 4 + 512 * 4 + (size_t)max_len * 10 + 16;
 }
 
 }  // namespace
 
-size_t update_smem_bytes(int max_len, int D, int P, int dtype) {
-  return smem_of(max_len, D, P, dtype == HKV_BF16 ? 2 : 4);
+size_t update_smem_bytes(int threads, int max_len, int D, int P, int dtype) {
+  return smem_of(threads, max_len, D, P, dtype == HKV_BF16 ? 2 : 4);
+}
+
+// (every segment that update_limit_bytes accepts fits with 512)
+int update_threads(int nheads, int max_len, int sms) {
+  if (max_len < 512) return nheads <= 2 * sms ? 256 : 128;
+  return nheads <= 4 * sms ? 512 : nheads <= 16 * sms ? 256 : 128;
 }
 
 size_t update_limit_bytes(int max_len, int D, int P, int dtype) {
@@ -1434,29 +1444,47 @@ cudaError_t update_prepare(int D, int dtype, size_t smem) {
   return cudaErrorInvalidValue;
 }
 
+// runs the statement with NT = `threads`
+#define HKV_THREADS(threads_, ...)     \
+  do {                                 \
+    if ((threads_) == 512) {           \
+      constexpr int NT = 512;          \
+      __VA_ARGS__;                     \
+    } else if ((threads_) == 256) {    \
+      constexpr int NT = 256;          \
+      __VA_ARGS__;                     \
+    } else {                           \
+      constexpr int NT = 128;          \
+      __VA_ARGS__;                     \
+    }                                  \
+  } while (0)
+
 cudaError_t launch_append_evict(const CacheArgs &c, const MethodArgs &m, int layer_base,
                                 int nheads, const void *q, const void *k, const void *v, int D,
-                                int dtype, int max_len, size_t smem, cudaStream_t s) {
+                                int dtype, int max_len, int threads, size_t smem,
+                                cudaStream_t s) {
   HKV_DISPATCH(D, dtype,
-               return pdl_launch(append_evict_kernel<kD, kT>, nheads, NT, smem, s, c, m,
-                                 layer_base, q, k, v, max_len));
+               HKV_THREADS(threads, return pdl_launch(append_evict_kernel<NT, kD, kT>, nheads, NT,
+                                                      smem, s, c, m, layer_base, q, k, v,
+                                                      max_len)));
   return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_evict(const CacheArgs &c, const MethodArgs &m, int layer_base, int nheads,
-                         int D, int dtype, int max_len, size_t smem, cudaStream_t s) {
+                         int D, int dtype, int max_len, int threads, size_t smem,
+                         cudaStream_t s) {
   HKV_DISPATCH(D, dtype,
-               return pdl_launch(evict_kernel<kD, kT>, nheads, NT, smem, s, c, m, layer_base,
-                                 max_len));
+               HKV_THREADS(threads, return pdl_launch(evict_kernel<NT, kD, kT>, nheads, NT, smem,
+                                                      s, c, m, layer_base, max_len)));
   return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_repack(const CacheArgs &dense, const CacheArgs &ragged, const MethodArgs &m,
-                          int layer_base, int nheads, int D, int dtype, int max_len, size_t smem,
-                          cudaStream_t s) {
+                          int layer_base, int nheads, int D, int dtype, int max_len, int threads,
+                          size_t smem, cudaStream_t s) {
   HKV_DISPATCH(D, dtype,
-               return pdl_launch(repack_kernel<kD, kT>, nheads, NT, smem, s, dense, ragged, m,
-                                 layer_base, max_len));
+               HKV_THREADS(threads, return pdl_launch(repack_kernel<NT, kD, kT>, nheads, NT, smem,
+                                                      s, dense, ragged, m, layer_base, max_len)));
   return cudaErrorInvalidValue;
 }
 

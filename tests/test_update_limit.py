@@ -23,13 +23,14 @@ def test_accepted_lengths_with_the_shipped_periods():
 def test_rule_of_the_header(H, D, dtype, P):  # noqa: F811
     lib = ctypes.CDLL(H.LIB_PATH)
     limit, used = (getattr(lib, n) for n in ("_ZN3hkv18update_limit_bytesEiiii",
-                                             "_ZN3hkv17update_smem_bytesEiiii"))
+                                             "_ZN3hkv17update_smem_bytesEiiiii"))
     for f in (limit, used):
         f.restype = ctypes.c_size_t
     code = 1 if dtype == "bf16" else 0
     n = _longest(D, dtype, P)
     assert limit(n, D, P, code) <= KB227 < limit(n + 1, D, P, code)
-    assert used(n, D, P, code) <= KB227  # what is accepted fits
+    for threads in (128, 256, 512):
+        assert used(threads, n, D, P, code) <= KB227  # what is accepted fits
 
 
 @pytest.mark.gpu
