@@ -593,12 +593,14 @@ hkv_status hkv_identify_heads(const hkv_config *cfg, const hkv_cache *cache, int
   const size_t upd = update_limit_bytes(max_segment(*cfg), cfg->head_dim, cfg->period, cfg->dtype);
   const size_t need = identify_smem_bytes(max_len, cfg->period,
                                           cfg->distance_mode == HKV_DIST_GRID2D, false);
-  const size_t staged = identify_stage_bytes(max_len, cfg->distance_mode == HKV_DIST_GRID2D);
+  const int hpl = heads_per_layer(cfg), sms = st->sms.load(std::memory_order_acquire);
+  const size_t staged =
+      identify_stage_bytes(hpl, max_len, cfg->distance_mode == HKV_DIST_GRID2D,
+                           cfg->head_dim * (cfg->dtype == HKV_BF16 ? 2 : 4), sms);
   HKV_TRY(update_ready(st, cfg->head_dim, cfg->dtype, staged > need ? staged : need,
                        upd > need ? upd : need));
-  const int hpl = heads_per_layer(cfg);
   return cuda_status(launch_identify(cache_args(cache), method_args(cfg), layer * hpl, hpl, q,
-                                     label_out, nh_out, cfg->head_dim, cfg->dtype, max_len,
+                                     label_out, nh_out, cfg->head_dim, cfg->dtype, max_len, sms,
                                      (cudaStream_t)stream));
 }
 

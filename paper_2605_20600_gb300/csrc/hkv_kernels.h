@@ -195,13 +195,13 @@ cudaError_t launch_init_dense(const CacheArgs &c, int nheads_total, int seg_toke
                               cudaStream_t s);
 cudaError_t launch_identify(const CacheArgs &c, const MethodArgs &m, int layer_base, int nheads,
                             const void *q, uint8_t *label_out, int32_t *nh_out, int D, int dtype,
-                            int max_len, cudaStream_t s);
+                            int max_len, int sms, cudaStream_t s);
 // shared memory of the identification kernels (single query, or multi:
 // the ring's newest min(P, ntok) queries) for dense segments of up to
 // max_len tokens; at most what update_prepare enabled
 size_t identify_smem_bytes(int max_len, int P, bool grid2d, bool multi);
 // with the key stages of the single-query kernel, 0 where it runs without
-size_t identify_stage_bytes(int max_len, bool grid2d);
+size_t identify_stage_bytes(int nheads, int max_len, bool grid2d, int row_bytes, int sms);
 // multi-query Step 2 over the ring's newest min(P, ntok) queries
 cudaError_t launch_identify_multi(const CacheArgs &c, const MethodArgs &m, int layer_base,
                                   int nheads, uint8_t *label_out, int32_t *nh_out, int D,

@@ -756,7 +756,8 @@ __host__ __device__ constexpr size_t id_smem(size_t floats, int max_len, bool gr
   return grid2d ? id_order_offset(floats) + (size_t)max_len * 12 : floats * 4;
 }
 __host__ __device__ constexpr size_t id_stage_at(size_t smem) { return (smem + 127) / 128 * 128; }
-constexpr size_t kIdMostSmem = 226 * 1024;  // dynamic, beside the kernels' static part
+// dynamic, beside the kernels' static part: of one CTA of an SM, of two
+constexpr size_t kIdMostSmem = 226 * 1024, kIdTwoSmem = 112 * 1024;
 
 // The count order of the grid-distance variant of Step 2: perm[j] = the row
 // of the j-th token counted. Image tokens by squared grid distance from image
@@ -1509,11 +1510,12 @@ cudaError_t launch_init_dense(const CacheArgs &c, int n, int seg, cudaStream_t s
 
 cudaError_t launch_identify(const CacheArgs &c, const MethodArgs &m, int layer_base, int nheads,
                             const void *q, uint8_t *label_out, int32_t *nh_out, int D, int dtype,
-                            int max_len, cudaStream_t s) {
+                            int max_len, int sms, cudaStream_t s) {
   const float qscale = (float)(1.4426950408889634 / sqrt((double)D));
   const size_t smem = identify_smem_bytes(max_len, m.P, m.grid2d != 0, false);
   // the stages lie behind the rest, where both fit (identify_stage_bytes)
-  const size_t staged = identify_stage_bytes(max_len, m.grid2d != 0);
+  const size_t staged = identify_stage_bytes(nheads, max_len, m.grid2d != 0,
+                                             D * (dtype == HKV_BF16 ? 2 : 4), sms);
   if (staged > 0) {
     HKV_DISPATCH(D, dtype,
                  return pdl_launch(identify_kernel<kD, kT, 8, true>, nheads, IT, staged, s, c, m,
@@ -1549,11 +1551,21 @@ cudaError_t launch_identify_multi(const CacheArgs &c, const MethodArgs &m, int l
   return cudaErrorInvalidValue;
 }
 
-size_t identify_stage_bytes(int max_len, bool grid2d) {
+// The stages pay while the heads have an SM, or half of one, each (their keys
+// are on the way before the first product, but they leave room for two CTAs an
+// SM at most), and where a head's keys take 256 KB and more. us without and
+// with, bf16 rows of 256 bytes: 628 tokens, 32 heads 7.8, 6.6, 256 13.3, 11.3,
+// 512 18.2, 20.0, 1216 37.7, 40.8, 2560 73.7, 72.8; 1128 tokens, 512 28.1, 29.4,
+// 704 47.0, 42.0, 2560 122, 113; of 128 bytes, 601 tokens, 512 12.9, 14.9, 4096
+// 67, 75, 2001 tokens 173, 168; fp32 rows of 512, 628 tokens, 1024 58.3, 55.4.
+// The count on the grid ranks every row and wants the other CTAs' warps: 2000
+// tokens, 128 heads 175, 157, 256 (one CTA an SM with the stages) 265, 305.
+size_t identify_stage_bytes(int nheads, int max_len, bool grid2d, int row_bytes, int sms) {
   if (max_len < kIdLongSegment) return 0;
+  if (nheads > 2 * sms && (grid2d || (size_t)max_len * row_bytes < 256 * 1024)) return 0;
   const size_t b = id_stage_at(identify_smem_bytes(max_len, 1, grid2d, false)) +
                    (size_t)kIdStages * kIdStageBytes;
-  return b <= kIdMostSmem ? b : 0;
+  return b <= (grid2d && nheads > sms ? kIdTwoSmem : kIdMostSmem) ? b : 0;
 }
 
 size_t identify_smem_bytes(int max_len, int P, bool grid2d, bool multi) {
